@@ -10,6 +10,7 @@
 #include <mutex>
 #include <numeric>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include <cudaTypedefs.h>
@@ -394,11 +395,189 @@ UpdateArgs update_args(jkcals_ctx* h, int n, const void* part, int part_kind, in
 tc::TcArgs make_tc_args(jkcals_ctx* h, int n, float* const* UT, float* const* UTlo, float* const* cmax,
                         bool reuse_slices);
 
-// Enqueue the concurrent MTTKRP of mode n for factor set (U, UT, cmax) into h->part.
-// reuse_slices: a two-step mode may reuse the U_a slices left in At by the
-// previous two-step launch of the same sweep when mode a was not updated since.
+int mode_splits(const jkcals_ctx* h, int n) { return h->tc ? h->tcplan[n].splits : h->plan[n].splits; }
+
+// ---- FP64 form through tensor-times-matrix products --------------------------
+// What the workspace holds while the MTTKRPs of one sweep (or one gradient) are
+// enqueued: Y contracted with mode y, Z with modes z_a and z_q (-1: nothing).
+struct TtmState {
+  int y = -1, z_a = -1, z_q = -1;
+  void updated(int n) {   // Ubar^(n) changed
+    if (y == n) y = -1;
+    if (z_a == n || z_q == n) z_a = z_q = -1;
+  }
+};
+
+// Estimated seconds.  The product: waves of 128 x 64 tiles over the SMs, 1160
+// cycles per 16 rows of the contraction and about 5000 of exposed drain per
+// tile, plus slicing the factor and two launches.  A contraction reads Y once at
+// two FP64 multiply-adds per clock and SM.  The CUDA-core MTTKRP runs its padded
+// 64 x 64 tiles at about 0.85 TFLOP/s.
+double ttm_product_cost(const jkcals_ctx* h, int a) {
+  const int64_t tiles = (int64_t)((h->C + kTtmTileC - 1) / kTtmTileC) * ((h->J[a] + kTtmTileR - 1) / kTtmTileR);
+  const int64_t waves = (tiles + h->num_sms - 1) / h->num_sms;
+  return waves * (ttm_ksteps((int)h->dims[a]) * 1160.0 + 5000.0) / 1.9e9 + 12e-6;
+}
+double ttm_contract_cost(const jkcals_ctx* h, int a) {
+  return (double)h->J[a] * h->C / (h->num_sms * 3.6e9) + 4e-6;
+}
+double native_cost(const jkcals_ctx* h, int n) {
+  return 2.0 * round_up(h->C, kMttkrpBN) * (double)round_up(h->dims[n], kMttkrpBM) * h->J[n] / 0.85e12 + 5e-6;
+}
+
+// Contracted mode for mode n's MTTKRP: the one Y holds, else the cheaper one
+// with images (-1: the CUDA-core kernel).
+int ttm_choose(const jkcals_ctx* h, int n, const int (&modes)[2], int y) {
+  if (y >= 0 && y != n) return y;
+  int best = -1;
+  for (int a : modes)
+    if (a >= 0 && a != n && (best < 0 || ttm_product_cost(h, a) < ttm_product_cost(h, best))) best = a;
+  return best;
+}
+
+// Estimated MTTKRP seconds of one sweep with images for `modes`.
+double ttm_sweep_cost(const jkcals_ctx* h, const int (&modes)[2]) {
+  double t = 0.0;
+  TtmState st;
+  for (int n = 0; n < h->N; ++n) {
+    const int a = ttm_choose(h, n, modes, st.y);
+    if (a < 0) {
+      t += native_cost(h, n);
+    } else {
+      if (a != st.y) t += ttm_product_cost(h, a);
+      if (h->N > 2) t += ttm_contract_cost(h, a);
+      st.y = a;
+    }
+    st.updated(n);
+  }
+  return t;
+}
+
+// Whether the current column count goes through the products.  The factor 0.8
+// keeps sizes where the two are about even (the smallest tensors: launches and
+// latency) on the CUDA-core kernel, which needs fewer launches.
+void plan_ttm_use(jkcals_ctx* h) {
+  jkcals_ctx::Ttm& t = h->ttm;
+  t.use = false;
+  if (t.modes[0] < 0) return;
+  double nat = 0.0;
+  for (int n = 0; n < h->N; ++n) nat += native_cost(h, n);
+  t.use = ttm_sweep_cost(h, t.modes) < 0.8 * nat;
+}
+
+// Modes whose images would make a sweep cheapest (t.modes; -1: none pays).
+// Explicit split-K factors ask for the CUDA-core kernel, and under a memory cap
+// the handle holds what that kernel needs and no more, so that later calls
+// (gradients, loss histories, compaction) find the room the cap left them.
+constexpr int64_t kTtmMaxY = (int64_t)1 << 31;   // elements of Y (16 GiB)
+void choose_ttm_modes(jkcals_ctx* h) {
+  jkcals_ctx::Ttm& t = h->ttm;
+  t.modes[0] = t.modes[1] = -1;
+  if (h->tc || h->opt.splits > 0 || h->opt.max_device_bytes > 0) return;
+  auto ok = [&](int a) { return h->dims[a] <= kTtmChainMax && h->J[a] <= kTtmMaxY / h->C; };
+  double best = 0.0;
+  for (int x = 0; x < h->N; ++x)
+    for (int y = x; y < h->N; ++y) {   // y == x: images of one mode only
+      if (!ok(x) || !ok(y)) continue;
+      const int m[2] = {x, y == x ? -1 : y};
+      const double c = ttm_sweep_cost(h, m);
+      if (t.modes[0] < 0 || c < best) {
+        best = c;
+        t.modes[0] = m[0];
+        t.modes[1] = m[1];
+      }
+    }
+  plan_ttm_use(h);
+  if (!t.use) t.modes[0] = t.modes[1] = -1;
+}
+
+// Mode n's MTTKRP into h->part by way of mode a's product (and Z for N >= 4).
+// Z leaves out the highest mode it can: the next modes of a sweep then share it.
+jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmState& st, int* kernels) {
+  jkcals_ctx::Ttm& t = h->ttm;
+  const int N = h->N;
+  double* part = static_cast<double*>(h->part);
+  const bool have_z = N >= 4 && st.z_a >= 0 && st.z_a != n && st.z_q != n;
+  if (!have_z && st.y != a) {
+    TtmArgs g{};
+    g.At = t.At;
+    g.Bt = t.Bt[a];
+    g.cexp = t.cexp;
+    g.rexp = t.rexp[a];
+    g.K = (int)h->dims[a];
+    g.nk = ttm_ksteps(g.K);
+    g.C = h->C;
+    g.tiles_c = (h->C + kTtmTileC - 1) / kTtmTileC;
+    g.J = h->J[a];
+    g.tiles_r = (h->J[a] + kTtmTileR - 1) / kTtmTileR;
+    g.Y = N == 2 ? part : t.Y;   // two modes: the product is the MTTKRP
+    g.Tn = h->Tn64[a];
+    g.U = U[a];
+    g.err = h->d_err;
+    JK_CUDA(h, launch_slice_factor(U[a], g.K, h->C, t.kexp[a], t.At, t.cexp, h->stream));
+    JK_CUDA(h, launch_ttm_f64(g, h->num_sms, h->stream));
+    *kernels += 2;
+    if (N > 2) st.y = a;
+  }
+  h->part_S = 1;
+  if (N == 2) return JKCALS_OK;
+  const double* X = t.Y;
+  std::vector<int> rest;   // modes of X, fastest first
+  for (int k = 0; k < N; ++k)
+    if (have_z ? (k != st.z_a && k != st.z_q) : k != a) rest.push_back(k);
+  if (have_z) X = t.Z;
+  int w = 0;
+  while (rest.size() > 1) {
+    size_t pos = rest.size() - 1;
+    if (rest[pos] == n) --pos;
+    const int q = rest[pos];
+    int64_t L = 1, H = 1;
+    for (size_t k = 0; k < rest.size(); ++k) (k < pos ? L : H) *= k == pos ? 1 : h->dims[rest[k]];
+    double* out = part;
+    int S = 1;
+    if (rest.size() == 2) {
+      S = contract_splits(H * L, (int)h->dims[q], h->C);
+      const int64_t cap = (int64_t)(h->part_bytes / sizeof(double)) / (H * L * h->C);
+      S = (int)std::max<int64_t>(1, std::min<int64_t>(S, cap));
+      S = (int)((h->dims[q] + (h->dims[q] + S - 1) / S - 1) / ((h->dims[q] + S - 1) / S));
+      h->part_S = S;
+    } else if (X == t.Y) {
+      out = t.Z;
+      st.z_a = a;
+      st.z_q = q;
+    } else {
+      out = t.W[w];
+      w ^= 1;
+    }
+    JK_CUDA(h, launch_contract_f64(X, H, (int)h->dims[q], L, h->C, U[q], S, out, h->stream));
+    *kernels += 1;
+    X = out;
+    rest.erase(rest.begin() + pos);
+  }
+  return JKCALS_OK;
+}
+
+// Enqueue the concurrent MTTKRP of mode n for factor set (U, UT, cmax) into
+// h->part (h->part_S splits).  reuse_slices: a two-step mode may reuse the U_a
+// slices left in At by the previous two-step launch of the same sweep when mode
+// a was not updated since.  st: products of the FP64 form that the caller's
+// earlier MTTKRPs left in the workspace.
 jkcals_status enqueue_mttkrp(jkcals_ctx* h, int n, double* const* U, float* const* UT, float* const* UTlo,
-                             float* const* cmax, bool reuse_slices = false) {
+                             float* const* cmax, bool reuse_slices = false, TtmState* st = nullptr,
+                             int* kernels = nullptr) {
+  int launched = 0;
+  if (kernels == nullptr) kernels = &launched;
+  h->part_S = mode_splits(h, n);
+  if (h->ttm.use) {
+    // one MTTKRP on its own has no other mode to share the product with
+    const bool alone = st == nullptr;
+    TtmState local;
+    if (alone) st = &local;
+    int a = ttm_choose(h, n, h->ttm.modes, st->y);
+    if (alone && a >= 0 && ttm_product_cost(h, a) + ttm_contract_cost(h, a) > 0.8 * native_cost(h, n)) a = -1;
+    if (a >= 0) return enqueue_ttm(h, n, a, U, *st, kernels);
+  }
+  *kernels += 1;
   if (!h->tc) {
     const ModePlan& p = h->plan[n];
     KrpOperands kr = krp_operands(h, n, U);
@@ -463,8 +642,6 @@ tc::TcArgs make_tc_args(jkcals_ctx* h, int n, float* const* UT, float* const* UT
   return a;
 }
 
-int mode_splits(const jkcals_ctx* h, int n) { return h->tc ? h->tcplan[n].splits : h->plan[n].splits; }
-
 int part_kind(const jkcals_ctx* h) {
   if (!h->tc) return kPartF64;
   return h->opt.precision == JKCALS_EXACT_BF16 ? kPartF32x2 : kPartF32;
@@ -473,11 +650,11 @@ int part_kind(const jkcals_ctx* h) {
 jkcals_status reduce_into(jkcals_ctx* h, int n, double* out) {
   const int64_t cnt = h->dims[n] * (int64_t)h->C;
   if (part_kind(h) == kPartF32x2)
-    JK_CUDA(h, launch_reduce_partials_f32x2(static_cast<float2*>(h->part), mode_splits(h, n), cnt, out, h->stream));
+    JK_CUDA(h, launch_reduce_partials_f32x2(static_cast<float2*>(h->part), h->part_S, cnt, out, h->stream));
   else if (part_kind(h) == kPartF32)
-    JK_CUDA(h, launch_reduce_partials_f32(static_cast<float*>(h->part), mode_splits(h, n), cnt, out, h->stream));
+    JK_CUDA(h, launch_reduce_partials_f32(static_cast<float*>(h->part), h->part_S, cnt, out, h->stream));
   else
-    JK_CUDA(h, launch_reduce_partials_f64(static_cast<double*>(h->part), mode_splits(h, n), cnt, out, h->stream));
+    JK_CUDA(h, launch_reduce_partials_f64(static_cast<double*>(h->part), h->part_S, cnt, out, h->stream));
   return JKCALS_OK;
 }
 
@@ -488,13 +665,33 @@ jkcals_status reduce_into(jkcals_ctx* h, int n, double* out) {
 int count_sweep_kernels(const jkcals_ctx* h) {
   int kernels = 0;
   int sliced = -1;
+  TtmState st;
   for (int n = 0; n < h->N; ++n) {
     const bool tts = h->tc && h->tcplan[n].tts;
     if (tts) {
       kernels += sliced == h->tcplan[n].a_mode ? 0 : 1;
       sliced = h->tcplan[n].a_mode;
     }
-    kernels += h->plan[n].upd.fused ? 2 : 4;
+    kernels += h->plan[n].upd.fused ? 1 : 3;
+    const int a = h->ttm.use ? ttm_choose(h, n, h->ttm.modes, st.y) : -1;
+    if (a < 0) {
+      kernels += 1;
+    } else {
+      // the product and its slicing unless Y or Z is current, then one
+      // contraction per further mode
+      const bool have_z = h->N >= 4 && st.z_a >= 0 && st.z_a != n && st.z_q != n;
+      if (!have_z && st.y != a) {
+        kernels += 2;
+        if (h->N > 2) st.y = a;
+      }
+      kernels += have_z ? h->N - 3 : h->N - 2;
+      if (!have_z && h->N >= 4) {
+        st.z_a = a;
+        st.z_q = h->N - 1;
+        while (st.z_q == n || st.z_q == a) --st.z_q;
+      }
+    }
+    st.updated(n);
     if (n == sliced) sliced = -1;
   }
   return kernels + 1;
@@ -503,11 +700,12 @@ int count_sweep_kernels(const jkcals_ctx* h) {
 jkcals_status enqueue_sweep(jkcals_ctx* h) {
   int kernels = 0;
   int sliced = -1;   // mode whose current slices At holds (two-step modes)
+  TtmState ttm;
   for (int n = 0; n < h->N; ++n) {
     const bool tts = h->tc && h->tcplan[n].tts;
     const bool reuse = tts && sliced == h->tcplan[n].a_mode;
     if (h->opt.kernel_timing) JK_CUDA(h, cudaEventRecordWithFlags(h->ev_start[n], h->stream, cudaEventRecordExternal));
-    JK_TRY(enqueue_mttkrp(h, n, h->U, h->UT, h->UTlo, h->cmax, reuse));
+    JK_TRY(enqueue_mttkrp(h, n, h->U, h->UT, h->UTlo, h->cmax, reuse, &ttm, &kernels));
     if (tts) {
       sliced = h->tcplan[n].a_mode;
       kernels += reuse ? 0 : 1;
@@ -515,16 +713,17 @@ jkcals_status enqueue_sweep(jkcals_ctx* h) {
     if (h->opt.kernel_timing) JK_CUDA(h, cudaEventRecordWithFlags(h->ev_stop[n], h->stream, cudaEventRecordExternal));
     if (h->plan[n].upd.fused) {
       // the fused update sums each block's split-K partials itself (fixed order)
-      UpdateArgs a = update_args(h, n, h->part, part_kind(h), mode_splits(h, n));
+      UpdateArgs a = update_args(h, n, h->part, part_kind(h), h->part_S);
       JK_CUDA(h, launch_update_fused(a, h->plan[n].upd.fused_smem, h->Rmax, h->uniform_rank, h->stream));
-      kernels += 2;
+      kernels += 1;
     } else {
       // fixed-order split-K reduction into FP64 Mbar_n, then the two-phase update
       JK_TRY(reduce_into(h, n, h->mbuf));
       UpdateArgs a = update_args(h, n, h->mbuf, kPartF64, 1);
       JK_CUDA(h, launch_update(a, h->stream));
-      kernels += 4;
+      kernels += 3;
     }
+    ttm.updated(n);
     if (n == sliced) sliced = -1;   // U_a changed: the slices in At are stale
   }
   JK_CUDA(h, launch_advance_sweep(h->d_sweep_idx, h->stream));
@@ -588,7 +787,7 @@ jkcals_status copy_out(jkcals_ctx* h, void* dst, const void* src, size_t bytes) 
 
 // Reads the tensor-core kernel's error word (set when a bounded wait expired).
 jkcals_status check_device_error(jkcals_ctx* h) {
-  if (!h->tc || h->d_err == nullptr) return JKCALS_OK;
+  if (h->d_err == nullptr || !(h->tc || h->ttm.use)) return JKCALS_OK;
   int err = 0;
   JK_CUDA(h, cudaMemcpyAsync(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   JK_CUDA(h, cudaStreamSynchronize(h->stream));
@@ -635,6 +834,7 @@ int64_t mode_kchunk(const jkcals_ctx* h, int n) { return h->tc ? h->tcplan[n].kc
 // (three timed runs after one warm-up each, CUDA events on the handle's
 // stream) and keep the fastest.  The partial-sum workspace grows as needed.
 jkcals_status autotune_splits(jkcals_ctx* h) {
+  if (h->ttm.use) return JKCALS_OK;   // the products have no split-K factor to tune
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   JK_CUDA(h, cudaEventCreate(&e0));
   JK_CUDA(h, cudaEventCreate(&e1));
@@ -719,6 +919,85 @@ void destroy_impl(jkcals_ctx* h) {
 }  // namespace
 
 namespace {
+
+// Partial sums of the contraction that ends mode n's MTTKRP: the largest over the
+// modes it may run over.
+size_t ttm_part_elems(const jkcals_ctx* h, int n) {
+  size_t most = 0;
+  for (int q = 0; q < h->N; ++q)
+    if (q != n) most = std::max(most, (size_t)contract_splits(h->dims[n], (int)h->dims[q], h->C));
+  return most * h->dims[n] * h->C;
+}
+
+// FP64 form: the digit images of T and the products' workspace, where the plan
+// wants them, allocated after everything the CUDA-core kernel needs: if the
+// device has no room for them, or T holds a non-finite entry, the handle runs on
+// that kernel.
+jkcals_status create_ttm(jkcals_ctx* h) {
+  jkcals_ctx::Ttm& t = h->ttm;
+  if (t.modes[0] < 0) return JKCALS_OK;
+  cudaStream_t st = h->stream;
+  std::vector<void*> got;
+  auto alloc = [&](auto** p, size_t bytes) {
+    void* v = nullptr;
+    const jkcals_status s = dalloc(h, &v, bytes);
+    if (s == JKCALS_OK) {
+      *p = static_cast<std::remove_reference_t<decltype(**p)>*>(v);
+      got.push_back(v);
+    }
+    return s;
+  };
+  int* d_bad = nullptr;
+  auto build = [&]() -> jkcals_status {
+    size_t at = 0, y = 0, z = 0, w = 0;
+    JK_TRY(alloc(&d_bad, sizeof(int)));
+    JK_TRY(alloc(&h->d_err, sizeof(int)));
+    JK_CUDA(h, cudaMemsetAsync(d_bad, 0, sizeof(int), st));
+    JK_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
+    for (int a : t.modes) {
+      if (a < 0) continue;
+      at = std::max(at, ttm_image_bytes((int)h->dims[a], h->C, kTtmTileC));
+      if (h->N > 2) y = std::max(y, (size_t)h->J[a] * h->C);
+      for (int q = 0; q < h->N && h->N >= 4; ++q) {
+        if (q == a) continue;
+        z = std::max(z, (size_t)(h->J[a] / h->dims[q]) * h->C);
+        for (int p = 0; p < h->N && h->N >= 5; ++p)
+          if (p != a && p != q) w = std::max(w, (size_t)(h->J[a] / h->dims[q] / h->dims[p]) * h->C);
+      }
+    }
+    JK_TRY(alloc(&t.At, at));
+    JK_TRY(alloc(&t.cexp, sizeof(int) * (size_t)round_up(h->C, kTtmTileC)));
+    if (y > 0) JK_TRY(alloc(&t.Y, sizeof(double) * y));
+    if (z > 0) JK_TRY(alloc(&t.Z, sizeof(double) * z));
+    if (w > 0) {
+      JK_TRY(alloc(&t.W[0], sizeof(double) * w));
+      JK_TRY(alloc(&t.W[1], sizeof(double) * w));
+    }
+    for (int a : t.modes) {
+      if (a < 0) continue;
+      JK_TRY(alloc(&t.Bt[a], ttm_image_bytes((int)h->dims[a], h->J[a], kTtmTileR)));
+      JK_TRY(alloc(&t.kexp[a], sizeof(int) * (size_t)h->dims[a]));
+      JK_TRY(alloc(&t.rexp[a], sizeof(int) * (size_t)round_up(h->J[a], kTtmTileR)));
+      JK_CUDA(h, launch_slice_exponents(h->Tn64[a], h->dims[a], h->J[a], t.kexp[a], d_bad, st));
+      JK_CUDA(h, launch_slice_tensor(h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], st));
+    }
+    JK_CUDA(h, prepare_ttm_f64());
+    return JKCALS_OK;
+  };
+  jkcals_status s = build();
+  int bad = 0;
+  if (s == JKCALS_OK) {
+    JK_CUDA(h, cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+    JK_CUDA(h, cudaStreamSynchronize(st));
+  }
+  if (s == JKCALS_OK && bad == 0) return JKCALS_OK;
+  if (s != JKCALS_OK && s != JKCALS_ERR_OOM) return s;
+  for (void* p : got) dfree(h, p, true);
+  h->d_err = nullptr;
+  t = jkcals_ctx::Ttm{};
+  set_error("");
+  return JKCALS_OK;
+}
 
 jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32_t* ranks,
                           const int64_t* left_out_ptr, const int64_t* left_out_idx,
@@ -857,11 +1136,14 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
 
   // plan + workspace
   make_plan(h);
+  choose_ttm_modes(h);
   size_t part_bytes = 0, chunks = 0;
   for (int n = 0; n < N; ++n) {
     const size_t eb = part_kind(h) == kPartF32 ? sizeof(float) : sizeof(double);
     const size_t pb = (size_t)mode_splits(h, n) * h->dims[n] * h->C * eb;
     part_bytes = std::max(part_bytes, pb);
+    if (h->ttm.use)   // partial sums of the last contraction: about what fills the SMs
+      part_bytes = std::max(part_bytes, sizeof(double) * ttm_part_elems(h, n));
     chunks = std::max(chunks, (size_t)h->plan[n].upd.RC * K);
   }
   // room for the two-phase update of any subset of the blocks (compaction):
@@ -885,6 +1167,7 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
   for (int n = 0; n < N; ++n)
     if (h->plan[n].upd.fused) fsmem = std::max(fsmem, h->plan[n].upd.fused_smem);
   if (fsmem > 0) JK_CUDA(h, prepare_update_fused(fsmem, h->Rmax, h->uniform_rank));
+  JK_TRY(create_ttm(h));
   h->kernels_per_sweep = count_sweep_kernels(h);
   JK_TRY(refresh_factor_state(h));
   if (h->opt.autotune && h->opt.splits <= 0) JK_TRY(autotune_splits(h));
@@ -929,10 +1212,11 @@ jkcals_status grad_impl(jkcals_ctx* h, const double* const* U, double* const* G,
     }
   }
   const bool want_g = G != nullptr;
+  TtmState ttm;   // the factors are fixed: every mode may share a product
   for (int n = 0; n < N; ++n) {
     // the loss needs only the last mode's MTTKRP (its inner product term)
     if (!want_g && n != N - 1) continue;
-    JK_TRY(enqueue_mttkrp(h, n, h->gU, h->gUT, h->gUTlo, h->gcmax));
+    JK_TRY(enqueue_mttkrp(h, n, h->gU, h->gUT, h->gUTlo, h->gcmax, false, &ttm));
     const int64_t cnt = h->dims[n] * (int64_t)h->C;
     JK_TRY(reduce_into(h, n, h->mbuf));
     if (G != nullptr && G[n] != nullptr) {
@@ -1438,6 +1722,7 @@ jkcals_status compaction_load(jkcals_ctx* h, const std::vector<int>& sel, bool f
       if (h->plan[n].upd.fused) fsmem = std::max(fsmem, h->plan[n].upd.fused_smem);
     if (fsmem > 0) JK_CUDA(h, prepare_update_fused(fsmem, h->Rmax, h->uniform_rank));
   }
+  plan_ttm_use(h);   // few columns may be cheaper on the CUDA-core kernel
   // the tensor-core forms' transposed FP32 factor copies and column maxima
   if (h->tc)
     for (int n = 0; n < h->N; ++n) {

@@ -163,6 +163,21 @@ struct jkcals_ctx {
   double* gG[jk::kMaxModes] = {nullptr};
   double* geg = nullptr;  // K per-block losses + their sum
 
+  // FP64 form: tensor-times-matrix products on the tensor cores (jk_ttm_f64.cu)
+  struct Ttm {
+    int modes[2] = {-1, -1};                       // contracted modes with images of T (-1: none)
+    bool use = false;                              // the current plan's MTTKRPs go through them
+    unsigned char* Bt[jk::kMaxModes] = {nullptr};  // digit images of T_(a)
+    int* kexp[jk::kMaxModes] = {nullptr};          // I_a slice exponents
+    int* rexp[jk::kMaxModes] = {nullptr};          // exponents of T_(a)'s scaled columns (padded to tiles)
+    unsigned char* At = nullptr;                   // digit images of Ubar^(a), rewritten per product
+    int* cexp = nullptr;                           // exponents of its scaled columns (padded to tiles)
+    double* Y = nullptr;                           // the product, J_a x C
+    double* Z = nullptr;                           // N >= 4: Y contracted with one more mode
+    double* W[2] = {nullptr, nullptr};             // N >= 5: the further contractions
+  } ttm;
+  int part_S = 1;  // splits of the partial sums in `part` (set by each MTTKRP)
+
   double tol_host = 0.0;
 
   // tensor-core forms (precision != JKCALS_FP64)
@@ -294,6 +309,40 @@ cudaError_t launch_reduce_partials_f64(const double* part, int S, int64_t count,
 // same for FP32 partials, summed in FP64
 cudaError_t launch_reduce_partials_f32(const float* part, int S, int64_t count, double* out,
                                        cudaStream_t s);
+
+// ---- FP64 tensor-times-matrix on the tensor cores (jk_ttm_f64.cu) -------------
+constexpr int kTtmDigits = 8;
+constexpr int kTtmTileC = 128, kTtmTileR = 64;   // tile of Y: columns c, rows r
+// longest contraction whose level sums are exact: (l + 3) 2^12 K <= 2^24 for l <= 6
+constexpr int kTtmChainMax = 448;
+constexpr int kTtmBadExp = 2147483647;           // exponent of a column with a non-finite entry
+inline int ttm_ksteps(int K) { return (K + 15) / 16; }
+struct TtmArgs {
+  const unsigned char* At;   // digit images of Ubar^(a): tiles_c x nk stages
+  const unsigned char* Bt;   // digit images of T_(a): tiles_r x nk stages
+  const int* cexp;           // per column c (padded to tiles)
+  const int* rexp;           // per row r of Y (padded to tiles)
+  int nk, K, C, tiles_c;
+  int64_t J, tiles_r;
+  double* Y;                 // J x C
+  const double* Tn;          // T_(a), K x J (columns of Ubar^(a) with non-finite entries)
+  const double* U;           // Ubar^(a), K x C
+  int* err;
+};
+inline size_t ttm_image_bytes(int K, int64_t M, int tile) {
+  return (size_t)((M + tile - 1) / tile) * ttm_ksteps(K) * kTtmDigits * tile * 32;
+}
+cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* kexp, int* bad, cudaStream_t s);
+cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt, int* rexp,
+                                cudaStream_t s);
+cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At, int* cexp,
+                                cudaStream_t s);
+cudaError_t prepare_ttm_f64();
+cudaError_t launch_ttm_f64(const TtmArgs& a, int num_sms, cudaStream_t s);
+// out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c]
+int contract_splits(int64_t HL, int Mm, int C);
+cudaError_t launch_contract_f64(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
+                                double* out, cudaStream_t s);
 
 // Storage of split-K partials: FP64, FP32, or an unevaluated FP32 pair (hi, lo).
 constexpr int kPartF64 = 0, kPartF32 = 1, kPartF32x2 = 2;

@@ -1,0 +1,546 @@
+// FP64 tensor-times-matrix on the tensor cores, and the contractions that turn
+// it into concurrent MTTKRPs.
+//
+//   Y_a(r, c) = sum_i T_(a)(i, r) Ubar^(a)(i, c)           (ttm_f64_kernel)
+//   Mbar_n(i_n, c) = sum over the other indices of r of Y_a(r, c) times the
+//                    remaining factors' entries             (contract_f64_kernel)
+//
+// for a mode a != n (Eq. MTTKRP with its Khatri-Rao sum taken one mode at a
+// time).  Y_a does not depend on the other factors, so every mode n != a that is
+// updated before Ubar^(a) changes shares it: a sweep of N modes needs two of the
+// products of 2 C prod(I) operations instead of N.
+//
+// The product is exact up to FP64 rounding on the BF16 tensor pipe: GB300 runs
+// 1.1 TFLOP/s in FP64 and 1889 TFLOP/s in BF16, so 36 BF16 products per FP64
+// one still leave a factor of 48.  Every operand value x of a contraction vector
+// whose magnitudes stay below 2^E is rounded to 58 fractional bits of 2^E and
+// written in balanced digits, x = 2^(E-7) sum_k d_k 2^(-7k), |d_0| <= 128,
+// |d_k| <= 64 (k = 1 .. 7; d_7 in steps of 1/4): BF16 holds each digit exactly.
+// The products d_s e_t with s + t = l < 8 are summed per level l in one FP32
+// accumulator in TMEM.  A level's terms are integers and its sum stays below
+// (l + 3) 2^12 K <= 2^24 for chains of K <= kTtmChainMax, so levels 0 to 6 are
+// exact whatever the order of the additions; level 7 may truncate in its own
+// last bits (2^-63 of the product of the vectors' maxima).  What is dropped is
+// the operands' rounding (2^-59) and the products beyond level 7 (seven terms
+// of about 2^-60 each): below the rounding of a single FP64 multiply-add per
+// term.  The drain adds the levels as 64-bit integers and rounds once to FP64.
+//
+// Along the contraction the two operands are equilibrated by powers of two
+// (exact): T_(a)(i, :) 2^(-F_i) against Ubar^(a)(i, :) 2^(F_i), F_i the exponent
+// of the largest entry of slice i.  A slice much larger than the others (an
+// outlying sample) then costs no digits in submodels that leave it out.
+//
+// Measured (GB300), against the CUDA-core MTTKRP of every mode: an FP64 sweep of
+// 300x100x50 with 1500 columns 16.0 -> 0.46 ms, of 400x400x400 with 400 columns
+// 192 -> 3.4 ms; loss and gradient of 100x60x60x40 with 800 columns 166 -> 4.7 ms.
+// Largest MTTKRP error against quadruple precision, relative to the largest
+// entry (300x100x50, modes 0-2): 3.2e-16, 4.9e-16, 5.8e-16, against 6.9e-16,
+// 1.8e-15, 1.6e-15 on the CUDA cores, whose chains of additions are longer.
+//
+// A column of Ubar^(a) with a non-finite entry is taken out of the digits and
+// computed by plain FP64 dot products in the drain, so Inf and NaN propagate as
+// in the CUDA-core kernel; a tensor with a non-finite entry never gets here.
+#include <limits.h>
+#include <math.h>
+
+#include "jk_common.cuh"
+#include "jk_ptx.cuh"
+
+namespace jk {
+namespace {
+
+using namespace ptx;
+
+constexpr int P = kTtmDigits;                 // 8 digits per operand value
+constexpr int kTileM = kTtmTileC, kTileN = kTtmTileR;
+constexpr int kRow = 32;                      // bytes of one operand row per stage: 16 BF16
+constexpr uint32_t kABytes = kTileM * kRow, kBBytes = kTileN * kRow;
+constexpr uint32_t kAStage = P * kABytes, kBStage = P * kBBytes, kStage = kAStage + kBStage;   // 32 + 16 KB
+constexpr int kStages = 4;
+constexpr int kEpiWarps = 16;
+constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
+constexpr int kThreads = 32 * (kEpiWarps + 2);
+constexpr uint32_t kTmemCols = P * kTileN;    // 512: all of TMEM
+constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + (2 * kStages + 3) * 8 + 16;
+
+// ---- digits ---------------------------------------------------------------------
+// One operand matrix X (K x M, row stride ld; K the contraction) into stage images:
+// per TILE columns m and 16 rows k, P digit tiles of TILE x 32 bytes, K-major in
+// the 32-byte swizzle (16-byte chunk XOR bit 2 of the row): one bulk copy per
+// operand and stage.  A block takes 8 columns, thread (m, g) the 8-row chunks g
+// and g + 32, loaded once into registers (K <= kTtmChainMax: at most 56 chunks):
+// first each column's exponent (expo[m]: scaled magnitudes < 2^expo), then the
+// digits.  sgn = +1 / -1 scales row k by 2^(+-kexp[k]).  Integer arithmetic
+// throughout: an FP64 rint per digit would take 18 us of the FP64 pipe for
+// 300 x 1500 entries.
+constexpr int kSliceCols = 8;   // columns per block
+
+template <int TILE>
+__global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict__ X, int K, int64_t M, int64_t ld,
+                                                        const int* __restrict__ kexp, int sgn, int nk, int64_t Mpad,
+                                                        unsigned char* __restrict__ img, int* __restrict__ expo) {
+  constexpr int kCols = kSliceCols, kGroups = 256 / kCols;
+  static_assert(2 * kGroups * 8 >= kTtmChainMax, "two chunks per thread hold a column");
+  __shared__ int red[kGroups][kCols + 1];
+  const int ml = threadIdx.x % kCols, g = threadIdx.x / kCols;
+  for (int64_t m0 = (int64_t)blockIdx.x * kCols; m0 < Mpad; m0 += (int64_t)gridDim.x * kCols) {
+    const int64_t m = m0 + ml;
+    const bool mv = m < M;
+    double x[2][8];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int k = 8 * (g + j * kGroups) + e;
+        x[j][e] = mv && k < K ? __ldg(X + (int64_t)k * ld + m) : 0.0;
+      }
+    int top = INT_MIN;   // largest biased exponent after scaling
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int k = 8 * (g + j * kGroups) + e;
+        const unsigned long long u = (unsigned long long)__double_as_longlong(x[j][e]) & 0x7fffffffffffffffull;
+        const int ef = (int)(u >> 52);
+        if (ef == 2047)
+          top = INT_MAX;
+        else if (u != 0)
+          top = max(top, (ef > 1 ? ef : 1) + sgn * __ldg(kexp + k));
+      }
+    __syncthreads();   // red of the previous columns is consumed
+    red[g][ml] = top;
+    __syncthreads();
+    for (int i = 0; i < kGroups; ++i) top = max(top, red[i][ml]);
+    const bool col_bad = top == INT_MAX;
+    const int E = (col_bad || top == INT_MIN) ? 0 : top - 1022;
+    if (g == 0) expo[m] = col_bad ? kTtmBadExp : E;
+    const int64_t tile = m / TILE;
+    const int row = (int)(m - tile * TILE);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int ch = g + j * kGroups;
+      if (ch >= 2 * nk) break;
+      uint32_t w[P][4];
+#pragma unroll
+      for (int pr = 0; pr < 4; ++pr) {
+        uint32_t lo[P], hi[P];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int k = 8 * ch + 2 * pr + e;
+          long long v = 0;
+          const unsigned long long b = (unsigned long long)__double_as_longlong(x[j][2 * pr + e]);
+          if ((b << 1) != 0 && !col_bad) {   // entries beyond K were loaded as zeros
+            const int ef = (int)((b >> 52) & 2047);
+            unsigned long long mant = b & 0xfffffffffffffull;
+            if (ef > 0) mant |= 1ull << 52;
+            // |x| 2^(58 - E) rounded: shift <= 5 as |x| < 2^E
+            const int sh = (ef > 0 ? ef : 1) + sgn * __ldg(kexp + k) - E - 1017;
+            if (sh >= 0)
+              mant <<= sh;
+            else
+              mant = sh < -54 ? 0ull : (mant + (1ull << (-sh - 1))) >> (-sh);
+            v = (b >> 63) ? -(long long)mant : (long long)mant;
+          }
+          // balanced digits: add half of every field, read the fields unsigned
+          constexpr long long kHalf = 256ll + (64ll << 9) + (64ll << 16) + (64ll << 23) + (64ll << 30) + (64ll << 37) +
+                                      (64ll << 44);
+          v += kHalf;
+          uint32_t d[P];
+          d[0] = __float_as_uint(__int_as_float(0x4B400000 + (int)(v >> 51)) - 12582912.f);
+#pragma unroll
+          for (int s = 1; s < P - 1; ++s)
+            d[s] = __float_as_uint(__int_as_float(0x4B400000 - 64 + (int)((v >> (51 - 7 * s)) & 127)) - 12582912.f);
+          d[P - 1] = __float_as_uint((__int_as_float(0x4B400000 - 256 + (int)(v & 511)) - 12582912.f) * 0.25f);
+#pragma unroll
+          for (int s = 0; s < P; ++s) (e == 0 ? lo[s] : hi[s]) = d[s];
+        }
+#pragma unroll
+        for (int s = 0; s < P; ++s) w[s][pr] = __byte_perm(lo[s], hi[s], 0x7632);   // high halves: BF16
+      }
+      unsigned char* dst = img + (tile * nk + (ch >> 1)) * (int64_t)(P * TILE * kRow) + (row >> 3) * (8 * kRow) +
+                           (row & 7) * kRow + (((ch & 1) ^ ((row >> 2) & 1)) << 4);
+#pragma unroll
+      for (int s = 0; s < P; ++s)
+        *reinterpret_cast<uint4*>(dst + s * (TILE * kRow)) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+    }
+  }
+}
+
+// kexp[i] = exponent F_i with max_j |T_(a)(i, j)| < 2^F_i (0 for a zero slice);
+// *bad = 1 if an entry is Inf or NaN.
+__global__ void slice_exponent_kernel(const double* __restrict__ Tn, int64_t J, int* __restrict__ kexp,
+                                      int* __restrict__ bad) {
+  __shared__ int red[8];
+  const int64_t i = blockIdx.x;
+  int top = 0;
+  for (int64_t j = threadIdx.x; j < J; j += blockDim.x) {
+    const unsigned long long u =
+        (unsigned long long)__double_as_longlong(__ldg(Tn + i * J + j)) & 0x7fffffffffffffffull;
+    const int ef = (int)(u >> 52);
+    if (u != 0) top = max(top, ef > 1 ? ef : 1);
+  }
+  for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) top = max(top, red[w]);
+    if (top == 2047) *bad = 1;
+    kexp[i] = top == 0 ? 0 : top - 1022;
+  }
+}
+
+// ---- the product ------------------------------------------------------------------
+__device__ __forceinline__ uint64_t smem_desc32(uint32_t saddr) {   // K-major, 32-byte swizzle
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)((8 * kRow) >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(taddr));
+}
+
+// m0 2^21 + m1 2^14 + m2 2^7 + m3 of four level sums (integers; the last one may
+// carry a fraction, rounded here).  |m| <= 2^22, the usual case: after adding
+// 1.5 2^23 the low mantissa bits are the integer.  Level sums of strongly
+// correlated digits may reach 2^24: those are converted (a quarter of the rate).
+__device__ __forceinline__ long long sum_levels(uint32_t m0, uint32_t m1, uint32_t m2, uint32_t m3) {
+  constexpr float kRound = 12582912.f;   // 1.5 * 2^23: bits 0x4B400000
+  const uint32_t b0 = __float_as_uint(__uint_as_float(m0) + kRound), b1 = __float_as_uint(__uint_as_float(m1) + kRound);
+  const uint32_t b2 = __float_as_uint(__uint_as_float(m2) + kRound), b3 = __float_as_uint(__uint_as_float(m3) + kRound);
+  const uint32_t chk = (b0 ^ 0x4B000000u) | (b1 ^ 0x4B000000u) | (b2 ^ 0x4B000000u) | (b3 ^ 0x4B000000u);
+  if ((chk & 0xFF800000u) != 0)
+    return ((long long)__float2int_rn(__uint_as_float(m0)) << 21) + ((long long)__float2int_rn(__uint_as_float(m1)) << 14) +
+           ((long long)__float2int_rn(__uint_as_float(m2)) << 7) + (long long)__float2int_rn(__uint_as_float(m3));
+  constexpr long long kBias = 0x4B400000ll * ((1 << 21) + (1 << 14) + (1 << 7) + 1);
+  return (long long)((unsigned long long)b0 << 21) + (long long)((unsigned long long)b1 << 14) +
+         (long long)((unsigned long long)b2 << 7) + (long long)b3 - kBias;
+}
+
+// (hi + lo 2^-28) 2^(ex - 35) rounded to FP64, |hi| < 2^47, lo < 2^28, in
+// integers: one FP64 add per output would take 4096 cycles of GB300's FP64 pipe
+// (two lanes per clock and SM) per tile.
+__device__ __forceinline__ double round_levels(long long hi, uint32_t lo, int ex) {
+  // magnitude by the ones' complement (off by one unit of level 7)
+  const uint32_t s = (uint32_t)(hi >> 63);
+  const uint32_t h1 = (uint32_t)((unsigned long long)hi >> 32) ^ s, h0 = (uint32_t)hi ^ s;
+  const uint32_t l1 = (lo ^ s) << 4;   // 28 bits, left aligned
+  const bool small = h1 == 0;
+  const uint32_t w2 = small ? h0 : h1, w1 = small ? l1 : h0, w0 = small ? 0u : l1;
+  const int n = __clz((int)w2);
+  const uint32_t m1 = __funnelshift_l(w1, w2, n), m0 = __funnelshift_l(w0, w1, n);
+  const int be = 1023 + 28 + ex - n - (small ? 32 : 0);
+  if (w2 == 0 || be < 1 || be > 2045)
+    // rare: zeros, sums below 2^-35 of the vectors' maxima, results outside the
+    // normal range (both addends exact: one rounding, and scalbn's)
+    return scalbn(fma((double)lo, 1.0 / 268435456.0, (double)hi), ex - 35);
+  const unsigned long long q =
+      ((((unsigned long long)m1 << 32) | m0) >> 11) + ((m0 >> 10) & 1u) + ((unsigned long long)(uint32_t)(be - 1) << 52);
+  return __longlong_as_double((long long)(q | ((unsigned long long)(s & 0x80000000u) << 32)));
+}
+
+// Persistent: one CTA per SM (all of TMEM, 4 x 48 KB stages) walks the 128 x 64
+// tiles of Y, C tiles fastest so that the CTAs in flight share T's images in L2.
+//   warp 16  TMA: one lane refills the ring in order, across tile boundaries
+//   warp 17  one lane issues the stage's 12 MMAs (B digits stacked along N, up to
+//            256 wide: digit s of U against digits t0..t1 of T lands in levels
+//            s + t0 .. s + t1, 64 columns each)
+//   warps 0-15  drain: 32 columns c x 16 rows r each, levels to FP64, Y
+// Bound: the tensor pipe, 1152 cycles per 16 rows of the contraction and tile.
+// TMEM holds one accumulator set, so the next tile's first MMA waits until every
+// level is read: the drain takes the levels into 64-bit integers first (exposed)
+// and rounds and stores them under the next tile's MMAs.
+__global__ void __launch_bounds__(kThreads, 1) ttm_f64_kernel(const TtmArgs a) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* ring =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)kStages * kStage);
+  uint64_t* empty = full + kStages;
+  uint64_t* accum = empty + kStages;      // a tile's MMAs are complete
+  uint64_t* tmem_empty = accum + 1;       // the drain has read the accumulators
+  uint64_t* drain = accum + 2;            // abort path: the MMAs so far are complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum + 3);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(accum, 1);
+    mbar_init(tmem_empty, kEpiWarps);
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    fence_barrier_init();
+  }
+  if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int64_t ntiles = (int64_t)a.tiles_c * a.tiles_r;
+  const int nk = a.nk;
+
+  if (warp == kTmaWarp) {
+    if (lane == 0) {
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true, issued = false;
+      for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        const int64_t tr = t / a.tiles_c;
+        const unsigned char* srca = a.At + (t - tr * a.tiles_c) * nk * (int64_t)kAStage;
+        const unsigned char* srcb = a.Bt + tr * nk * (int64_t)kBStage;
+        for (int ks = 0; ks < nk; ++ks) {
+          ok = wait_bounded(&empty[s], ph ^ 1u, abort_flag, a.err, 1);
+          if (!ok) break;
+          unsigned char* dst = ring + (size_t)s * kStage;
+          mbar_arrive_expect_tx(&full[s], kStage);
+          bulk_load(dst, srca + (int64_t)ks * kAStage, kAStage, &full[s]);
+          bulk_load(dst + kAStage, srcb + (int64_t)ks * kBStage, kBStage, &full[s]);
+          issued = true;
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      if (*abort_flag && issued) {   // let the copies in flight land before the CTA exits
+        const uint64_t t0 = global_ns();
+        while (global_ns() - t0 < 200000ull) {
+        }
+      }
+    }
+  } else if (warp == kMmaWarp) {
+    if (lane == 0) {
+      const uint64_t desc0 = smem_desc32(smem_u32(ring));
+      uint32_t idesc[5];
+#pragma unroll
+      for (int c = 0; c < 5; ++c)   // FP32 accumulator, BF16 operands, both K-major, N >> 3, M >> 4
+        idesc[c] = (1u << 4) | (1u << 7) | (1u << 10) | (((uint32_t)(c * kTileN) >> 3) << 17) |
+                   ((uint32_t)(kTileM >> 4) << 24);
+      int s = 0;
+      uint32_t ph = 0, use = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++use) {
+        if (use > 0) {
+          ok = wait_bounded(tmem_empty, (use - 1) & 1u, abort_flag, a.err, 7);
+          if (!ok) break;
+          tc_fence_after();
+        }
+        for (int ks = 0; ks < nk; ++ks) {
+          ok = wait_bounded(&full[s], ph, abort_flag, a.err, 2);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t ad = desc0 + (uint64_t)(((uint32_t)s * kStage) >> 4);
+          const uint64_t bd = ad + (uint64_t)(kAStage >> 4);
+#pragma unroll
+          for (int p = 0; p < P; ++p) {
+#pragma unroll
+            for (int t0 = 0; t0 < P - p; t0 += 4) {
+              const int cnt = P - p - t0 < 4 ? P - p - t0 : 4;
+              tc_mma<kKindBF16>(tmem + (uint32_t)((p + t0) * kTileN), ad + (uint64_t)(p * (kABytes >> 4)),
+                                bd + (uint64_t)(t0 * (kBBytes >> 4)), idesc[cnt], (ks == 0 && p == 0) ? 0u : 1u);
+            }
+          }
+          tc_commit(&empty[s]);
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+        if (ok) tc_commit(accum);
+      }
+      if (!ok) {
+        tc_commit(drain);
+        wait_drain(drain, 0);
+      }
+    }
+  } else {
+    const int quarter = warp & 3, grp = warp >> 2;
+    const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(16 * grp);
+    uint32_t use = 0;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++use) {
+      const int64_t tr = t / a.tiles_c;
+      const int c = (int)(t - tr * a.tiles_c) * kTileM + quarter * 32 + lane;
+      const int64_t r0 = tr * kTileN + 16 * grp;
+      const int ec = __ldg(a.cexp + c);   // padded to whole tiles, as rexp
+      bool have = wait_sleepy(accum, use & 1u, abort_flag, a.err, 5);
+      have = __all_sync(0xffffffffu, have);
+      if (!have) break;
+      tc_fence_after();
+      // read the levels into integers, so that the next tile's MMAs start early ...
+      long long hi[16];
+      uint32_t lo[16];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        uint32_t v[4][4];
+        __syncwarp();
+#pragma unroll
+        for (int l = 0; l < 4; ++l) tmem_ld4(base + (uint32_t)(l * kTileN + 4 * h), v[l]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) hi[4 * h + k] = sum_levels(v[0][k], v[1][k], v[2][k], v[3][k]);
+        __syncwarp();
+#pragma unroll
+        for (int l = 0; l < 4; ++l) tmem_ld4(base + (uint32_t)((l + 4) * kTileN + 4 * h), v[l]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const long long low = sum_levels(v[0][k], v[1][k], v[2][k], v[3][k]);
+          hi[4 * h + k] += low >> 28;
+          lo[4 * h + k] = (uint32_t)low & 0xFFFFFFFu;
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tmem_empty);
+      // ... and round and store them meanwhile
+      double* y = a.Y + r0 * a.C + c;
+#pragma unroll
+      for (int k = 0; k < 16; ++k, y += a.C) {
+        const int64_t r = r0 + k;
+        if (r >= a.J || c >= a.C) continue;
+        if (ec == kTtmBadExp) {
+          double acc = 0.0;
+          for (int i = 0; i < a.K; ++i)
+            acc = fma(__ldg(a.Tn + (int64_t)i * a.J + r), __ldg(a.U + (int64_t)i * a.C + c), acc);
+          *y = acc;
+        } else {
+          *y = round_levels(hi[k], lo[k], ec + __ldg(a.rexp + r));
+        }
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kTmemCols);
+  }
+}
+
+// ---- contraction with one more factor ------------------------------------------------
+// out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c].  A thread takes
+// RB outputs (h, l) of one column, so U's entry is loaded once per RB entries of X;
+// columns are fastest, so every load is coalesced.  Bound: X read once, against two
+// FP64 multiply-adds per clock and SM (4.6 TB/s of X at 1.9 GHz).
+template <int RB>
+__global__ void __launch_bounds__(256) contract_f64_kernel(const double* __restrict__ X, int64_t H, int Mm, int64_t L,
+                                                           int C, const double* __restrict__ U, int mchunk,
+                                                           double* __restrict__ out) {
+  const int64_t HL = H * L, groups = (HL + RB - 1) / RB;
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= groups * C) return;
+  const int64_t g = idx / C;
+  const int c = (int)(idx - g * C);
+  const int mb = blockIdx.y * mchunk, me = mb + mchunk < Mm ? mb + mchunk : Mm;
+  const double* x[RB];
+  double acc[RB];
+#pragma unroll
+  for (int q = 0; q < RB; ++q) {
+    const int64_t o = g * RB + q < HL ? g * RB + q : HL - 1;
+    const int64_t hh = o / L;
+    x[q] = X + ((hh * Mm + mb) * L + (o - hh * L)) * C + c;
+    acc[q] = 0.0;
+  }
+  const int64_t step = L * C;
+  const double* u = U + (int64_t)mb * C + c;
+  constexpr int UN = RB == 1 ? 8 : 4;
+  int m = mb;
+  for (; m + UN <= me; m += UN) {
+    double uv[UN], xv[UN][RB];
+#pragma unroll
+    for (int e = 0; e < UN; ++e) {
+      uv[e] = __ldg(u + (int64_t)e * C);
+#pragma unroll
+      for (int q = 0; q < RB; ++q) xv[e][q] = __ldg(x[q] + e * step);
+    }
+#pragma unroll
+    for (int e = 0; e < UN; ++e)
+#pragma unroll
+      for (int q = 0; q < RB; ++q) acc[q] = fma(xv[e][q], uv[e], acc[q]);
+    u += (int64_t)UN * C;
+#pragma unroll
+    for (int q = 0; q < RB; ++q) x[q] += UN * step;
+  }
+  for (; m < me; ++m) {
+    const double uv = __ldg(u);
+    u += C;
+#pragma unroll
+    for (int q = 0; q < RB; ++q) {
+      acc[q] = fma(__ldg(x[q]), uv, acc[q]);
+      x[q] += step;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < RB; ++q)
+    if (g * RB + q < HL) out[((int64_t)blockIdx.y * HL + g * RB + q) * C + c] = acc[q];
+}
+
+template <int TILE>
+cudaError_t launch_slice(const double* X, int K, int64_t M, int64_t ld, const int* kexp, int sgn, unsigned char* img,
+                         int* expo, cudaStream_t s) {
+  const int64_t Mpad = (M + TILE - 1) / TILE * TILE;
+  const int64_t blocks = Mpad / kSliceCols;
+  slice_f64_kernel<TILE><<<(unsigned)(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
+      X, K, M, ld, kexp, sgn, ttm_ksteps(K), Mpad, img, expo);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* kexp, int* bad, cudaStream_t s) {
+  slice_exponent_kernel<<<(unsigned)I, 256, 0, s>>>(Tn, J, kexp, bad);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt, int* rexp,
+                                cudaStream_t s) {
+  return launch_slice<kTileN>(Tn, I, J, J, kexp, -1, Bt, rexp, s);
+}
+
+cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At, int* cexp,
+                                cudaStream_t s) {
+  return launch_slice<kTileM>(U, I, C, C, kexp, +1, At, cexp, s);
+}
+
+cudaError_t prepare_ttm_f64() {
+  return cudaFuncSetAttribute(ttm_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+}
+
+cudaError_t launch_ttm_f64(const TtmArgs& a, int num_sms, cudaStream_t s) {
+  const int64_t tiles = (int64_t)a.tiles_c * a.tiles_r;
+  ttm_f64_kernel<<<(unsigned)(tiles < num_sms ? tiles : num_sms), kThreads, kSmem, s>>>(a);
+  return cudaGetLastError();
+}
+
+// Threads the contraction wants in flight: about 512 per SM hide an L2 round trip.
+static constexpr int64_t kContractThreads = 152 * 512;
+
+int contract_splits(int64_t HL, int Mm, int C) {
+  const int64_t threads = HL * C;
+  int64_t S = (kContractThreads + threads - 1) / threads;
+  if (S > (Mm + 7) / 8) S = (Mm + 7) / 8;
+  if (S < 1) S = 1;
+  const int chunk = (int)((Mm + S - 1) / S);
+  return (Mm + chunk - 1) / chunk;
+}
+
+cudaError_t launch_contract_f64(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
+                                double* out, cudaStream_t s) {
+  const int64_t HL = H * L;
+  const int chunk = (Mm + S - 1) / S;
+  // four outputs per thread where that still leaves enough threads
+  const int RB = HL * C / 4 >= kContractThreads ? 4 : 1;
+  const int64_t n = (HL + RB - 1) / RB * C;
+  const dim3 grid((unsigned)((n + 255) / 256), (unsigned)S);
+  if (RB == 4)
+    contract_f64_kernel<4><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+  else
+    contract_f64_kernel<1><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+  return cudaGetLastError();
+}
+
+}  // namespace jk
