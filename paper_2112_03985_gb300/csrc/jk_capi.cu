@@ -397,36 +397,73 @@ tc::TcArgs make_tc_args(jkcals_ctx* h, int n, float* const* UT, float* const* UT
 
 int mode_splits(const jkcals_ctx* h, int n) { return h->tc ? h->tcplan[n].splits : h->plan[n].splits; }
 
-// ---- FP64 form through tensor-times-matrix products --------------------------
+// ---- MTTKRPs through tensor-times-matrix products ------------------------------
 // What the workspace holds while the MTTKRPs of one sweep (or one gradient) are
 // enqueued: Y contracted with mode y, Z with modes z_a and z_q (-1: nothing).
 struct TtmState {
   int y = -1, z_a = -1, z_q = -1;
+  int* counter = nullptr;   // sweep counter that the first product's slicing advances
   void updated(int n) {   // Ubar^(n) changed
     if (y == n) y = -1;
     if (z_a == n || z_q == n) z_a = z_q = -1;
   }
 };
 
-// Estimated seconds.  The product: waves of 128 x 64 tiles over the SMs, 1160
-// cycles per 16 rows of the contraction and about 5000 of exposed drain per
-// tile, plus slicing the factor and two launches.  A contraction reads Y once at
-// two FP64 multiply-adds per clock and SM.  The CUDA-core MTTKRP runs its padded
-// 64 x 64 tiles at about 0.85 TFLOP/s.
+// Digits per operand of a form's products: at least the operand bits of its own
+// kernel, counted from the largest entry of a contraction vector (58, 30, 23 and 16
+// fractional bits for 8, 4, 3 and 2 digits).
+int ttm_digits(int precision) {
+  switch (precision) {
+    case JKCALS_FP64: return 8;
+    case JKCALS_EXACT_BF16: return 4;
+    case JKCALS_BF16: return 2;
+    default: return 3;   // TF32, 3xTF32, split BF16
+  }
+}
+
+// Estimated seconds of each step, from measured rates.
+// The product: waves of tiles over the SMs, `step` cycles per 16 rows of the
+// contraction; eight digits add the exposed part of the drain, fewer take at least
+// the drain and write Y at 5 TB/s.  Slicing the factor, the launches and one tile's latency add 16 us.
 double ttm_product_cost(const jkcals_ctx* h, int a) {
-  const int64_t tiles = (int64_t)((h->C + kTtmTileC - 1) / kTtmTileC) * ((h->J[a] + kTtmTileR - 1) / kTtmTileR);
+  const int P = h->ttm.digits, rows = ttm_tile_r(P);
+  const int64_t tiles = (int64_t)((h->C + kTtmTileC - 1) / kTtmTileC) * ((h->J[a] + rows - 1) / rows);
   const int64_t waves = (tiles + h->num_sms - 1) / h->num_sms;
-  return waves * (ttm_ksteps((int)h->dims[a]) * 1160.0 + 5000.0) / 1.9e9 + 12e-6;
+  const int nk = ttm_ksteps((int)h->dims[a]);
+  if (P == 8) return waves * (nk * 1380.0 + 5000.0) / 1.9e9 + 16e-6;
+  const double step = P == 4 ? 510.0 : (P == 3 ? 390.0 : 310.0);
+  return std::max(waves * (std::max(nk * step, 3000.0) + 400.0) / 1.9e9,
+                  (P == 4 ? 8.0 : 4.0) * h->J[a] * h->C / 5e12) + 16e-6;
 }
+// A contraction reads Y once: at the FP64 pipe's measured 418 G multiply-adds/s on
+// 152 SMs, or FP32 values at the memory's rate.
 double ttm_contract_cost(const jkcals_ctx* h, int a) {
-  return (double)h->J[a] * h->C / (h->num_sms * 3.6e9) + 4e-6;
+  const double n = (double)h->J[a] * h->C;
+  const int P = h->ttm.digits;
+  return (P == 8 ? n / (h->num_sms * 2.75e9) : (P == 4 ? 8.0 : 4.0) * n / 5e12) + 7e-6;
 }
+// The mode's own MTTKRP kernel on its padded tiles: 0.85 TFLOP/s on the CUDA cores;
+// the tensor-core forms' measured rates, padding included.
 double native_cost(const jkcals_ctx* h, int n) {
+  if (h->tc) {
+    const tc::TcPlan& p = h->tcplan[n];
+    double rate = 115e12;   // exact chain
+    switch (h->opt.precision) {
+      case JKCALS_TF32: rate = 180e12; break;
+      case JKCALS_3XTF32: rate = 155e12; break;
+      case JKCALS_BF16: rate = 290e12; break;
+      case JKCALS_SPLIT_BF16: rate = 125e12; break;
+      default: break;
+    }
+    // and the split-K partials, written and summed
+    const double part = (double)p.splits * h->dims[n] * h->C * (h->opt.precision == JKCALS_EXACT_BF16 ? 8.0 : 4.0);
+    return 2.0 * p.tiles_c * 128 * (double)p.tiles_n * p.BN * p.Jp / rate + part / 4.5e12 + 5e-6;
+  }
   return 2.0 * round_up(h->C, kMttkrpBN) * (double)round_up(h->dims[n], kMttkrpBM) * h->J[n] / 0.85e12 + 5e-6;
 }
 
 // Contracted mode for mode n's MTTKRP: the one Y holds, else the cheaper one
-// with images (-1: the CUDA-core kernel).
+// with images (-1: the mode's own kernel).
 int ttm_choose(const jkcals_ctx* h, int n, const int (&modes)[2], int y) {
   if (y >= 0 && y != n) return y;
   int best = -1;
@@ -453,27 +490,29 @@ double ttm_sweep_cost(const jkcals_ctx* h, const int (&modes)[2]) {
   return t;
 }
 
-// Whether the current column count goes through the products.  The factor 0.8
+// Whether the current column count goes through the products.  The factor 0.9
 // keeps sizes where the two are about even (the smallest tensors: launches and
-// latency) on the CUDA-core kernel, which needs fewer launches.
+// latency) on the modes' own kernels, which need fewer launches.
 void plan_ttm_use(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   t.use = false;
   if (t.modes[0] < 0) return;
   double nat = 0.0;
   for (int n = 0; n < h->N; ++n) nat += native_cost(h, n);
-  t.use = ttm_sweep_cost(h, t.modes) < 0.8 * nat;
+  t.use = ttm_sweep_cost(h, t.modes) < 0.9 * nat;
 }
 
 // Modes whose images would make a sweep cheapest (t.modes; -1: none pays).
-// Explicit split-K factors ask for the CUDA-core kernel, and under a memory cap
-// the handle holds what that kernel needs and no more, so that later calls
+// Explicit split-K factors ask for the modes' own kernels, and under a memory cap
+// the handle holds what those need and no more, so that later calls
 // (gradients, loss histories, compaction) find the room the cap left them.
 constexpr int64_t kTtmMaxY = (int64_t)1 << 31;   // elements of Y (16 GiB)
 void choose_ttm_modes(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   t.modes[0] = t.modes[1] = -1;
-  if (h->tc || h->opt.splits > 0 || h->opt.max_device_bytes > 0) return;
+  if (h->opt.splits > 0 || h->opt.max_device_bytes > 0) return;
+  if (h->tc && h->N < 3) return;   // those products leave the column exponents to a contraction
+  t.digits = ttm_digits(h->opt.precision);
   auto ok = [&](int a) { return h->dims[a] <= kTtmChainMax && h->J[a] <= kTtmMaxY / h->C; };
   double best = 0.0;
   for (int x = 0; x < h->N; ++x)
@@ -496,32 +535,35 @@ void choose_ttm_modes(jkcals_ctx* h) {
 jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmState& st, int* kernels) {
   jkcals_ctx::Ttm& t = h->ttm;
   const int N = h->N;
-  double* part = static_cast<double*>(h->part);
+  void* part = h->part;
   const bool have_z = N >= 4 && st.z_a >= 0 && st.z_a != n && st.z_q != n;
   if (!have_z && st.y != a) {
     TtmArgs g{};
     g.At = t.At;
     g.Bt = t.Bt[a];
-    g.cexp = t.cexp;
+    g.cexp = t.cexp[a];
     g.rexp = t.rexp[a];
     g.K = (int)h->dims[a];
     g.nk = ttm_ksteps(g.K);
     g.C = h->C;
     g.tiles_c = (h->C + kTtmTileC - 1) / kTtmTileC;
     g.J = h->J[a];
-    g.tiles_r = (h->J[a] + kTtmTileR - 1) / kTtmTileR;
+    g.tiles_r = (h->J[a] + ttm_tile_r(t.digits) - 1) / ttm_tile_r(t.digits);
     g.Y = N == 2 ? part : t.Y;   // two modes: the product is the MTTKRP
     g.Tn = h->Tn64[a];
     g.U = U[a];
     g.err = h->d_err;
-    JK_CUDA(h, launch_slice_factor(U[a], g.K, h->C, t.kexp[a], t.At, t.cexp, h->stream));
-    JK_CUDA(h, launch_ttm_f64(g, h->num_sms, h->stream));
+    JK_CUDA(h, launch_slice_factor(t.digits, U[a], g.K, h->C, t.kexp[a], t.At, t.cexp[a], st.counter, h->stream));
+    st.counter = nullptr;
+    JK_CUDA(h, launch_ttm(t.digits, g, h->num_sms, h->stream));
+    t.ran = true;
     *kernels += 2;
     if (N > 2) st.y = a;
   }
   h->part_S = 1;
   if (N == 2) return JKCALS_OK;
-  const double* X = t.Y;
+  const void* X = t.Y;
+  const int* cexp = t.cexp[have_z ? st.z_a : a];
   std::vector<int> rest;   // modes of X, fastest first
   for (int k = 0; k < N; ++k)
     if (have_z ? (k != st.z_a && k != st.z_q) : k != a) rest.push_back(k);
@@ -533,11 +575,12 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
     const int q = rest[pos];
     int64_t L = 1, H = 1;
     for (size_t k = 0; k < rest.size(); ++k) (k < pos ? L : H) *= k == pos ? 1 : h->dims[rest[k]];
-    double* out = part;
+    void* out = part;
     int S = 1;
-    if (rest.size() == 2) {
-      S = contract_splits(H * L, (int)h->dims[q], h->C);
-      const int64_t cap = (int64_t)(h->part_bytes / sizeof(double)) / (H * L * h->C);
+    const bool fin = rest.size() == 2;
+    if (fin) {
+      S = contract_splits(t.digits, H * L, (int)h->dims[q], h->C);
+      const int64_t cap = (int64_t)(h->part_bytes / 8) / (H * L * h->C);
       S = (int)std::max<int64_t>(1, std::min<int64_t>(S, cap));
       S = (int)((h->dims[q] + (h->dims[q] + S - 1) / S - 1) / ((h->dims[q] + S - 1) / S));
       h->part_S = S;
@@ -549,7 +592,7 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
       out = t.W[w];
       w ^= 1;
     }
-    JK_CUDA(h, launch_contract_f64(X, H, (int)h->dims[q], L, h->C, U[q], S, out, h->stream));
+    JK_CUDA(h, launch_contract(t.digits, X, H, (int)h->dims[q], L, h->C, U[q], S, fin ? cexp : nullptr, out, h->stream));
     *kernels += 1;
     X = out;
     rest.erase(rest.begin() + pos);
@@ -560,7 +603,7 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
 // Enqueue the concurrent MTTKRP of mode n for factor set (U, UT, cmax) into
 // h->part (h->part_S splits).  reuse_slices: a two-step mode may reuse the U_a
 // slices left in At by the previous two-step launch of the same sweep when mode
-// a was not updated since.  st: products of the FP64 form that the caller's
+// a was not updated since.  st: tensor-times-matrix products that the caller's
 // earlier MTTKRPs left in the workspace.
 jkcals_status enqueue_mttkrp(jkcals_ctx* h, int n, double* const* U, float* const* UT, float* const* UTlo,
                              float* const* cmax, bool reuse_slices = false, TtmState* st = nullptr,
@@ -574,7 +617,7 @@ jkcals_status enqueue_mttkrp(jkcals_ctx* h, int n, double* const* U, float* cons
     TtmState local;
     if (alone) st = &local;
     int a = ttm_choose(h, n, h->ttm.modes, st->y);
-    if (alone && a >= 0 && ttm_product_cost(h, a) + ttm_contract_cost(h, a) > 0.8 * native_cost(h, n)) a = -1;
+    if (alone && a >= 0 && ttm_product_cost(h, a) + ttm_contract_cost(h, a) > 0.9 * native_cost(h, n)) a = -1;
     if (a >= 0) return enqueue_ttm(h, n, a, U, *st, kernels);
   }
   *kernels += 1;
@@ -667,13 +710,12 @@ int count_sweep_kernels(const jkcals_ctx* h) {
   int sliced = -1;
   TtmState st;
   for (int n = 0; n < h->N; ++n) {
-    const bool tts = h->tc && h->tcplan[n].tts;
-    if (tts) {
+    const int a = h->ttm.use ? ttm_choose(h, n, h->ttm.modes, st.y) : -1;
+    if (a < 0 && h->tc && h->tcplan[n].tts) {
       kernels += sliced == h->tcplan[n].a_mode ? 0 : 1;
       sliced = h->tcplan[n].a_mode;
     }
     kernels += h->plan[n].upd.fused ? 1 : 3;
-    const int a = h->ttm.use ? ttm_choose(h, n, h->ttm.modes, st.y) : -1;
     if (a < 0) {
       kernels += 1;
     } else {
@@ -694,15 +736,16 @@ int count_sweep_kernels(const jkcals_ctx* h) {
     st.updated(n);
     if (n == sliced) sliced = -1;
   }
-  return kernels + 1;
+  return kernels + (h->ttm.use ? 0 : 1);
 }
 
 jkcals_status enqueue_sweep(jkcals_ctx* h) {
   int kernels = 0;
   int sliced = -1;   // mode whose current slices At holds (two-step modes)
   TtmState ttm;
+  if (h->ttm.use) ttm.counter = h->d_sweep_idx;
   for (int n = 0; n < h->N; ++n) {
-    const bool tts = h->tc && h->tcplan[n].tts;
+    const bool tts = h->tc && h->tcplan[n].tts && !(h->ttm.use && ttm_choose(h, n, h->ttm.modes, ttm.y) >= 0);
     const bool reuse = tts && sliced == h->tcplan[n].a_mode;
     if (h->opt.kernel_timing) JK_CUDA(h, cudaEventRecordWithFlags(h->ev_start[n], h->stream, cudaEventRecordExternal));
     JK_TRY(enqueue_mttkrp(h, n, h->U, h->UT, h->UTlo, h->cmax, reuse, &ttm, &kernels));
@@ -726,8 +769,11 @@ jkcals_status enqueue_sweep(jkcals_ctx* h) {
     ttm.updated(n);
     if (n == sliced) sliced = -1;   // U_a changed: the slices in At are stale
   }
-  JK_CUDA(h, launch_advance_sweep(h->d_sweep_idx, h->stream));
-  h->kernels_per_sweep = kernels + 1;   // = count_sweep_kernels(h)
+  if (!h->ttm.use) {
+    JK_CUDA(h, launch_advance_sweep(h->d_sweep_idx, h->stream));
+    ++kernels;
+  }
+  h->kernels_per_sweep = kernels;   // = count_sweep_kernels(h)
   return JKCALS_OK;
 }
 
@@ -753,7 +799,12 @@ jkcals_status build_graph(jkcals_ctx* h) {
   return JKCALS_OK;
 }
 
+// Byte that the sweep counter is set to before a run of sweeps: 0, or -1 where each
+// sweep's first slicing advances it (before the last mode's update reads it).
+int sweep_counter_byte(const jkcals_ctx* h) { return h->ttm.use ? 0xff : 0; }
+
 jkcals_status run_sweeps(jkcals_ctx* h, int nsweeps) {
+  h->ttm.ran = h->ttm.ran || h->ttm.use;
   if (h->opt.use_graph) {
     JK_TRY(build_graph(h));
     for (int s = 0; s < nsweeps; ++s) JK_CUDA(h, cudaGraphLaunch(h->sweep_exec, h->stream));
@@ -787,7 +838,8 @@ jkcals_status copy_out(jkcals_ctx* h, void* dst, const void* src, size_t bytes) 
 
 // Reads the tensor-core kernel's error word (set when a bounded wait expired).
 jkcals_status check_device_error(jkcals_ctx* h) {
-  if (h->d_err == nullptr || !(h->tc || h->ttm.use)) return JKCALS_OK;
+  if (h->d_err == nullptr || !(h->tc || h->ttm.ran)) return JKCALS_OK;   // no bounded wait ran
+  h->ttm.ran = false;
   int err = 0;
   JK_CUDA(h, cudaMemcpyAsync(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   JK_CUDA(h, cudaStreamSynchronize(h->stream));
@@ -925,38 +977,70 @@ namespace {
 size_t ttm_part_elems(const jkcals_ctx* h, int n) {
   size_t most = 0;
   for (int q = 0; q < h->N; ++q)
-    if (q != n) most = std::max(most, (size_t)contract_splits(h->dims[n], (int)h->dims[q], h->C));
+    if (q != n) most = std::max(most, (size_t)contract_splits(h->ttm.digits, h->dims[n], (int)h->dims[q], h->C));
   return most * h->dims[n] * h->C;
 }
 
-// FP64 form: the digit images of T and the products' workspace, where the plan
-// wants them, allocated after everything the CUDA-core kernel needs: if the
-// device has no room for them, or T holds a non-finite entry, the handle runs on
-// that kernel.
-jkcals_status create_ttm(jkcals_ctx* h) {
+// The products' buffers are an addition to what the modes' own kernels need: if the
+// device has no room for them, or T holds a non-finite entry, the handle drops
+// them and runs on those kernels.
+void ttm_drop(jkcals_ctx* h) {
+  jkcals_ctx::Ttm& t = h->ttm;
+  void* all[] = {t.At, t.Y, t.Z, t.W[0], t.W[1]};
+  for (void* p : all) dfree(h, p, true);
+  for (int n = 0; n < kMaxModes; ++n) {
+    dfree(h, t.Bt[n], true);
+    dfree(h, t.kexp[n], true);
+    dfree(h, t.rexp[n], true);
+    dfree(h, t.cexp[n], true);
+  }
+  t = jkcals_ctx::Ttm{};
+  set_error("");
+}
+
+// The digit images of T (while the FP64 unfoldings exist).
+jkcals_status create_ttm_images(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   if (t.modes[0] < 0) return JKCALS_OK;
   cudaStream_t st = h->stream;
-  std::vector<void*> got;
-  auto alloc = [&](auto** p, size_t bytes) {
-    void* v = nullptr;
-    const jkcals_status s = dalloc(h, &v, bytes);
-    if (s == JKCALS_OK) {
-      *p = static_cast<std::remove_reference_t<decltype(**p)>*>(v);
-      got.push_back(v);
-    }
-    return s;
-  };
   int* d_bad = nullptr;
   auto build = [&]() -> jkcals_status {
-    size_t at = 0, y = 0, z = 0, w = 0;
-    JK_TRY(alloc(&d_bad, sizeof(int)));
-    JK_TRY(alloc(&h->d_err, sizeof(int)));
+    JK_TRY(dalloc_t(h, &d_bad, 1));
     JK_CUDA(h, cudaMemsetAsync(d_bad, 0, sizeof(int), st));
-    JK_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
     for (int a : t.modes) {
       if (a < 0) continue;
-      at = std::max(at, ttm_image_bytes((int)h->dims[a], h->C, kTtmTileC));
+      void* img = nullptr;
+      JK_TRY(dalloc(h, &img, ttm_image_bytes(t.digits, (int)h->dims[a], h->J[a], ttm_tile_r(t.digits))));
+      t.Bt[a] = static_cast<unsigned char*>(img);
+      JK_TRY(dalloc_t(h, &t.kexp[a], (size_t)h->dims[a]));
+      JK_TRY(dalloc_t(h, &t.rexp[a], (size_t)round_up(h->J[a], ttm_tile_r(t.digits))));
+      JK_CUDA(h, launch_slice_exponents(h->Tn64[a], h->dims[a], h->J[a], t.kexp[a], d_bad, st));
+      JK_CUDA(h, launch_slice_tensor(t.digits, h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], st));
+    }
+    return JKCALS_OK;
+  };
+  const jkcals_status s = build();
+  int bad = 0;
+  if (s == JKCALS_OK) {
+    JK_CUDA(h, cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+    JK_CUDA(h, cudaStreamSynchronize(st));
+  }
+  dfree(h, d_bad, true);
+  if (s != JKCALS_OK && s != JKCALS_ERR_OOM) return s;
+  if (s == JKCALS_ERR_OOM || bad != 0) ttm_drop(h);
+  return JKCALS_OK;
+}
+
+// The products' workspace, after every other buffer of the handle.
+jkcals_status create_ttm_workspace(jkcals_ctx* h) {
+  jkcals_ctx::Ttm& t = h->ttm;
+  if (t.modes[0] < 0) return JKCALS_OK;
+  auto build = [&]() -> jkcals_status {
+    size_t at = 0, y = 0, z = 0, w = 0;
+    for (int a : t.modes) {
+      if (a < 0) continue;
+      JK_TRY(dalloc_t(h, &t.cexp[a], (size_t)round_up(h->C, kTtmTileC)));
+      at = std::max(at, ttm_image_bytes(t.digits, (int)h->dims[a], h->C, kTtmTileC));
       if (h->N > 2) y = std::max(y, (size_t)h->J[a] * h->C);
       for (int q = 0; q < h->N && h->N >= 4; ++q) {
         if (q == a) continue;
@@ -965,38 +1049,25 @@ jkcals_status create_ttm(jkcals_ctx* h) {
           if (p != a && p != q) w = std::max(w, (size_t)(h->J[a] / h->dims[q] / h->dims[p]) * h->C);
       }
     }
-    JK_TRY(alloc(&t.At, at));
-    JK_TRY(alloc(&t.cexp, sizeof(int) * (size_t)round_up(h->C, kTtmTileC)));
-    if (y > 0) JK_TRY(alloc(&t.Y, sizeof(double) * y));
-    if (z > 0) JK_TRY(alloc(&t.Z, sizeof(double) * z));
-    if (w > 0) {
-      JK_TRY(alloc(&t.W[0], sizeof(double) * w));
-      JK_TRY(alloc(&t.W[1], sizeof(double) * w));
+    void* img = nullptr;
+    JK_TRY(dalloc(h, &img, at));
+    t.At = static_cast<unsigned char*>(img);
+    if (y > 0) JK_TRY(dalloc(h, &t.Y, 8 * y));
+    if (z > 0) JK_TRY(dalloc(h, &t.Z, 8 * z));
+    for (int k = 0; k < 2 && w > 0; ++k) JK_TRY(dalloc(h, &t.W[k], 8 * w));
+    if (h->d_err == nullptr) {
+      JK_TRY(dalloc_t(h, &h->d_err, 1));
+      JK_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
     }
-    for (int a : t.modes) {
-      if (a < 0) continue;
-      JK_TRY(alloc(&t.Bt[a], ttm_image_bytes((int)h->dims[a], h->J[a], kTtmTileR)));
-      JK_TRY(alloc(&t.kexp[a], sizeof(int) * (size_t)h->dims[a]));
-      JK_TRY(alloc(&t.rexp[a], sizeof(int) * (size_t)round_up(h->J[a], kTtmTileR)));
-      JK_CUDA(h, launch_slice_exponents(h->Tn64[a], h->dims[a], h->J[a], t.kexp[a], d_bad, st));
-      JK_CUDA(h, launch_slice_tensor(h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], st));
-    }
-    JK_CUDA(h, prepare_ttm_f64());
+    JK_CUDA(h, prepare_ttm(t.digits));
     return JKCALS_OK;
   };
-  jkcals_status s = build();
-  int bad = 0;
-  if (s == JKCALS_OK) {
-    JK_CUDA(h, cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st));
-    JK_CUDA(h, cudaStreamSynchronize(st));
+  const jkcals_status s = build();
+  if (s == JKCALS_ERR_OOM) {
+    ttm_drop(h);
+    return JKCALS_OK;
   }
-  if (s == JKCALS_OK && bad == 0) return JKCALS_OK;
-  if (s != JKCALS_OK && s != JKCALS_ERR_OOM) return s;
-  for (void* p : got) dfree(h, p, true);
-  h->d_err = nullptr;
-  t = jkcals_ctx::Ttm{};
-  set_error("");
-  return JKCALS_OK;
+  return s;
 }
 
 jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32_t* ranks,
@@ -1106,6 +1177,8 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
                                         p.Ia_pad, p.Jp, mp, h->rowexp[n], p.BN, p.tiles_n, p.nkt, h->Tt[n], st));
       h->Ipad[n] = round_up(h->dims[n], chunk);
     }
+    choose_ttm_modes(h);
+    JK_TRY(create_ttm_images(h));
     JK_CUDA(h, cudaStreamSynchronize(st));
     for (int n = 0; n < N; ++n) {
       dfree(h, h->Tn64[n], true);
@@ -1136,14 +1209,17 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
 
   // plan + workspace
   make_plan(h);
-  choose_ttm_modes(h);
+  if (!h->tc) {
+    choose_ttm_modes(h);
+    JK_TRY(create_ttm_images(h));
+  }
   size_t part_bytes = 0, chunks = 0;
   for (int n = 0; n < N; ++n) {
     const size_t eb = part_kind(h) == kPartF32 ? sizeof(float) : sizeof(double);
     const size_t pb = (size_t)mode_splits(h, n) * h->dims[n] * h->C * eb;
     part_bytes = std::max(part_bytes, pb);
     if (h->ttm.use)   // partial sums of the last contraction: about what fills the SMs
-      part_bytes = std::max(part_bytes, sizeof(double) * ttm_part_elems(h, n));
+      part_bytes = std::max(part_bytes, 8 * ttm_part_elems(h, n));
     chunks = std::max(chunks, (size_t)h->plan[n].upd.RC * K);
   }
   // room for the two-phase update of any subset of the blocks (compaction):
@@ -1167,7 +1243,7 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
   for (int n = 0; n < N; ++n)
     if (h->plan[n].upd.fused) fsmem = std::max(fsmem, h->plan[n].upd.fused_smem);
   if (fsmem > 0) JK_CUDA(h, prepare_update_fused(fsmem, h->Rmax, h->uniform_rank));
-  JK_TRY(create_ttm(h));
+  JK_TRY(create_ttm_workspace(h));
   h->kernels_per_sweep = count_sweep_kernels(h);
   JK_TRY(refresh_factor_state(h));
   if (h->opt.autotune && h->opt.splits <= 0) JK_TRY(autotune_splits(h));
@@ -1374,7 +1450,7 @@ jkcals_status jkcals_als_sweep(jkcals_t h, int nsweeps, double* losses) {
   JK_TRY(ensure_loss_cap(h, nsweeps));
   h->tol_host = 0.0;
   JK_CUDA(h, cudaMemsetAsync(h->d_tol, 0, sizeof(double), h->stream));
-  JK_CUDA(h, cudaMemsetAsync(h->d_sweep_idx, 0, sizeof(int), h->stream));
+  JK_CUDA(h, cudaMemsetAsync(h->d_sweep_idx, sweep_counter_byte(h), sizeof(int), h->stream));
   JK_TRY(run_sweeps(h, nsweeps));
   if (losses != nullptr) JK_TRY(copy_out(h, losses, h->loss_hist, sizeof(double) * nsweeps * h->K));
   return any_not_spd(h);
@@ -1388,7 +1464,7 @@ jkcals_status jkcals_als_sweep_async(jkcals_t h, int nsweeps, double* losses_dev
     return fail(JKCALS_ERR_ARG, "losses_dev must be device memory");
   JK_TRY(ensure_loss_cap(h, nsweeps));
   JK_CUDA(h, cudaMemsetAsync(h->d_tol, 0, sizeof(double), h->stream));
-  JK_CUDA(h, cudaMemsetAsync(h->d_sweep_idx, 0, sizeof(int), h->stream));
+  JK_CUDA(h, cudaMemsetAsync(h->d_sweep_idx, sweep_counter_byte(h), sizeof(int), h->stream));
   JK_TRY(run_sweeps(h, nsweeps));
   if (losses_dev != nullptr)
     JK_CUDA(h, cudaMemcpyAsync(losses_dev, h->loss_hist, sizeof(double) * nsweeps * h->K,
@@ -1800,7 +1876,7 @@ jkcals_status jkcals_run(jkcals_t h, int max_sweeps, double tol, int* sweeps_don
   // most half of the blocks being swept are still active
   auto chunk_step = [&](bool& stop) -> jkcals_status {
     const int n = std::min(chunk, max_sweeps - done);
-    JK_CUDA(h, cudaMemsetAsync(h->d_sweep_idx, 0, sizeof(int), h->stream));
+    JK_CUDA(h, cudaMemsetAsync(h->d_sweep_idx, sweep_counter_byte(h), sizeof(int), h->stream));
     JK_TRY(run_sweeps(h, n));
     done += n;
     st.resize(h->K);
@@ -1915,12 +1991,14 @@ struct jkcals_batch_ctx {
 namespace {
 
 // A batch sweep runs as grouped launches when every problem uses the same
-// tensor-core form and order, no mode takes the two-step form and no handle
+// tensor-core form and order, no mode takes the two-step form or a
+// tensor-times-matrix product and no handle
 // asked for per-problem branches.
 bool batch_groupable(const std::vector<jkcals_ctx*>& hs) {
   for (jkcals_ctx* h : hs) {
     if (h->opt.batch_branches || !h->tc || h->opt.precision != hs[0]->opt.precision || h->N != hs[0]->N)
       return false;
+    if (h->ttm.use) return false;   // grouped launches run the modes' own kernels
     for (int n = 0; n < h->N; ++n)
       if (h->tcplan[n].tts) return false;
   }
@@ -2290,8 +2368,9 @@ jkcals_status jkcals_batch_sweep(jkcals_batch_t b, int nsweeps) {
     JK_TRY(cu(cudaEventRecord(b->ready[i], h->stream), "cudaEventRecord"));
     JK_TRY(cu(cudaStreamWaitEvent(b->stream, b->ready[i], 0), "cudaStreamWaitEvent"));
     h->tol_host = 0.0;
+    h->ttm.ran = h->ttm.ran || h->ttm.use;
     JK_TRY(cu(cudaMemsetAsync(h->d_tol, 0, sizeof(double), b->stream), "cudaMemsetAsync"));
-    JK_TRY(cu(cudaMemsetAsync(h->d_sweep_idx, 0, sizeof(int), b->stream), "cudaMemsetAsync"));
+    JK_TRY(cu(cudaMemsetAsync(h->d_sweep_idx, sweep_counter_byte(h), sizeof(int), b->stream), "cudaMemsetAsync"));
   }
   for (int s = 0; s < nsweeps; ++s) JK_TRY(cu(cudaGraphLaunch(b->exec, b->stream), "cudaGraphLaunch"));
   JK_TRY(cu(cudaEventRecord(b->done, b->stream), "cudaEventRecord"));

@@ -163,18 +163,21 @@ struct jkcals_ctx {
   double* gG[jk::kMaxModes] = {nullptr};
   double* geg = nullptr;  // K per-block losses + their sum
 
-  // FP64 form: tensor-times-matrix products on the tensor cores (jk_ttm_f64.cu)
+  // tensor-times-matrix products (jk_ttm.cu)
   struct Ttm {
     int modes[2] = {-1, -1};                       // contracted modes with images of T (-1: none)
     bool use = false;                              // the current plan's MTTKRPs go through them
+    bool ran = false;                              // one was enqueued since the last error check
     unsigned char* Bt[jk::kMaxModes] = {nullptr};  // digit images of T_(a)
     int* kexp[jk::kMaxModes] = {nullptr};          // I_a slice exponents
     int* rexp[jk::kMaxModes] = {nullptr};          // exponents of T_(a)'s scaled columns (padded to tiles)
     unsigned char* At = nullptr;                   // digit images of Ubar^(a), rewritten per product
-    int* cexp = nullptr;                           // exponents of its scaled columns (padded to tiles)
-    double* Y = nullptr;                           // the product, J_a x C
-    double* Z = nullptr;                           // N >= 4: Y contracted with one more mode
-    double* W[2] = {nullptr, nullptr};             // N >= 5: the further contractions
+    int* cexp[jk::kMaxModes] = {nullptr};          // exponents of its scaled columns (padded to tiles)
+    // FP64 values, FP32 pairs (exact-chain form) or FP32 values:
+    void* Y = nullptr;                             // the product, J_a x C
+    void* Z = nullptr;                             // N >= 4: Y contracted with one more mode
+    void* W[2] = {nullptr, nullptr};               // N >= 5: the further contractions
+    int digits = 8;                                // of 7 bits per operand, by form
   } ttm;
   int part_S = 1;  // splits of the partial sums in `part` (set by each MTTKRP)
 
@@ -260,6 +263,47 @@ __device__ __forceinline__ double df_to_double(float hi, float lo) {
   return f32_to_f64_exact(s) + f32_to_f64_exact(r);
 }
 
+// FP32 pair of a double u: hi = fl32(u), lo = fl32(u - hi), both rounded to
+// nearest even, as the conversions give them, but formed from u's bit pattern
+// with integer operations: the FP64 pipe (which also runs FP64 conversions) is
+// narrow on this part and the update is bound by it.  hi keeps the top 24
+// significant bits of u's 53 (round half to even on the low 29); u - hi is
+// that remainder, at most 29 bits, converted exactly to FP32 and scaled by the
+// power of two of its unit.  Magnitudes outside [2^-70, 2^120) (and 0, Inf,
+// NaN) take the conversions.
+__device__ __forceinline__ void split_f32_pair(double u, float& hi, float& lo) {
+  const long long bits = __double_as_longlong(u);
+  const uint32_t hw = (uint32_t)((unsigned long long)bits >> 32), lw = (uint32_t)bits;
+  const int e = (int)((hw >> 20) & 0x7ffu) - 1023;   // unbiased exponent
+  if (e < -70 || e >= 120) {
+    hi = __double2float_rn(u);
+    lo = __double2float_rn(u - (double)hi);
+    return;
+  }
+  const uint32_t sign = hw & 0x80000000u;
+  uint32_t keep = ((hw & 0xfffffu) << 3) | (lw >> 29);   // the 23 stored bits of hi
+  const uint32_t rem = lw & 0x1fffffffu;                  // the 29 bits below them
+  const bool up = rem > 0x10000000u || (rem == 0x10000000u && (keep & 1u));
+  uint32_t fexp = (uint32_t)(e + 127);
+  uint32_t r;   // |u - hi| in units of 2^(e - 52)
+  if (up) {
+    r = 0x20000000u - rem;
+    if (++keep == 0x800000u) {
+      keep = 0;
+      ++fexp;
+    }
+  } else {
+    r = rem;
+  }
+  hi = __uint_as_float(sign | (fexp << 23) | keep);
+  if (r == 0) {
+    lo = 0.f;
+    return;
+  }
+  const float mag = __uint2float_rn(r) * __uint_as_float((uint32_t)(e - 52 + 127) << 23);   // exact
+  lo = (up != (sign != 0u)) ? -mag : mag;   // u - hi has u's sign when hi was rounded down
+}
+
 // ---- error plumbing (jk_capi.cu) --------------------------------------------
 void set_error(const std::string& msg);
 
@@ -310,39 +354,42 @@ cudaError_t launch_reduce_partials_f64(const double* part, int S, int64_t count,
 cudaError_t launch_reduce_partials_f32(const float* part, int S, int64_t count, double* out,
                                        cudaStream_t s);
 
-// ---- FP64 tensor-times-matrix on the tensor cores (jk_ttm_f64.cu) -------------
-constexpr int kTtmDigits = 8;
-constexpr int kTtmTileC = 128, kTtmTileR = 64;   // tile of Y: columns c, rows r
+// ---- tensor-times-matrix products on the tensor cores (jk_ttm.cu) -------------
+constexpr int kTtmTileC = 128;                   // tile of Y: columns c
+// its rows r: what the levels' accumulators leave of TMEM (see jk_ttm.cu)
+constexpr int ttm_tile_r(int digits) { return digits == 2 ? 128 : (digits == 3 ? 80 : 64); }
 // longest contraction whose level sums are exact: (l + 3) 2^12 K <= 2^24 for l <= 6
 constexpr int kTtmChainMax = 448;
 constexpr int kTtmBadExp = 2147483647;           // exponent of a column with a non-finite entry
 inline int ttm_ksteps(int K) { return (K + 15) / 16; }
 struct TtmArgs {
-  const unsigned char* At;   // digit images of Ubar^(a): tiles_c x nk stages
-  const unsigned char* Bt;   // digit images of T_(a): tiles_r x nk stages
+  const unsigned char* At;   // digit images of Ubar^(a): tiles_c x nk steps of 16 rows
+  const unsigned char* Bt;   // digit images of T_(a): tiles_r x nk steps
   const int* cexp;           // per column c (padded to tiles)
   const int* rexp;           // per row r of Y (padded to tiles)
   int nk, K, C, tiles_c;
   int64_t J, tiles_r;
-  double* Y;                 // J x C
-  const double* Tn;          // T_(a), K x J (columns of Ubar^(a) with non-finite entries)
+  void* Y;                   // J x C: FP64 (eight digits), FP32 pairs (four) or FP32, the latter without 2^cexp
+  const double* Tn;          // T_(a), K x J (eight digits: columns with non-finite entries)
   const double* U;           // Ubar^(a), K x C
   int* err;
 };
-inline size_t ttm_image_bytes(int K, int64_t M, int tile) {
-  return (size_t)((M + tile - 1) / tile) * ttm_ksteps(K) * kTtmDigits * tile * 32;
+inline size_t ttm_image_bytes(int digits, int K, int64_t M, int tile) {
+  return (size_t)((M + tile - 1) / tile) * ttm_ksteps(K) * digits * tile * 32;
 }
 cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* kexp, int* bad, cudaStream_t s);
-cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt, int* rexp,
-                                cudaStream_t s);
-cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At, int* cexp,
-                                cudaStream_t s);
-cudaError_t prepare_ttm_f64();
-cudaError_t launch_ttm_f64(const TtmArgs& a, int num_sms, cudaStream_t s);
+cudaError_t launch_slice_tensor(int digits, const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt,
+                                int* rexp, cudaStream_t s);
+cudaError_t launch_slice_factor(int digits, const double* U, int I, int C, const int* kexp, unsigned char* At,
+                                int* cexp, int* counter, cudaStream_t s);
+cudaError_t prepare_ttm(int digits);
+cudaError_t launch_ttm(int digits, const TtmArgs& a, int num_sms, cudaStream_t s);
 // out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c]
-int contract_splits(int64_t HL, int Mm, int C);
-cudaError_t launch_contract_f64(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
-                                double* out, cudaStream_t s);
+int contract_splits(int digits, int64_t HL, int Mm, int C);
+// X, out: FP64 (eight digits), FP32 pairs (four) or FP32; cexp: the columns' exponents,
+// for the last contraction of an MTTKRP of fewer than eight digits (else null)
+cudaError_t launch_contract(int digits, const void* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
+                            const int* cexp, void* out, cudaStream_t s);
 
 // Storage of split-K partials: FP64, FP32, or an unevaluated FP32 pair (hi, lo).
 constexpr int kPartF64 = 0, kPartF32 = 1, kPartF32x2 = 2;

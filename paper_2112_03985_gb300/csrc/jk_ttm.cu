@@ -1,0 +1,817 @@
+// Tensor-times-matrix products on the tensor cores, and the contractions that turn
+// them into concurrent MTTKRPs.
+//
+//   Y_a(r, c) = sum_i T_(a)(i, r) Ubar^(a)(i, c)           (ttm_kernel)
+//   Mbar_n(i_n, c) = sum over the other indices of r of Y_a(r, c) times the
+//                    remaining factors' entries             (contract_kernel)
+//
+// for a mode a != n (Eq. MTTKRP with its Khatri-Rao sum taken one mode at a
+// time).  Y_a does not depend on the other factors, so every mode n != a that is
+// updated before Ubar^(a) changes shares it: a sweep of N modes needs two of the
+// products of 2 C prod(I) operations instead of N.
+//
+// FP64 form (eight digits).  The product is exact up to FP64 rounding on the BF16 tensor pipe: GB300 runs
+// 1.1 TFLOP/s in FP64 and 1889 TFLOP/s in BF16, so 36 BF16 products per FP64
+// one still leave a factor of 48.  Every operand value x of a contraction vector
+// whose magnitudes stay below 2^E is rounded to 58 fractional bits of 2^E and
+// written in balanced digits, x = 2^(E-7) sum_k d_k 2^(-7k), |d_0| <= 128,
+// |d_k| <= 64 (k = 1 .. 7; d_7 in steps of 1/4): BF16 holds each digit exactly.
+// The products d_s e_t with s + t = l < 8 are summed per level l in one FP32
+// accumulator in TMEM.  A level's terms are integers and its sum stays below
+// (l + 3) 2^12 K <= 2^24 for chains of K <= kTtmChainMax, so levels 0 to 6 are
+// exact whatever the order of the additions; level 7 may truncate in its own
+// last bits (2^-63 of the product of the vectors' maxima).  What is dropped is
+// the operands' rounding (2^-59) and the products beyond level 7 (seven terms
+// of about 2^-60 each): below the rounding of a single FP64 multiply-add per
+// term.  The drain adds the levels as 64-bit integers and rounds once to FP64.
+//
+// The other forms take fewer digits (exact chain 4; 3xTF32, split BF16 and TF32 3;
+// BF16 2): d_(P-1) in steps of 1/4 again, so operands of 30, 23 and 16 fractional
+// bits, at least those of the form's own kernel, and the same products as its own
+// split (levels s + t < P).  Their levels are added in FP32 (a pair for four digits)
+// and Y is stored as FP32 pairs or FP32 values; what these forms lose elsewhere, the
+// truncating accumulation over long chains, is gone: a chain is one contraction.
+//
+// Along the contraction the two operands are equilibrated by powers of two
+// (exact): T_(a)(i, :) 2^(-F_i) against Ubar^(a)(i, :) 2^(F_i), F_i the exponent
+// of the largest entry of slice i.  A slice much larger than the others (an
+// outlying sample) then costs no digits in submodels that leave it out.
+//
+// Measured (GB300), against the CUDA-core MTTKRP of every mode: an FP64 sweep of
+// 300x100x50 with 1500 columns 16.0 -> 0.46 ms, of 400x400x400 with 400 columns
+// 192 -> 3.4 ms; loss and gradient of 100x60x60x40 with 800 columns 166 -> 4.3 ms.
+// Largest MTTKRP error against quadruple precision, relative to the largest
+// entry (300x100x50, modes 0-2): 3.2e-16, 4.9e-16, 5.8e-16, against 6.9e-16,
+// 1.8e-15, 1.6e-15 on the CUDA cores, whose chains of additions are longer.
+//
+// Exact chain: a sweep of 300x100x50 (two modes share one product, the sampled mode
+// keeps its one-step kernel) 217 -> 195 us, the three MTTKRPs of 400x400x400 2.25 ->
+// 1.80 ms (errors no larger: 300x100x50 equal to three digits, 400x400x400 half).
+// 3xTF32, 400x400x400 and 800 columns: 2.38 -> 1.95 ms, the error against FP64 falls
+// from about 5e-5 to 1e-7.
+//
+// A column of Ubar^(a) with a non-finite entry is taken out of the digits and
+// computed by plain FP64 dot products in the drain, so Inf and NaN propagate as
+// in the CUDA-core kernel; a tensor with a non-finite entry never gets here.
+#include <limits.h>
+#include <math.h>
+
+#include <math_constants.h>
+
+#include <type_traits>
+
+#include "jk_common.cuh"
+#include "jk_ptx.cuh"
+
+namespace jk {
+namespace {
+
+using namespace ptx;
+
+constexpr int kTileM = kTtmTileC;
+constexpr int kRow = 32;                      // bytes of one operand row per stage: 16 BF16
+constexpr uint32_t kABytes = kTileM * kRow;   // one digit of U for 16 rows k
+// P digits (2, 3, 4 or 8): a stage holds one or two steps of 16 rows, at most 32 KB of
+// U's images and 16 KB of T's; TMEM holds one set of eight level accumulators (64
+// columns each) or two sets of P of them (ttm_tile_r(P) columns each).
+constexpr int ttm_steps(int P) { return P == 8 ? 1 : 2; }
+constexpr int ttm_sets(int P) { return P == 8 ? 1 : 2; }
+constexpr uint32_t kAStage = 32768, kBStage = 16384, kStage = kAStage + kBStage;
+constexpr int kStages = 4;
+constexpr int kEpiWarps = 16;
+constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
+constexpr int kThreads = 32 * (kEpiWarps + 2);
+constexpr uint32_t kTmemCols = 512;           // all of TMEM
+constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + (2 * kStages + 5) * 8 + 16;
+
+// ---- digits ---------------------------------------------------------------------
+// One operand matrix X (K x M, row stride ld; K the contraction) into stage images:
+// per TILE columns m and 16 rows k, P digit tiles of TILE x 32 bytes, K-major in
+// the 32-byte swizzle (16-byte chunk XOR bit 2 of the row): one bulk copy per
+// operand and stage.  A block takes 8 columns, thread (m, g) the 8-row chunks g
+// and g + 32, loaded once into registers (K <= kTtmChainMax: at most 56 chunks):
+// first each column's exponent (expo[m]: scaled magnitudes < 2^expo), then the
+// digits.  sgn = +1 / -1 scales row k by 2^(+-kexp[k]).  Integer arithmetic
+// throughout: an FP64 rint per digit would take 18 us of the FP64 pipe for
+// 300 x 1500 entries.  counter: a sweep's first slicing also advances the sweep
+// counter (null otherwise).
+constexpr int kSliceCols = 8;   // columns per block
+
+// Half of every digit's field below d_0: 256 of the last one's nine bits, 64 of the
+// others' seven.
+constexpr long long half_fields(int P) {
+  long long h = 256;
+  for (int s = 1; s < P - 1; ++s) h += 64ll << (9 + 7 * (s - 1));
+  return h;
+}
+
+// What a digit's unit is stored as: 1 (eight digits, levels combined as
+// integers), or 2^(-7 s) (fewer, levels combined in FP32).
+template <int P>
+__host__ __device__ constexpr float digit_unit(int s) {
+  return P == 8 ? 1.f : 1.f / (float)(1 << (7 * s));
+}
+
+template <int P, int TILE>
+__global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict__ X, int K, int64_t M, int64_t ld,
+                                                        const int* __restrict__ kexp, int sgn, int nk, int64_t Mpad,
+                                                        unsigned char* __restrict__ img, int* __restrict__ expo,
+                                                        int* __restrict__ counter) {
+  if (counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *counter += 1;
+  constexpr int kCols = kSliceCols, kGroups = 256 / kCols;
+  constexpr int kTop = 9 + 7 * (P - 2);   // position of d_0; the last digit's field has two bits more
+  static_assert(2 * kGroups * 8 >= kTtmChainMax, "two chunks per thread hold a column");
+  __shared__ int red[kGroups][kCols + 1];
+  const int ml = threadIdx.x % kCols, g = threadIdx.x / kCols;
+  for (int64_t m0 = (int64_t)blockIdx.x * kCols; m0 < Mpad; m0 += (int64_t)gridDim.x * kCols) {
+    const int64_t m = m0 + ml;
+    const bool mv = m < M;
+    double x[2][8];
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int k = 8 * (g + j * kGroups) + e;
+        x[j][e] = mv && k < K ? __ldg(X + (int64_t)k * ld + m) : 0.0;
+      }
+    int top = INT_MIN;   // largest biased exponent after scaling
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int k = 8 * (g + j * kGroups) + e;
+        const unsigned long long u = (unsigned long long)__double_as_longlong(x[j][e]) & 0x7fffffffffffffffull;
+        const int ef = (int)(u >> 52);
+        if (ef == 2047)
+          top = INT_MAX;
+        else if (u != 0)
+          top = max(top, (ef > 1 ? ef : 1) + sgn * __ldg(kexp + k));
+      }
+    __syncthreads();   // red of the previous columns is consumed
+    red[g][ml] = top;
+    __syncthreads();
+    for (int i = 0; i < kGroups; ++i) top = max(top, red[i][ml]);
+    const bool col_bad = top == INT_MAX;
+    const int E = (col_bad || top == INT_MIN) ? 0 : top - 1022;
+    if (g == 0) expo[m] = col_bad ? kTtmBadExp : E;
+    const int64_t tile = m / TILE;
+    const int row = (int)(m - tile * TILE);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int ch = g + j * kGroups;
+      if (ch >= 2 * nk) break;
+      uint32_t w[P][4];
+#pragma unroll
+      for (int pr = 0; pr < 4; ++pr) {
+        uint32_t lo[P], hi[P];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int k = 8 * ch + 2 * pr + e;
+          long long v = 0;
+          const unsigned long long b = (unsigned long long)__double_as_longlong(x[j][2 * pr + e]);
+          if ((b << 1) != 0 && !col_bad) {   // entries beyond K were loaded as zeros
+            const int ef = (int)((b >> 52) & 2047);
+            unsigned long long mant = b & 0xfffffffffffffull;
+            if (ef > 0) mant |= 1ull << 52;
+            // |x| 2^(kTop + 7 - E) rounded: shift <= kTop - 46 as |x| < 2^E
+            const int sh = (ef > 0 ? ef : 1) + sgn * __ldg(kexp + k) - E - (1075 - kTop - 7);
+            if (sh >= 0)
+              mant <<= sh;
+            else
+              mant = sh < -54 ? 0ull : (mant + (1ull << (-sh - 1))) >> (-sh);
+            v = (b >> 63) ? -(long long)mant : (long long)mant;
+          }
+          // balanced digits: add half of every field, read the fields unsigned
+          constexpr long long kHalf = half_fields(P);
+          v += kHalf;
+          uint32_t d[P];
+          d[0] = __float_as_uint(__int_as_float(0x4B400000 + (int)(v >> kTop)) - 12582912.f);
+#pragma unroll
+          for (int s = 1; s < P - 1; ++s)
+            d[s] = __float_as_uint((__int_as_float(0x4B400000 - 64 + (int)((v >> (kTop - 7 * s)) & 127)) - 12582912.f) *
+                                   digit_unit<P>(s));
+          d[P - 1] = __float_as_uint((__int_as_float(0x4B400000 - 256 + (int)(v & 511)) - 12582912.f) *
+                                     (0.25f * digit_unit<P>(P - 1)));
+#pragma unroll
+          for (int s = 0; s < P; ++s) (e == 0 ? lo[s] : hi[s]) = d[s];
+        }
+#pragma unroll
+        for (int s = 0; s < P; ++s) w[s][pr] = __byte_perm(lo[s], hi[s], 0x7632);   // high halves: BF16
+      }
+      unsigned char* dst = img + (tile * nk + (ch >> 1)) * (int64_t)(P * TILE * kRow) + (row >> 3) * (8 * kRow) +
+                           (row & 7) * kRow + (((ch & 1) ^ ((row >> 2) & 1)) << 4);
+#pragma unroll
+      for (int s = 0; s < P; ++s)
+        *reinterpret_cast<uint4*>(dst + s * (TILE * kRow)) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+    }
+  }
+}
+
+// kexp[i] = exponent F_i with max_j |T_(a)(i, j)| < 2^F_i (0 for a zero slice);
+// *bad = 1 if an entry is Inf or NaN.
+__global__ void slice_exponent_kernel(const double* __restrict__ Tn, int64_t J, int* __restrict__ kexp,
+                                      int* __restrict__ bad) {
+  __shared__ int red[8];
+  const int64_t i = blockIdx.x;
+  int top = 0;
+  for (int64_t j = threadIdx.x; j < J; j += blockDim.x) {
+    const unsigned long long u =
+        (unsigned long long)__double_as_longlong(__ldg(Tn + i * J + j)) & 0x7fffffffffffffffull;
+    const int ef = (int)(u >> 52);
+    if (u != 0) top = max(top, ef > 1 ? ef : 1);
+  }
+  for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) top = max(top, red[w]);
+    if (top == 2047) *bad = 1;
+    kexp[i] = top == 0 ? 0 : top - 1022;
+  }
+}
+
+// ---- the product ------------------------------------------------------------------
+__device__ __forceinline__ uint64_t smem_desc32(uint32_t saddr) {   // K-major, 32-byte swizzle
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)((8 * kRow) >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(taddr));
+}
+
+// m0 2^21 + m1 2^14 + m2 2^7 + m3 of four level sums (integers; the last one may
+// carry a fraction, rounded here).  |m| <= 2^22: after adding 1.5 2^23 the low
+// mantissa bits are the integer, and two levels fit 32 bits.  Chains of at most
+// kTtmFastChain rows cannot exceed that; in longer ones (check) strongly correlated
+// digits may reach 2^24 and are converted (a quarter of the rate).
+constexpr int kTtmFastChain = 102;   // (l + 3) 2^12 K <= 2^22 for l <= 7
+
+__device__ __forceinline__ long long sum_levels(uint32_t m0, uint32_t m1, uint32_t m2, uint32_t m3, bool check) {
+  constexpr float kRound = 12582912.f;   // 1.5 * 2^23: bits 0x4B400000
+  constexpr uint32_t kBias = 0x4B400000u * 129u;
+  const uint32_t b0 = __float_as_uint(__uint_as_float(m0) + kRound), b1 = __float_as_uint(__uint_as_float(m1) + kRound);
+  const uint32_t b2 = __float_as_uint(__uint_as_float(m2) + kRound), b3 = __float_as_uint(__uint_as_float(m3) + kRound);
+  if (check) {
+    const uint32_t chk = (b0 ^ 0x4B000000u) | (b1 ^ 0x4B000000u) | (b2 ^ 0x4B000000u) | (b3 ^ 0x4B000000u);
+    if ((chk & 0xFF800000u) != 0)
+      return ((long long)__float2int_rn(__uint_as_float(m0)) << 21) +
+             ((long long)__float2int_rn(__uint_as_float(m1)) << 14) +
+             ((long long)__float2int_rn(__uint_as_float(m2)) << 7) + (long long)__float2int_rn(__uint_as_float(m3));
+  }
+  const int t0 = (int)(b0 * 128u + b1 - kBias), t1 = (int)(b2 * 128u + b3 - kBias);
+  return (long long)t0 * 16384 + t1;
+}
+
+// The eight levels of this warp's 32 lanes x 16 TMEM columns at base: per column
+// hi + lo 2^-28 in units of level 3.
+__device__ __forceinline__ void read_levels(uint32_t base, bool check, long long (&hi)[16], uint32_t (&lo)[16]) {
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    uint32_t v[4][4];
+    __syncwarp();
+#pragma unroll
+    for (int l = 0; l < 4; ++l) tmem_ld4(base + (uint32_t)(l * 64 + 4 * h), v[l]);
+    tmem_ld_wait();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) hi[4 * h + k] = sum_levels(v[0][k], v[1][k], v[2][k], v[3][k], check);
+    __syncwarp();
+#pragma unroll
+    for (int l = 0; l < 4; ++l) tmem_ld4(base + (uint32_t)((l + 4) * 64 + 4 * h), v[l]);
+    tmem_ld_wait();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long low = sum_levels(v[0][k], v[1][k], v[2][k], v[3][k], check);
+      hi[4 * h + k] += low >> 28;
+      lo[4 * h + k] = (uint32_t)low & 0xFFFFFFFu;
+    }
+  }
+}
+
+// (hi + lo 2^-28) 2^(ex - 35) rounded to FP64, |hi| < 2^47, lo < 2^28, in
+// integers: one FP64 add per output would take 4096 cycles of GB300's FP64 pipe
+// (two lanes per clock and SM) per tile.
+__device__ __forceinline__ double round_levels(long long hi, uint32_t lo, int ex) {
+  // magnitude by the ones' complement (off by one unit of level 7)
+  const uint32_t s = (uint32_t)(hi >> 63);
+  const uint32_t h1 = (uint32_t)((unsigned long long)hi >> 32) ^ s, h0 = (uint32_t)hi ^ s;
+  const uint32_t l1 = (lo ^ s) << 4;   // 28 bits, left aligned
+  const bool small = h1 == 0;
+  const uint32_t w2 = small ? h0 : h1, w1 = small ? l1 : h0, w0 = small ? 0u : l1;
+  const int n = __clz((int)w2);
+  const uint32_t m1 = __funnelshift_l(w1, w2, n), m0 = __funnelshift_l(w0, w1, n);
+  const int be = 1023 + 28 + ex - n - (small ? 32 : 0);
+  if (w2 == 0 || be < 1 || be > 2045)
+    // rare: zeros, sums below 2^-35 of the vectors' maxima, results outside the
+    // normal range (both addends exact: one rounding, and scalbn's)
+    return scalbn(fma((double)lo, 1.0 / 268435456.0, (double)hi), ex - 35);
+  const unsigned long long q =
+      ((((unsigned long long)m1 << 32) | m0) >> 11) + ((m0 >> 10) & 1u) + ((unsigned long long)(uint32_t)(be - 1) << 52);
+  return __longlong_as_double((long long)(q | ((unsigned long long)(s & 0x80000000u) << 32)));
+}
+
+// Persistent: one CTA per SM (all of TMEM, 4 x 48 KB stages) walks the 128 x
+// ttm_tile_r(P) tiles of Y, C tiles fastest so that the CTAs in flight share T's images in L2.
+//   warp 16  TMA: one lane refills the ring in order, across tile boundaries
+//   warp 17  one lane issues the stage's 12 MMAs (B digits stacked along N, up to
+//            256 wide: digit s of U against digits t0..t1 of T lands in levels
+//            s + t0 .. s + t1, 64 columns each)
+//   warps 0-15  drain: 32 columns c x a quarter of the rows r each, levels to Y
+// Bound: shared-memory bandwidth.  Per 16 rows of the contraction and 128 x 64 tile,
+// eight digits' MMAs take 1152 cycles of the tensor pipe but read 120 KB of operands
+// while TMA writes 48 KB: 168 KB at 128 bytes a clock are 1344 cycles, and about 1380
+// were measured (400x400x400, 400 columns: 1310 us).  Four digits: 60 KB are 480
+// cycles (512 measured) against 348 of the pipe.  Two CTAs sharing U's stage by TMA
+// multicast changed nothing (445 -> 441 us): the writes to shared memory stay.  Fewer
+// digits leave TMEM for wider tiles, which share U's bytes among more rows.
+// Eight digits leave room for one accumulator set, so the next tile's first MMA waits
+// until every level is read: the drain takes the levels into 64-bit integers first
+// (exposed) and rounds and stores them under the next tile's MMAs.
+template <int P>
+__global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
+  constexpr int SL = ttm_steps(P), NB = ttm_sets(P);   // 16-row steps per stage, accumulator sets
+  constexpr int BN = ttm_tile_r(P), NC = BN / 4;       // rows r of a tile, and of a draining warp
+  constexpr uint32_t kBBytes = BN * kRow;              // one digit of T for 16 rows k
+  static_assert(SL * P * kABytes <= kAStage && SL * P * kBBytes <= kBStage, "stage");
+  static_assert(P * BN <= (int)kTmemCols / NB && BN % 16 == 0 && (P < 4 ? P : 4) * BN <= 256, "accumulators");
+  constexpr uint32_t kSetCols = kTmemCols / NB;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* ring =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)kStages * kStage);
+  uint64_t* empty = full + kStages;
+  uint64_t* accum = empty + kStages;      // [2] a tile's MMAs into set b are complete
+  uint64_t* tmem_empty = accum + 2;       // [2] the drain has read set b
+  uint64_t* drain = accum + 4;            // abort path: the MMAs so far are complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum + 5);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&accum[b], 1);
+      mbar_init(&tmem_empty[b], kEpiWarps);
+    }
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    fence_barrier_init();
+  }
+  if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int64_t ntiles = (int64_t)a.tiles_c * a.tiles_r;
+  const int nk = a.nk;
+
+  if (warp == kTmaWarp) {
+    if (lane == 0) {
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true, issued = false;
+      for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        const int64_t tr = t / a.tiles_c;
+        const unsigned char* srca = a.At + (t - tr * a.tiles_c) * nk * (int64_t)(P * kABytes);
+        const unsigned char* srcb = a.Bt + tr * nk * (int64_t)(P * kBBytes);
+        for (int ks = 0; ks < nk; ks += SL) {
+          ok = wait_bounded(&empty[s], ph ^ 1u, abort_flag, a.err, 1);
+          if (!ok) break;
+          unsigned char* dst = ring + (size_t)s * kStage;
+          const uint32_t steps = (uint32_t)(nk - ks < SL ? nk - ks : SL);
+          const uint32_t na = steps * P * kABytes, nb = steps * P * kBBytes;
+          mbar_arrive_expect_tx(&full[s], na + nb);
+          bulk_load(dst, srca + (int64_t)ks * (P * kABytes), na, &full[s]);
+          bulk_load(dst + kAStage, srcb + (int64_t)ks * (P * kBBytes), nb, &full[s]);
+          issued = true;
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      if (*abort_flag && issued) {   // let the copies in flight land before the CTA exits
+        const uint64_t t0 = global_ns();
+        while (global_ns() - t0 < 200000ull) {
+        }
+      }
+    }
+  } else if (warp == kMmaWarp) {
+    if (lane == 0) {
+      const uint64_t desc0 = smem_desc32(smem_u32(ring));
+      uint32_t idesc[5];
+#pragma unroll
+      for (int c = 0; c < 5; ++c)   // FP32 accumulator, BF16 operands, both K-major, N >> 3, M >> 4
+        idesc[c] = (1u << 4) | (1u << 7) | (1u << 10) | (((uint32_t)(c * BN) >> 3) << 17) |
+                   ((uint32_t)(kTileM >> 4) << 24);
+      int s = 0;
+      uint32_t ph = 0, use = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++use) {
+        const uint32_t b = use % NB;
+        if (use >= NB) {
+          ok = wait_bounded(&tmem_empty[b], (use / NB - 1) & 1u, abort_flag, a.err, 7);
+          if (!ok) break;
+          tc_fence_after();
+        }
+        const uint32_t td = tmem + b * kSetCols;
+        for (int ks = 0; ks < nk; ks += SL) {
+          ok = wait_bounded(&full[s], ph, abort_flag, a.err, 2);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t ad = desc0 + (uint64_t)(((uint32_t)s * kStage) >> 4);
+          const uint64_t bd = ad + (uint64_t)(kAStage >> 4);
+#pragma unroll
+          for (int k = 0; k < SL; ++k) {
+            if (k > 0 && ks + k >= nk) break;
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+#pragma unroll
+              for (int t0 = 0; t0 < P - p; t0 += 4) {
+                const int cnt = P - p - t0 < 4 ? P - p - t0 : 4;
+                tc_mma<kKindBF16>(td + (uint32_t)((p + t0) * BN), ad + (uint64_t)((k * P + p) * (kABytes >> 4)),
+                                  bd + (uint64_t)((k * P + t0) * (kBBytes >> 4)), idesc[cnt],
+                                  (ks == 0 && k == 0 && p == 0) ? 0u : 1u);
+              }
+            }
+          }
+          tc_commit(&empty[s]);
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+        if (ok) tc_commit(&accum[b]);
+      }
+      if (!ok) {
+        tc_commit(drain);
+        wait_drain(drain, 0);
+      }
+    }
+  } else {
+    const int quarter = warp & 3, grp = warp >> 2;
+    uint32_t use = 0;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++use) {
+      const int64_t tr = t / a.tiles_c;
+      const int c = (int)(t - tr * a.tiles_c) * kTileM + quarter * 32 + lane;
+      const int64_t r0 = tr * BN + NC * grp;
+      const int ec = __ldg(a.cexp + c);   // padded to whole tiles, as rexp
+      // this warp's row exponents, in flight while the tile's MMAs run
+      const int re = __ldg(a.rexp + r0 + (lane < NC ? lane : 0));
+      const uint32_t b = use % NB;
+      const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + b * kSetCols + (uint32_t)(NC * grp);
+      bool have = wait_sleepy(&accum[b], (use / NB) & 1u, abort_flag, a.err, 5);
+      have = __all_sync(0xffffffffu, have);
+      if (!have) break;
+      tc_fence_after();
+      if constexpr (P == 8) {
+        // read the levels into integers, so that the next tile's MMAs start early ...
+        long long hi[16];
+        uint32_t lo[16];
+        read_levels(base, a.K > kTtmFastChain, hi, lo);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tmem_empty[b]);
+        // ... and round and store them meanwhile
+        double* y = static_cast<double*>(a.Y) + r0 * a.C + c;
+#pragma unroll
+        for (int k = 0; k < 16; ++k, y += a.C) {
+          const int64_t r = r0 + k;
+          const int er = __shfl_sync(0xffffffffu, re, k);
+          if (r >= a.J || c >= a.C) continue;
+          if (ec == kTtmBadExp) {
+            double acc = 0.0;
+            for (int i = 0; i < a.K; ++i)
+              acc = fma(__ldg(a.Tn + (int64_t)i * a.J + r), __ldg(a.U + (int64_t)i * a.C + c), acc);
+            *y = acc;
+          } else {
+            *y = round_levels(hi[k], lo[k], ec + er);
+          }
+        }
+      } else {
+        // four digits: the levels as an FP32 pair (TwoSum; levels 0 and 1 exact, 2 and
+        // 3 small); fewer: their FP32 sum, smallest first
+        float vh[NC], vl[P == 4 ? NC : 1];
+#pragma unroll
+        for (int h = 0; h < NC / 4; ++h) {
+          uint32_t v[P][4];
+          __syncwarp();
+#pragma unroll
+          for (int l = 0; l < P; ++l) tmem_ld4(base + (uint32_t)(l * BN + 4 * h), v[l]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            float sh = __uint_as_float(v[0][k]);
+            if constexpr (P == 4) {
+              float sl = 0.f;
+              df_add(sh, sl, __uint_as_float(v[1][k]));
+              df_add(sh, sl, __fadd_rn(__uint_as_float(v[2][k]), __uint_as_float(v[3][k])));
+              vl[4 * h + k] = sl;
+            } else if constexpr (P == 3) {
+              sh = __fadd_rn(sh, __fadd_rn(__uint_as_float(v[1][k]), __uint_as_float(v[2][k])));
+            } else {
+              sh = __fadd_rn(sh, __uint_as_float(v[1][k]));
+            }
+            vh[4 * h + k] = sh;
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tmem_empty[b]);
+        // times 2^(rexp - 14): the column's exponent is left to the contraction, so
+        // that the FP32 values stay in range
+        using YT = std::conditional_t<P == 4, float2, float>;
+        YT* y = static_cast<YT*>(a.Y) + r0 * a.C + c;
+#pragma unroll
+        for (int k = 0; k < NC; ++k, y += a.C) {
+          const int e = __shfl_sync(0xffffffffu, re, k) - 14;
+          if (r0 + k >= a.J || c >= a.C) continue;
+          const float sc = __int_as_float((127 + (e < -126 ? -126 : e)) << 23);
+          const float yh = ec == kTtmBadExp ? CUDART_NAN_F : vh[k] * sc;
+          if constexpr (P == 4)
+            *y = make_float2(yh, vl[k] * sc);
+          else
+            *y = yh;
+        }
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kTmemCols);
+  }
+}
+
+// ---- contraction with one more factor ------------------------------------------------
+// out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c], X of FP64 values, FP32
+// pairs or FP32 values.  A thread takes RB outputs (h, l) of V adjacent columns: one load
+// of U serves RB of X, and a load of V columns is 16 bytes (a warp's 512: at 128 bytes a
+// row the FP32 case read 2.7 to 3.6 TB/s).  Bound: X read once, or in FP64 the pipe's two
+// multiply-adds per clock and SM.
+//   FP64: fused multiply-adds in m order.
+//   Pairs: double-float arithmetic on the FP32 pipe (about 2^-44 per operation), U's entry
+//   split into a pair, the leading products error-free.
+//   FP32: chains of UN products in FP32, their sums into a pair.
+// cexp: the last contraction of an MTTKRP of fewer than eight digits applies the columns'
+// exponents (null otherwise).
+template <class XT, int V>
+struct alignas(sizeof(XT) * V) Cols {
+  XT v[V];
+};
+
+template <class XT, int RB, int V>
+__global__ void __launch_bounds__(256) contract_kernel(const XT* __restrict__ X, int64_t H, int Mm, int64_t L, int C,
+                                                       const double* __restrict__ U, int mchunk,
+                                                       const int* __restrict__ cexp, XT* __restrict__ out) {
+  using XV = Cols<XT, V>;
+  constexpr bool kF64 = std::is_same_v<XT, double>, kF32 = std::is_same_v<XT, float>;
+  constexpr int UN = RB * V >= 8 ? 2 : (RB * V >= 4 ? 4 : 8);   // terms loaded together
+  const int64_t HL = H * L, groups = (HL + RB - 1) / RB;
+  const int CV = C / V;
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= groups * CV) return;
+  const int64_t g = idx / CV;
+  const int c = (int)(idx - g * CV) * V;
+  const int mb = blockIdx.y * mchunk, me = mb + mchunk < Mm ? mb + mchunk : Mm;
+  const XT* x[RB];
+  using AT = std::conditional_t<kF64, double, float>;
+  AT ah[RB][V], al[kF64 ? 1 : RB][V];   // the sum, FP64 or an FP32 pair
+#pragma unroll
+  for (int q = 0; q < RB; ++q) {
+    const int64_t o = g * RB + q < HL ? g * RB + q : HL - 1;
+    const int64_t hh = o / L;
+    x[q] = X + ((hh * Mm + mb) * L + (o - hh * L)) * C + c;
+#pragma unroll
+    for (int w = 0; w < V; ++w) {
+      ah[q][w] = 0;
+      if constexpr (!kF64) al[q][w] = 0;
+    }
+  }
+  const int64_t step = L * C;
+  const double* u = U + (int64_t)mb * C + c;
+  auto load = [](const XT* p) {
+    XV r;
+    if constexpr (sizeof(XV) == 16) {
+      const uint4 t = __ldg(reinterpret_cast<const uint4*>(p));
+      memcpy(&r, &t, 16);
+    } else {
+#pragma unroll
+      for (int w = 0; w < V; ++w) r.v[w] = __ldg(p + w);
+    }
+    return r;
+  };
+  // N terms: N <= UN, all loaded first
+  auto terms = [&](auto nt) {
+    constexpr int N = decltype(nt)::value;
+    double uv[N][V];
+    XV xv[N][RB];
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      if constexpr (V % 2 == 0) {
+#pragma unroll
+        for (int w = 0; w < V; w += 2) {
+          const double2 t = __ldg(reinterpret_cast<const double2*>(u + (int64_t)e * C + w));
+          uv[e][w] = t.x;
+          uv[e][w + 1] = t.y;
+        }
+      } else {
+#pragma unroll
+        for (int w = 0; w < V; ++w) uv[e][w] = __ldg(u + (int64_t)e * C + w);
+      }
+#pragma unroll
+      for (int q = 0; q < RB; ++q) xv[e][q] = load(x[q] + e * step);
+    }
+    if constexpr (kF64) {
+#pragma unroll
+      for (int e = 0; e < N; ++e)
+#pragma unroll
+        for (int q = 0; q < RB; ++q)
+#pragma unroll
+          for (int w = 0; w < V; ++w) ah[q][w] = fma(xv[e][q].v[w], uv[e][w], ah[q][w]);
+    } else if constexpr (kF32) {
+#pragma unroll
+      for (int w = 0; w < V; ++w) {
+        float uf[N];
+#pragma unroll
+        for (int e = 0; e < N; ++e) uf[e] = (float)uv[e][w];
+#pragma unroll
+        for (int q = 0; q < RB; ++q) {
+          float p = __fmul_rn(xv[0][q].v[w], uf[0]);
+#pragma unroll
+          for (int e = 1; e < N; ++e) p = __fmaf_rn(xv[e][q].v[w], uf[e], p);
+          df_add(ah[q][w], al[q][w], p);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < N; ++e)
+#pragma unroll
+        for (int w = 0; w < V; ++w) {
+          float uh, ul;
+          split_f32_pair(uv[e][w], uh, ul);
+#pragma unroll
+          for (int q = 0; q < RB; ++q) {
+            const float2 xw = xv[e][q].v[w];
+            const float p = __fmul_rn(xw.x, uh);
+            const float r = __fmaf_rn(xw.y, uh, __fmaf_rn(xw.x, ul, __fmaf_rn(xw.x, uh, -p)));
+            df_add(ah[q][w], al[q][w], p);
+            al[q][w] = __fadd_rn(al[q][w], r);
+          }
+        }
+    }
+    u += (int64_t)N * C;
+#pragma unroll
+    for (int q = 0; q < RB; ++q) x[q] += N * step;
+  };
+  int m = mb;
+  for (; m + UN <= me; m += UN) terms(std::integral_constant<int, UN>{});
+  for (; m < me; ++m) terms(std::integral_constant<int, 1>{});
+  // 2^cexp in two factors: each in range where the product is
+  float s1[V], s2[V];
+  if constexpr (!kF64) {
+#pragma unroll
+    for (int w = 0; w < V; ++w) {
+      int e = cexp != nullptr ? __ldg(cexp + c + w) : 0;
+      e = e < -250 ? -250 : (e > 250 ? 250 : e);
+      s1[w] = __int_as_float((127 + e / 2) << 23);
+      s2[w] = __int_as_float((127 + e - e / 2) << 23);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < RB; ++q)
+    if (g * RB + q < HL) {
+      XT* o = out + ((int64_t)blockIdx.y * HL + g * RB + q) * C + c;
+#pragma unroll
+      for (int w = 0; w < V; ++w) {
+        if constexpr (kF64) {
+          o[w] = ah[q][w];
+        } else {
+          const float h = __fadd_rn(ah[q][w], al[q][w]);
+          if constexpr (kF32)
+            o[w] = h * s1[w] * s2[w];
+          else
+            o[w] = make_float2(h * s1[w] * s2[w], __fsub_rn(al[q][w], __fsub_rn(h, ah[q][w])) * s1[w] * s2[w]);
+        }
+      }
+    }
+}
+
+template <int P, int TILE>
+cudaError_t launch_slice(const double* X, int K, int64_t M, int64_t ld, const int* kexp, int sgn, unsigned char* img,
+                         int* expo, int* counter, cudaStream_t s) {
+  const int64_t Mpad = (M + TILE - 1) / TILE * TILE;
+  const int64_t blocks = Mpad / kSliceCols;
+  slice_f64_kernel<P, TILE><<<(unsigned)(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
+      X, K, M, ld, kexp, sgn, ttm_ksteps(K), Mpad, img, expo, counter);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* kexp, int* bad, cudaStream_t s) {
+  slice_exponent_kernel<<<(unsigned)I, 256, 0, s>>>(Tn, J, kexp, bad);
+  return cudaGetLastError();
+}
+
+// calls f with the number of digits as a compile-time constant
+namespace {
+template <class F>
+cudaError_t with_digits(int digits, F f) {
+  switch (digits) {
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    default: return f(std::integral_constant<int, 8>{});
+  }
+}
+}  // namespace
+
+cudaError_t launch_slice_tensor(int digits, const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt,
+                                int* rexp, cudaStream_t s) {
+  return with_digits(digits, [&](auto p) {
+    constexpr int P = decltype(p)::value;
+    return launch_slice<P, ttm_tile_r(P)>(Tn, I, J, J, kexp, -1, Bt, rexp, nullptr, s);
+  });
+}
+
+cudaError_t launch_slice_factor(int digits, const double* U, int I, int C, const int* kexp, unsigned char* At,
+                                int* cexp, int* counter, cudaStream_t s) {
+  return with_digits(digits, [&](auto p) {
+    return launch_slice<decltype(p)::value, kTileM>(U, I, C, C, kexp, +1, At, cexp, counter, s);
+  });
+}
+
+cudaError_t prepare_ttm(int digits) {
+  return with_digits(digits, [&](auto p) {
+    return cudaFuncSetAttribute(ttm_kernel<decltype(p)::value>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  });
+}
+
+cudaError_t launch_ttm(int digits, const TtmArgs& a, int num_sms, cudaStream_t s) {
+  const int64_t tiles = (int64_t)a.tiles_c * a.tiles_r;
+  const unsigned grid = (unsigned)(tiles < num_sms ? tiles : num_sms);
+  return with_digits(digits, [&](auto p) {
+    ttm_kernel<decltype(p)::value><<<grid, kThreads, kSmem, s>>>(a);
+    return cudaGetLastError();
+  });
+}
+
+// Shape of a contraction: V columns per 16-byte load where C allows, four rows of outputs
+// per thread where enough threads remain, and m split into about 1280 threads per SM, at
+// least eight terms each (400x400x400, FP32 pairs of 400 columns: 94 us, with 512 threads
+// per SM 135; FP32 values of 800 columns: 109 us, two columns' width 143 to 188).
+namespace {
+constexpr int64_t kContractThreads = 152 * 1280;
+
+int contract_vec(int digits, int C) {
+  if (digits < 4) return C % 4 == 0 ? 4 : 1;
+  return C % 2 == 0 ? 2 : 1;
+}
+
+int contract_rb(int64_t HL, int Mm, int C, int V) {
+  return HL >= 4 && (HL + 3) / 4 * (C / V) * ((Mm + 7) / 8) >= kContractThreads / 2 ? 4 : 1;
+}
+
+template <class XT, int V>
+cudaError_t launch_contract_v(dim3 grid, int RB, const void* X, int64_t H, int Mm, int64_t L, int C, const double* U,
+                              int chunk, const int* cexp, void* out, cudaStream_t s) {
+  if (RB == 4)
+    contract_kernel<XT, 4, V><<<grid, 256, 0, s>>>(static_cast<const XT*>(X), H, Mm, L, C, U, chunk, cexp,
+                                                   static_cast<XT*>(out));
+  else
+    contract_kernel<XT, 1, V><<<grid, 256, 0, s>>>(static_cast<const XT*>(X), H, Mm, L, C, U, chunk, cexp,
+                                                   static_cast<XT*>(out));
+  return cudaGetLastError();
+}
+}  // namespace
+
+int contract_splits(int digits, int64_t HL, int Mm, int C) {
+  const int V = contract_vec(digits, C), RB = contract_rb(HL, Mm, C, V);
+  const int64_t threads = (HL + RB - 1) / RB * (C / V);
+  int64_t S = (kContractThreads + threads - 1) / threads;
+  if (S > (Mm + 7) / 8) S = (Mm + 7) / 8;
+  if (S < 1) S = 1;
+  const int chunk = (int)((Mm + S - 1) / S);
+  return (Mm + chunk - 1) / chunk;
+}
+
+cudaError_t launch_contract(int digits, const void* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
+                            const int* cexp, void* out, cudaStream_t s) {
+  const int64_t HL = H * L;
+  const int chunk = (Mm + S - 1) / S;
+  const int V = contract_vec(digits, C), RB = contract_rb(HL, Mm, C, V);
+  const dim3 grid((unsigned)(((HL + RB - 1) / RB * (C / V) + 255) / 256), (unsigned)S);
+  auto go = [&](auto f) { return f(grid, RB, X, H, Mm, L, C, U, chunk, cexp, out, s); };
+  if (digits == 8) return V == 2 ? go(launch_contract_v<double, 2>) : go(launch_contract_v<double, 1>);
+  if (digits == 4) return V == 2 ? go(launch_contract_v<float2, 2>) : go(launch_contract_v<float2, 1>);
+  return V == 4 ? go(launch_contract_v<float, 4>) : go(launch_contract_v<float, 1>);
+}
+
+}  // namespace jk
