@@ -764,11 +764,18 @@ cudaError_t launch_ttm(int digits, const TtmArgs& a, int num_sms, cudaStream_t s
 }
 
 // Shape of a contraction: V columns per 16-byte load where C allows, four rows of outputs
-// per thread where enough threads remain, and m split into about 1280 threads per SM, at
-// least eight terms each (400x400x400, FP32 pairs of 400 columns: 94 us, with 512 threads
-// per SM 135; FP32 values of 800 columns: 109 us, two columns' width 143 to 188).
+// per thread where enough threads remain, and m split to fill the SMs, at least eight
+// terms each.  A large X wants about 1280 threads per SM in flight (400x400x400, FP32
+// pairs of 400 columns: 94 us, with 512 threads per SM 135; FP32 values of 800 columns:
+// 109 us, one column per load 143 to 188); a small one 512, as every split lengthens
+// the sums of the update that follows (20 uneven 3xTF32 problems: 15.6 against 16.0 ms).
 namespace {
-constexpr int64_t kContractThreads = 152 * 1280;
+constexpr int64_t kContractSms = 152, kLargeX = 64ll << 20;
+
+int64_t contract_threads(int digits, int64_t HL, int Mm, int C) {
+  const int64_t bytes = HL * Mm * C * (digits < 4 ? 4 : 8);
+  return kContractSms * (bytes > kLargeX ? 1280 : 512);
+}
 
 int contract_vec(int digits, int C) {
   if (digits < 4) return C % 4 == 0 ? 4 : 1;
@@ -776,7 +783,7 @@ int contract_vec(int digits, int C) {
 }
 
 int contract_rb(int64_t HL, int Mm, int C, int V) {
-  return HL >= 4 && (HL + 3) / 4 * (C / V) * ((Mm + 7) / 8) >= kContractThreads / 2 ? 4 : 1;
+  return HL >= 4 && (HL + 3) / 4 * (C / V) * ((Mm + 7) / 8) >= kContractSms * 512 ? 4 : 1;
 }
 
 template <class XT, int V>
@@ -795,7 +802,7 @@ cudaError_t launch_contract_v(dim3 grid, int RB, const void* X, int64_t H, int M
 int contract_splits(int digits, int64_t HL, int Mm, int C) {
   const int V = contract_vec(digits, C), RB = contract_rb(HL, Mm, C, V);
   const int64_t threads = (HL + RB - 1) / RB * (C / V);
-  int64_t S = (kContractThreads + threads - 1) / threads;
+  int64_t S = (contract_threads(digits, HL, Mm, C) + threads - 1) / threads;
   if (S > (Mm + 7) / 8) S = (Mm + 7) / 8;
   if (S < 1) S = 1;
   const int chunk = (int)((Mm + S - 1) / S);
