@@ -763,7 +763,7 @@ jkcals_status enqueue_sweep(jkcals_ctx* h) {
       // fixed-order split-K reduction into FP64 Mbar_n, then the two-phase update
       JK_TRY(reduce_into(h, n, h->mbuf));
       UpdateArgs a = update_args(h, n, h->mbuf, kPartF64, 1);
-      JK_CUDA(h, launch_update(a, h->stream));
+      JK_CUDA(h, launch_update(a, h->Rmax, h->stream));
       kernels += 3;
     }
     ttm.updated(n);
@@ -2210,7 +2210,7 @@ jkcals_status capture_grouped(jkcals_batch_ctx* b, cudaGraph_t* graph) {
       e = part_kind(h) == kPartF32x2
               ? launch_reduce_partials_f32x2(static_cast<float2*>(h->part), mode_splits(h, n), cnt, h->mbuf, s2)
               : launch_reduce_partials_f32(static_cast<float*>(h->part), mode_splits(h, n), cnt, h->mbuf, s2);
-      if (e == cudaSuccess) e = launch_update(update_args(h, n, h->mbuf, kPartF64, 1), s2);
+      if (e == cudaSuccess) e = launch_update(update_args(h, n, h->mbuf, kPartF64, 1), h->Rmax, s2);
       if (e != cudaSuccess) st = fail(JKCALS_ERR_CUDA, std::string("batched two-phase update: ") + cudaGetErrorString(e));
     }
     for (size_t k = 0; k < nside && st == JKCALS_OK; ++k) {

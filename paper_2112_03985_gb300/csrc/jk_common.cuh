@@ -424,7 +424,8 @@ struct UpdateArgs {
   float* cmax;                      // NULL or C column maxima of UT, refreshed
   float* UT_lo;                     // NULL or the low parts fl32(U - UT), refreshed
 };
-cudaError_t launch_update(const UpdateArgs& a, cudaStream_t s);
+// two-phase update; Rmax: the largest rank of the blocks
+cudaError_t launch_update(const UpdateArgs& a, int Rmax, cudaStream_t s);
 // fused one-CTA-per-block update (jk_update_fused.cu); part = reduced Mbar_n (FP64)
 size_t update_fused_smem(int64_t I, int Rmax);
 cudaError_t prepare_update_fused(size_t smem, int Rmax, bool uniform_rank);

@@ -20,13 +20,14 @@
 // of the S partials and one write + one read-modify-write of Ubar^(n).
 #include <math.h>
 
+#include "jk_chol.cuh"
 #include "jk_common.cuh"
 
 namespace jk {
 namespace {
 
 constexpr int NTA = 128;  // threads of phase A = max rows per chunk
-constexpr int NTB = 128;
+constexpr int NTB = 512;
 constexpr int GP = kMaxRank * kMaxRank;  // stride of one partial Gram
 
 __device__ __forceinline__ bool is_left_out(const BlockMeta& bm, int g, int64_t i) {
@@ -48,9 +49,11 @@ __device__ __forceinline__ double load_part<float2>(const float2* p) {
   return (double)v.x + (double)v.y;
 }
 
-constexpr int kPartBatch = 8;   // split-K partials loaded together per element
-
-template <typename PT>
+// RMAX: the rank class (8, 16 or 32) that the row registers and unrolled substitutions
+// are sized by.  One class of 32 for every rank kept the rows behind guards and one load
+// at a time, and one thread summed a Gram pair over the chunk's rows: 65 us for 40
+// blocks of 400 rows of rank 10 on GB300, 27 us now.
+template <typename PT, int RMAX>
 __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
   const int g = blockIdx.x, rc = blockIdx.y;
   const int tid = threadIdx.x;
@@ -58,9 +61,9 @@ __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
   const int R = a.bm.R[g], off = a.bm.off[g];
   const int go = a.bm.gram_off[g];
 
-  __shared__ double Hs[kMaxRank][kMaxRank + 1];
-  __shared__ double invd[kMaxRank];   // 1 / L_jj
-  __shared__ double X[NTA * kMaxRank];
+  __shared__ double Hs[RMAX][RMAX + 1];
+  __shared__ double invd[RMAX];   // 1 / L_jj
+  __shared__ double X[NTA * RMAX];
   __shared__ double red[NTA];
   __shared__ int spd_ok;
 
@@ -74,35 +77,7 @@ __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
   if (tid == 0) spd_ok = 1;
   __syncthreads();
 
-  // Cholesky H = L L^T in place (lower triangle), column by column, one warp.
-  if (tid < 32) {
-    const int lane = tid;
-    bool ok = true;
-    for (int j = 0; j < R; ++j) {
-      if (lane == 0) {
-        double d = Hs[j][j];
-        for (int k = 0; k < j; ++k) d -= Hs[j][k] * Hs[j][k];
-        if (!(d > 0.0) || !isfinite(d)) {
-          spd_ok = 0;
-          d = 1.0;
-        }
-        // 1 / L_jj from the reciprocal square root: the column below and both
-        // substitutions multiply by it (no FP64 division on the serial paths)
-        const double rs = rsqrt(d);
-        Hs[j][j] = d * rs;
-        invd[j] = rs;
-      }
-      __syncwarp();
-      const int i = j + 1 + lane;
-      if (i < R) {
-        double v = Hs[i][j];
-        for (int k = 0; k < j; ++k) v -= Hs[i][k] * Hs[j][k];
-        Hs[i][j] = v * invd[j];
-      }
-      __syncwarp();
-    }
-    (void)ok;
-  }
+  if (tid < 32) warp_cholesky(Hs, invd, R, tid, &spd_ok);
   __syncthreads();
   if (!spd_ok) {
     if (rc == 0 && tid == 0) atomicOr(&a.status[g], (int)JKCALS_BLOCK_NOT_SPD);
@@ -118,32 +93,35 @@ __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
   const int64_t IC = a.I * (int64_t)a.C;
   double fit = 0.0;
   if (active) {
-    double m[kMaxRank], x[kMaxRank];
+    double m[RMAX], x[RMAX];
+    // the S partials in split order: a batch of splits of every element loaded
+    // together (all in flight), then added
+    constexpr int kBatch = RMAX <= 8 ? 4 : (RMAX <= 16 ? 2 : 1);
+    const PT* p = part + row * a.C + off;
 #pragma unroll
-    for (int r = 0; r < kMaxRank; ++r) {
-      double v = 0.0;
-      if (r < R) {
-        // the S partials in split order, loaded kPartBatch at a time (all in flight)
-        const PT* p = part + row * a.C + off + r;
-        for (int s0 = 0; s0 < a.S; s0 += kPartBatch) {
-          double t[kPartBatch];
+    for (int r = 0; r < RMAX; ++r) m[r] = 0.0;
+    for (int s0 = 0; s0 < a.S; s0 += kBatch) {
+      double t[kBatch][RMAX];
 #pragma unroll
-          for (int u = 0; u < kPartBatch; ++u) t[u] = s0 + u < a.S ? load_part(p + (int64_t)(s0 + u) * IC) : 0.0;
+      for (int u = 0; u < kBatch; ++u)
 #pragma unroll
-          for (int u = 0; u < kPartBatch; ++u)
-            if (s0 + u < a.S) v += t[u];
+        for (int r = 0; r < RMAX; ++r)
+          t[u][r] = s0 + u < a.S && r < R ? load_part(p + (int64_t)(s0 + u) * IC + r) : 0.0;
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        if (s0 + u < a.S) {
+#pragma unroll
+          for (int r = 0; r < RMAX; ++r) m[r] += t[u][r];
         }
-      }
-      m[r] = v;
     }
     const bool zero = (a.n == a.n_hat) && is_left_out(a.bm, g, row);
     if (zero) {
 #pragma unroll
-      for (int r = 0; r < kMaxRank; ++r) x[r] = 0.0;
+      for (int r = 0; r < RMAX; ++r) x[r] = 0.0;
     } else {
       // forward: L y = m
 #pragma unroll
-      for (int r = 0; r < kMaxRank; ++r) {
+      for (int r = 0; r < RMAX; ++r) {
         if (r < R) {
           double v = m[r];
 #pragma unroll
@@ -155,11 +133,11 @@ __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
       }
       // backward: L^T u = y
 #pragma unroll
-      for (int r = kMaxRank - 1; r >= 0; --r) {
+      for (int r = RMAX - 1; r >= 0; --r) {
         if (r < R) {
           double v = x[r];
 #pragma unroll
-          for (int k = r + 1; k < kMaxRank; ++k)
+          for (int k = r + 1; k < RMAX; ++k)
             if (k < R) v -= Hs[k][r] * x[k];
           x[r] = v * invd[r];
         }
@@ -167,7 +145,7 @@ __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
     }
     double* urow = a.U + row * a.C + off;
 #pragma unroll
-    for (int r = 0; r < kMaxRank; ++r) {
+    for (int r = 0; r < RMAX; ++r) {
       if (r < R) {
         urow[r] = x[r];
         X[tid * R + r] = x[r];
@@ -177,15 +155,30 @@ __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
   }
   __syncthreads();
 
-  // Partial Gram (upper triangle) over this chunk's rows.
+  // Partial Gram (upper triangle) over this chunk's rows: thread (p, q) sums pair p
+  // over rows q, q + nq, ..., the partial sums are added in order.
   const int nrows = (int)(r1 > r0 ? r1 - r0 : 0);
   double* gp = a.gpart + ((int64_t)g * a.RC + rc) * GP;
-  for (int p = tid; p < R * R; p += NTA) {
-    const int r = p / R, c = p % R;
-    if (c < r) continue;
+  const int np = R * (R + 1) / 2;
+  const int nq = NTA / np > 0 ? NTA / np : 1;
+  for (int p0 = 0; p0 < np; p0 += NTA) {
+    const int q = tid / np, p = p0 + tid - q * np;
+    int r = 0, c = p < np ? p : 0;
+    while (c >= R - r) {
+      c -= R - r;
+      ++r;
+    }
+    c += r;
     double acc = 0.0;
-    for (int t = 0; t < nrows; ++t) acc = fma(X[t * R + r], X[t * R + c], acc);
-    gp[r * kMaxRank + c] = acc;
+    if (q < nq && p < np)
+      for (int t = q; t < nrows; t += nq) acc = fma(X[t * R + r], X[t * R + c], acc);
+    red[tid] = acc;
+    __syncthreads();
+    if (q == 0 && p < np) {
+      for (int t = 1; t < nq; ++t) acc += red[t * np + p];
+      gp[r * kMaxRank + c] = acc;
+    }
+    __syncthreads();
   }
   if (a.n == a.N - 1) {
     red[tid] = fit;
@@ -224,20 +217,22 @@ __global__ void __launch_bounds__(NTB) update_phase_b(UpdateArgs a) {
   }
   __syncthreads();
   if (a.normalise && a.n < a.N - 1) {
+    // by the reciprocal norms, as the one-CTA updates do: a division per entry took
+    // most of this kernel (40 blocks of 400 rows of rank 10: 32 us, now 12 us)
     if (tid < R) {
       const double v = sqrt(G[tid][tid]);
-      nrm[tid] = (v > 0.0) ? v : 1.0;
+      nrm[tid] = (v > 0.0) ? 1.0 / v : 1.0;
     }
     __syncthreads();
     for (int p = tid; p < R * R; p += NTB) {
       const int r = p / R, c = p % R;
-      G[r][c] = G[r][c] / (nrm[r] * nrm[c]);
+      G[r][c] = G[r][c] * nrm[r] * nrm[c];
     }
     for (int64_t t = tid; t < a.I * R; t += NTB) {
       const int64_t i = t / R;
       const int r = (int)(t - i * R);
       double* u = a.U + i * a.C + off + r;
-      *u = *u / nrm[r];
+      *u = *u * nrm[r];
     }
     __syncthreads();
   }
@@ -383,15 +378,24 @@ __global__ void sum_blocks_kernel(const double* eg, int K, double* out) {
 
 }  // namespace
 
-cudaError_t launch_update(const UpdateArgs& a, cudaStream_t s) {
-  dim3 ga((unsigned)a.K, (unsigned)a.RC);
-  if (a.part_kind == kPartF32)
-    update_phase_a<float><<<ga, NTA, 0, s>>>(a);
-  else if (a.part_kind == kPartF32x2)
-    update_phase_a<float2><<<ga, NTA, 0, s>>>(a);
+namespace {
+template <typename PT>
+cudaError_t launch_phase_a(const UpdateArgs& a, int Rmax, cudaStream_t s) {
+  const dim3 ga((unsigned)a.K, (unsigned)a.RC);
+  if (Rmax <= 8)
+    update_phase_a<PT, 8><<<ga, NTA, 0, s>>>(a);
+  else if (Rmax <= 16)
+    update_phase_a<PT, 16><<<ga, NTA, 0, s>>>(a);
   else
-    update_phase_a<double><<<ga, NTA, 0, s>>>(a);
-  cudaError_t e = cudaGetLastError();
+    update_phase_a<PT, kMaxRank><<<ga, NTA, 0, s>>>(a);
+  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_update(const UpdateArgs& a, int Rmax, cudaStream_t s) {
+  const cudaError_t e = a.part_kind == kPartF32     ? launch_phase_a<float>(a, Rmax, s)
+                        : a.part_kind == kPartF32x2 ? launch_phase_a<float2>(a, Rmax, s)
+                                                    : launch_phase_a<double>(a, Rmax, s);
   if (e != cudaSuccess) return e;
   update_phase_b<<<a.K, NTB, 0, s>>>(a);
   return cudaGetLastError();

@@ -22,6 +22,7 @@
 
 #include <string>
 
+#include "jk_chol.cuh"
 #include "jk_common.cuh"
 
 namespace jk {
@@ -131,30 +132,12 @@ __device__ __forceinline__ void update_fused_body(const UpdateArgs& a, int g, do
       Hc[p] = h;
     }
     __syncwarp();
-    for (int j = 0; j < R; ++j) {
-      if (lane == 0) {
-        double d = L[j][j];
-        for (int k = 0; k < j; ++k) d -= L[j][k] * L[j][k];
-        if (!(d > 0.0) || !isfinite(d)) {
-          spd_ok = 0;
-          d = 1.0;
-        }
-        // 1 / L_jj straight from the reciprocal square root (the solves use
-        // only the reciprocals; one FP64 sequence instead of a root and a
-        // division on the serial path)
-        const double rs = rsqrt(d);
-        L[j][j] = d * rs;
-        invd[j] = rs;
-      }
-      __syncwarp();
-      const int i = j + 1 + lane;
-      if (i < R) {
-        double v = L[i][j];
-        for (int k = 0; k < j; ++k) v -= L[i][k] * L[j][k];
-        L[i][j] = v * invd[j];
-      }
-      __syncwarp();
-    }
+    if constexpr (FIXED)
+      warp_cholesky_left(L, invd, R, lane, &spd_ok);
+    else if constexpr (RMAX == 16)
+      warp_cholesky_call(L, invd, R, lane, &spd_ok);
+    else
+      warp_cholesky(L, invd, R, lane, &spd_ok);
   } else {
     // warps 1.. : this block's rows of Mbar_n into X, each element the sum of its
     // S partials in split order (a few rows per thread, each split's loads
@@ -484,27 +467,7 @@ __device__ __forceinline__ void update_wide_body(const UpdateArgs& a, int g, dou
       Hc[p] = h;
     }
     __syncwarp();
-    for (int j = 0; j < R; ++j) {
-      if (lane == 0) {
-        double d = L[j][j];
-        for (int k = 0; k < j; ++k) d -= L[j][k] * L[j][k];
-        if (!(d > 0.0) || !isfinite(d)) {
-          spd_ok = 0;
-          d = 1.0;
-        }
-        const double rs = rsqrt(d);
-        L[j][j] = d * rs;
-        invd[j] = rs;
-      }
-      __syncwarp();
-      const int i = j + 1 + lane;
-      if (i < R) {
-        double v = L[i][j];
-        for (int k = 0; k < j; ++k) v -= L[i][k] * L[j][k];
-        L[i][j] = v * invd[j];
-      }
-      __syncwarp();
-    }
+    warp_cholesky_left(L, invd, R, lane, &spd_ok);
     if constexpr (DF) {
       for (int p = lane; p < R * R; p += 32) {
         const int r = p / R, k = p % R;
@@ -921,7 +884,7 @@ cudaError_t run_wide(const UpdateArgs* a, size_t smem, cudaStream_t s, bool prep
 }
 
 // Instances: exact ranks 1..8 when all blocks share one rank, otherwise the
-// rank classes 8, 16, 32 with per-rank guards.
+// rank classes 8, 12, 16, 32 with per-rank guards.
 template <int RM, bool F>
 cudaError_t run_fused(const UpdateArgs* a, size_t smem, cudaStream_t s, bool prepare) {
   if (prepare) {
@@ -953,6 +916,7 @@ static cudaError_t dispatch_fused(const UpdateArgs* a, size_t smem, int Rmax, bo
     }
   }
   if (Rmax <= 8) return run_fused<8, false>(a, smem, s, prepare);
+  if (Rmax <= 12) return run_fused<12, false>(a, smem, s, prepare);
   if (Rmax <= 16) return run_fused<16, false>(a, smem, s, prepare);
   return run_fused<32, false>(a, smem, s, prepare);
 }
@@ -1011,6 +975,8 @@ cudaError_t dispatch_grouped(bool prepare, const UpdateArgs* args, const int* fi
     }
   }
   if (Rmax <= 8) return run_grouped(update_fused_grouped_kernel<8, false>, prepare, NT, args, first, nprob, total, smem, s);
+  if (Rmax <= 12)
+    return run_grouped(update_fused_grouped_kernel<12, false>, prepare, NT, args, first, nprob, total, smem, s);
   if (Rmax <= 16)
     return run_grouped(update_fused_grouped_kernel<16, false>, prepare, NT, args, first, nprob, total, smem, s);
   return run_grouped(update_fused_grouped_kernel<32, false>, prepare, NT, args, first, nprob, total, smem, s);
