@@ -91,6 +91,48 @@ cudaMemPool_t library_pool(int device) {
   return pool;
 }
 
+// Error words of the bounded waits in mapped host memory: a kernel writes one only
+// when a wait expires, and the host reads it after the stream's synchronisation,
+// without a copy from the device (about 10 us per call).  One page per process, one
+// word per handle, returned at destroy; a handle beyond them uses device memory.
+struct ErrorWords {
+  std::mutex mu;
+  int* page = nullptr;
+  bool tried = false;
+  std::vector<int*> free_words;
+};
+
+ErrorWords& error_words() {
+  static ErrorWords* w = new ErrorWords();   // lives until exit: handles may outlast statics
+  return *w;
+}
+
+int* take_error_word() {
+  ErrorWords& w = error_words();
+  std::lock_guard<std::mutex> lock(w.mu);
+  if (!w.tried) {
+    w.tried = true;
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, 4096, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) {
+      w.page = static_cast<int*>(p);
+      for (int k = 1023; k >= 0; --k) w.free_words.push_back(w.page + k);
+    } else {
+      cudaGetLastError();
+    }
+  }
+  if (w.free_words.empty()) return nullptr;
+  int* p = w.free_words.back();
+  w.free_words.pop_back();
+  *p = 0;
+  return p;
+}
+
+void give_error_word(int* p) {
+  ErrorWords& w = error_words();
+  std::lock_guard<std::mutex> lock(w.mu);
+  w.free_words.push_back(p);
+}
+
 jkcals_status dalloc(jkcals_ctx* h, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
@@ -137,6 +179,17 @@ bool is_host_pointer(const void* p) {
     return true;
   }
   return attr.type == cudaMemoryTypeHost || attr.type == cudaMemoryTypeUnregistered;
+}
+
+// Plain device memory of the handle's device, aligned for double.
+bool writable_by_kernels(const jkcals_ctx* h, const void* p) {
+  cudaPointerAttributes attr{};
+  if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return attr.type == cudaMemoryTypeDevice && attr.device == h->device &&
+         reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0;
 }
 
 BlockMeta block_meta(const jkcals_ctx* h) {
@@ -836,18 +889,43 @@ jkcals_status copy_out(jkcals_ctx* h, void* dst, const void* src, size_t bytes) 
   return JKCALS_OK;
 }
 
-// Reads the tensor-core kernel's error word (set when a bounded wait expired).
-jkcals_status check_device_error(jkcals_ctx* h) {
+// The handle's error word (h->d_err, written by the tensor-core kernels).
+jkcals_status create_error_word(jkcals_ctx* h) {
+  if (h->d_err != nullptr) return JKCALS_OK;
+  h->err_host = take_error_word();
+  if (h->err_host != nullptr) {
+    void* d = nullptr;
+    if (cudaHostGetDevicePointer(&d, h->err_host, 0) == cudaSuccess) {
+      h->d_err = static_cast<int*>(d);
+      return JKCALS_OK;
+    }
+    cudaGetLastError();
+    give_error_word(h->err_host);
+    h->err_host = nullptr;
+  }
+  JK_TRY(dalloc_t(h, &h->d_err, 1));
+  JK_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
+  return JKCALS_OK;
+}
+
+// Waits for the stream (unless the caller just has) and reads the error word, set when a
+// bounded wait expired.
+jkcals_status check_device_error(jkcals_ctx* h, bool synced = false) {
   if (h->d_err == nullptr || !(h->tc || h->ttm.ran)) return JKCALS_OK;   // no bounded wait ran
   h->ttm.ran = false;
   int err = 0;
-  JK_CUDA(h, cudaMemcpyAsync(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  JK_CUDA(h, cudaStreamSynchronize(h->stream));
-  if (err != 0) {
-    JK_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
+  if (h->err_host != nullptr) {
+    if (!synced) JK_CUDA(h, cudaStreamSynchronize(h->stream));
+    err = *static_cast<volatile int*>(h->err_host);
+    if (err != 0) *h->err_host = 0;
+  } else {
+    JK_CUDA(h, cudaMemcpyAsync(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    JK_CUDA(h, cudaStreamSynchronize(h->stream));
+    if (err != 0) JK_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
+  }
+  if (err != 0)
     return fail(JKCALS_ERR_TIMEOUT, "a bounded wait in the tensor-core MTTKRP expired (code " +
                                         std::to_string(err) + "); results of that call are invalid");
-  }
   return JKCALS_OK;
 }
 
@@ -963,6 +1041,7 @@ void destroy_impl(jkcals_ctx* h) {
   }
   h->allocations.clear();
   if (h->pool && h->stream) cudaStreamSynchronize(h->stream);
+  if (h->err_host) give_error_word(h->err_host);
   if (h->stream && h->owns_stream) cudaStreamDestroy(h->stream);
   cudaSetDevice(cur);
   delete h;
@@ -1055,10 +1134,7 @@ jkcals_status create_ttm_workspace(jkcals_ctx* h) {
     if (y > 0) JK_TRY(dalloc(h, &t.Y, 8 * y));
     if (z > 0) JK_TRY(dalloc(h, &t.Z, 8 * z));
     for (int k = 0; k < 2 && w > 0; ++k) JK_TRY(dalloc(h, &t.W[k], 8 * w));
-    if (h->d_err == nullptr) {
-      JK_TRY(dalloc_t(h, &h->d_err, 1));
-      JK_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream));
-    }
+    JK_TRY(create_error_word(h));
     JK_CUDA(h, prepare_ttm(t.digits));
     return JKCALS_OK;
   };
@@ -1194,8 +1270,7 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
     size_t smem = 0;
     for (int n = 0; n < N; ++n) smem = std::max(smem, tc::tc_smem_bytes(h->tcplan[n]));
     JK_CUDA(h, tc::prepare_mttkrp_tc(h->opt.precision, smem));
-    JK_TRY(dalloc_t(h, &h->d_err, 1));
-    JK_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
+    JK_TRY(create_error_word(h));
   }
 
   // factors and Grams
@@ -1427,17 +1502,21 @@ jkcals_status jkcals_mttkrp(jkcals_t h, int mode, double* M_out) {
   if (mode < 0 || mode >= h->N) return fail(JKCALS_ERR_ARG, "mode out of range");
   if (M_out == nullptr) return fail(JKCALS_ERR_ARG, "M_out is NULL");
   JK_TRY(enqueue_mttkrp(h, mode, h->U, h->UT, h->UTlo, h->cmax));
-  const int64_t cnt = h->dims[mode] * (int64_t)h->C;
-  JK_TRY(reduce_into(h, mode, h->mbuf));
-  JK_TRY(copy_out(h, M_out, h->mbuf, sizeof(double) * cnt));
+  // memory of the handle's own device takes the sums directly, anything else a copy
+  if (writable_by_kernels(h, M_out)) {
+    JK_TRY(reduce_into(h, mode, M_out));
+  } else {
+    JK_TRY(reduce_into(h, mode, h->mbuf));
+    JK_TRY(copy_out(h, M_out, h->mbuf, sizeof(double) * h->dims[mode] * (int64_t)h->C));
+  }
   return check_device_error(h);
 }
 
 static jkcals_status any_not_spd(jkcals_ctx* h) {
-  JK_TRY(check_device_error(h));
   std::vector<int32_t> st(h->K);
   JK_CUDA(h, cudaMemcpyAsync(st.data(), h->d_status, sizeof(int32_t) * h->K, cudaMemcpyDeviceToHost, h->stream));
   JK_CUDA(h, cudaStreamSynchronize(h->stream));
+  JK_TRY(check_device_error(h, true));
   for (int32_t v : st)
     if (v & JKCALS_BLOCK_NOT_SPD) return fail(JKCALS_ERR_NOT_SPD, "a submodel met a non-SPD Hadamard-of-Grams matrix");
   return JKCALS_OK;

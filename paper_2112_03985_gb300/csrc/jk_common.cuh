@@ -196,7 +196,8 @@ struct jkcals_ctx {
   float* cmax[jk::kMaxModes] = {nullptr};    // column maxima of UT (exact-chain grid)
   float* gcmax[jk::kMaxModes] = {nullptr};
   int* rowexp[jk::kMaxModes] = {nullptr};    // row exponents of T_(n) (exact-chain grid)
-  int* d_err = nullptr;                      // bounded-wait expiry code of the TC kernel
+  int* d_err = nullptr;                      // bounded-wait expiry code of the tensor-core kernels
+  int* err_host = nullptr;                   // the same word where it is in mapped host memory
   std::vector<int32_t> run_block_sweeps;     // sweeps each block ran in the latest jkcals_run
 
   // compaction of converged blocks inside jkcals_run: while compacted, the
