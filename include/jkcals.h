@@ -58,7 +58,10 @@ typedef enum {
 /* Arithmetic of the concurrent MTTKRP (Alg. 3 MTTKRP line).  The Gram,
  * Cholesky, solve, normalisation and error kernels are FP64 in every form.  */
 typedef enum {
-  JKCALS_FP64 = 0,        /* FP64 products and sums (CUDA cores)                       */
+  JKCALS_FP64 = 0,        /* FP64 accuracy: products and sums on the CUDA cores, or, where
+                             cheaper, tensor-times-matrix products shared by several modes
+                             whose operands are cut into eight 7-bit BF16 digits and summed
+                             exactly on the tensor cores, rounded to FP64 once           */
   JKCALS_TF32 = 1,        /* tcgen05 kind::tf32, FP32 accumulation in TMEM             */
   JKCALS_3XTF32 = 2,      /* hi*hi + hi*lo + lo*hi TF32 products, FP32 accumulation    */
   JKCALS_BF16 = 3,        /* tcgen05 kind::f16 with BF16 operands, FP32 accumulation   */
@@ -89,9 +92,11 @@ typedef struct {
   int normalise;        /* 1 (default): after updating mode n < N-1, scale each column of
                            every block to unit 2-norm (a zero column is left as is)       */
   int use_graph;        /* 1 (default): replay sweeps from a captured CUDA graph          */
-  int splits;           /* 0 (default) = automatic split-K factor of the MTTKRP, else fixed */
+  int splits;           /* 0 (default) = automatic split-K factor of the MTTKRP, else fixed
+                           (FP64: then always the CUDA-core kernel)                       */
   int64_t max_device_bytes; /* 0 (default) = no cap; > 0: allocations beyond this many bytes
-                               fail with JKCALS_ERR_OOM (lets callers bound device memory) */
+                               fail with JKCALS_ERR_OOM (lets callers bound device memory;
+                               FP64: then always the CUDA-core kernel) */
   int kernel_timing;    /* 1: record CUDA events around every MTTKRP launch of a sweep
                            (read with jkcals_kernel_times); 0 (default): off            */
   int update_mode;      /* per-block update kernels: 0 (default) automatic, 1 one CTA per
@@ -237,7 +242,8 @@ jkcals_status jkcals_jackknife_se(jkcals_t h, int ref_block, const double* const
 /*
  * jkcals_mode_plan -- how one mode's concurrent MTTKRP (Alg. 3 MTTKRP line) runs.
  *  mode          0 <= mode < N, else JKCALS_ERR_ARG
- *  kernel        receives 0 (FP64 on the CUDA cores), 1 (tensor cores, the Khatri-Rao
+ *  kernel        receives 0 (FP64; the plan reported is the CUDA-core kernel's also
+ *                where sweeps go through shared products), 1 (tensor cores, the Khatri-Rao
  *                tile built in shared memory), 2 (exact-chain two-step form: one GEMM
  *                against the sliced rows of mode fastest_mode per index of the remaining
  *                modes, scaled by their factor entries in the epilogue)

@@ -462,61 +462,30 @@ struct TtmState {
   }
 };
 
-// Digits per operand of a form's products: at least the operand bits of its own
-// kernel, counted from the largest entry of a contraction vector (58, 30, 23 and 16
-// fractional bits for 8, 4, 3 and 2 digits).
-int ttm_digits(int precision) {
-  switch (precision) {
-    case JKCALS_FP64: return 8;
-    case JKCALS_EXACT_BF16: return 4;
-    case JKCALS_BF16: return 2;
-    default: return 3;   // TF32, 3xTF32, split BF16
-  }
-}
-
 // Estimated seconds of each step, from measured rates.
-// The product: waves of tiles over the SMs, `step` cycles per 16 rows of the
-// contraction; eight digits add the exposed part of the drain, fewer take at least
-// the drain and write Y at 5 TB/s.  Slicing the factor, the launches and one tile's latency add 16 us.
+// The product: waves of tiles over the SMs, cycles per 16 rows of the contraction, the
+// exposed drain of a wide tile; a narrow one takes at least its drain.  Slicing the
+// factor, the launches and one tile's latency add 16 us.
 double ttm_product_cost(const jkcals_ctx* h, int a) {
-  const int P = h->ttm.digits, rows = ttm_tile_r(P);
+  const int rows = ttm_tile_r((int)h->dims[a]);
   const int64_t tiles = (int64_t)((h->C + kTtmTileC - 1) / kTtmTileC) * ((h->J[a] + rows - 1) / rows);
   const int64_t waves = (tiles + h->num_sms - 1) / h->num_sms;
   const int nk = ttm_ksteps((int)h->dims[a]);
-  if (P == 8) return waves * (nk * 1380.0 + 5000.0) / 1.9e9 + 16e-6;
-  const double step = P == 4 ? 510.0 : (P == 3 ? 390.0 : 310.0);
-  return std::max(waves * (std::max(nk * step, 3000.0) + 400.0) / 1.9e9,
-                  (P == 4 ? 8.0 : 4.0) * h->J[a] * h->C / 5e12) + 16e-6;
+  const double tile = rows == 64 ? nk * 1380.0 + 5000.0 : std::max(nk * 1130.0, 4000.0) + 600.0;
+  return waves * tile / 1.9e9 + 16e-6;
 }
-// A contraction reads Y once: at the FP64 pipe's measured 418 G multiply-adds/s on
-// 152 SMs, or FP32 values at the memory's rate.
+// A contraction reads Y once, at the FP64 pipe's measured 418 G multiply-adds/s on 152
+// SMs.
 double ttm_contract_cost(const jkcals_ctx* h, int a) {
-  const double n = (double)h->J[a] * h->C;
-  const int P = h->ttm.digits;
-  return (P == 8 ? n / (h->num_sms * 2.75e9) : (P == 4 ? 8.0 : 4.0) * n / 5e12) + 7e-6;
+  return (double)h->J[a] * h->C / (h->num_sms * 2.75e9) + 7e-6;
 }
-// The mode's own MTTKRP kernel on its padded tiles: 0.85 TFLOP/s on the CUDA cores;
-// the tensor-core forms' measured rates, padding included.
+// The CUDA-core MTTKRP runs its padded 64 x 64 tiles at about 0.85 TFLOP/s.
 double native_cost(const jkcals_ctx* h, int n) {
-  if (h->tc) {
-    const tc::TcPlan& p = h->tcplan[n];
-    double rate = 115e12;   // exact chain
-    switch (h->opt.precision) {
-      case JKCALS_TF32: rate = 180e12; break;
-      case JKCALS_3XTF32: rate = 155e12; break;
-      case JKCALS_BF16: rate = 290e12; break;
-      case JKCALS_SPLIT_BF16: rate = 125e12; break;
-      default: break;
-    }
-    // and the split-K partials, written and summed
-    const double part = (double)p.splits * h->dims[n] * h->C * (h->opt.precision == JKCALS_EXACT_BF16 ? 8.0 : 4.0);
-    return 2.0 * p.tiles_c * 128 * (double)p.tiles_n * p.BN * p.Jp / rate + part / 4.5e12 + 5e-6;
-  }
   return 2.0 * round_up(h->C, kMttkrpBN) * (double)round_up(h->dims[n], kMttkrpBM) * h->J[n] / 0.85e12 + 5e-6;
 }
 
 // Contracted mode for mode n's MTTKRP: the one Y holds, else the cheaper one
-// with images (-1: the mode's own kernel).
+// with images (-1: the CUDA-core kernel).
 int ttm_choose(const jkcals_ctx* h, int n, const int (&modes)[2], int y) {
   if (y >= 0 && y != n) return y;
   int best = -1;
@@ -545,7 +514,7 @@ double ttm_sweep_cost(const jkcals_ctx* h, const int (&modes)[2]) {
 
 // Whether the current column count goes through the products.  The factor 0.9
 // keeps sizes where the two are about even (the smallest tensors: launches and
-// latency) on the modes' own kernels, which need fewer launches.
+// latency) on the CUDA-core kernel, which needs fewer launches.
 void plan_ttm_use(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   t.use = false;
@@ -556,16 +525,14 @@ void plan_ttm_use(jkcals_ctx* h) {
 }
 
 // Modes whose images would make a sweep cheapest (t.modes; -1: none pays).
-// Explicit split-K factors ask for the modes' own kernels, and under a memory cap
-// the handle holds what those need and no more, so that later calls
+// Explicit split-K factors ask for the CUDA-core kernel, and under a memory cap
+// the handle holds what that kernel needs and no more, so that later calls
 // (gradients, loss histories, compaction) find the room the cap left them.
 constexpr int64_t kTtmMaxY = (int64_t)1 << 31;   // elements of Y (16 GiB)
 void choose_ttm_modes(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   t.modes[0] = t.modes[1] = -1;
-  if (h->opt.splits > 0 || h->opt.max_device_bytes > 0) return;
-  if (h->tc && h->N < 3) return;   // those products leave the column exponents to a contraction
-  t.digits = ttm_digits(h->opt.precision);
+  if (h->tc || h->opt.splits > 0 || h->opt.max_device_bytes > 0) return;
   auto ok = [&](int a) { return h->dims[a] <= kTtmChainMax && h->J[a] <= kTtmMaxY / h->C; };
   double best = 0.0;
   for (int x = 0; x < h->N; ++x)
@@ -588,7 +555,7 @@ void choose_ttm_modes(jkcals_ctx* h) {
 jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmState& st, int* kernels) {
   jkcals_ctx::Ttm& t = h->ttm;
   const int N = h->N;
-  void* part = h->part;
+  double* part = static_cast<double*>(h->part);
   const bool have_z = N >= 4 && st.z_a >= 0 && st.z_a != n && st.z_q != n;
   if (!have_z && st.y != a) {
     TtmArgs g{};
@@ -601,22 +568,22 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
     g.C = h->C;
     g.tiles_c = (h->C + kTtmTileC - 1) / kTtmTileC;
     g.J = h->J[a];
-    g.tiles_r = (h->J[a] + ttm_tile_r(t.digits) - 1) / ttm_tile_r(t.digits);
+    const int rows = ttm_tile_r(g.K);
+    g.tiles_r = (h->J[a] + rows - 1) / rows;
     g.Y = N == 2 ? part : t.Y;   // two modes: the product is the MTTKRP
     g.Tn = h->Tn64[a];
     g.U = U[a];
     g.err = h->d_err;
-    JK_CUDA(h, launch_slice_factor(t.digits, U[a], g.K, h->C, t.kexp[a], t.At, t.cexp[a], st.counter, h->stream));
+    JK_CUDA(h, launch_slice_factor(U[a], g.K, h->C, t.kexp[a], t.At, t.cexp[a], st.counter, h->stream));
     st.counter = nullptr;
-    JK_CUDA(h, launch_ttm(t.digits, g, h->num_sms, h->stream));
+    JK_CUDA(h, launch_ttm(g, h->num_sms, h->stream));
     t.ran = true;
     *kernels += 2;
     if (N > 2) st.y = a;
   }
   h->part_S = 1;
   if (N == 2) return JKCALS_OK;
-  const void* X = t.Y;
-  const int* cexp = t.cexp[have_z ? st.z_a : a];
+  const double* X = t.Y;
   std::vector<int> rest;   // modes of X, fastest first
   for (int k = 0; k < N; ++k)
     if (have_z ? (k != st.z_a && k != st.z_q) : k != a) rest.push_back(k);
@@ -628,11 +595,10 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
     const int q = rest[pos];
     int64_t L = 1, H = 1;
     for (size_t k = 0; k < rest.size(); ++k) (k < pos ? L : H) *= k == pos ? 1 : h->dims[rest[k]];
-    void* out = part;
+    double* out = part;
     int S = 1;
-    const bool fin = rest.size() == 2;
-    if (fin) {
-      S = contract_splits(t.digits, H * L, (int)h->dims[q], h->C);
+    if (rest.size() == 2) {
+      S = contract_splits(H * L, (int)h->dims[q], h->C);
       const int64_t cap = (int64_t)(h->part_bytes / 8) / (H * L * h->C);
       S = (int)std::max<int64_t>(1, std::min<int64_t>(S, cap));
       S = (int)((h->dims[q] + (h->dims[q] + S - 1) / S - 1) / ((h->dims[q] + S - 1) / S));
@@ -645,7 +611,7 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
       out = t.W[w];
       w ^= 1;
     }
-    JK_CUDA(h, launch_contract(t.digits, X, H, (int)h->dims[q], L, h->C, U[q], S, fin ? cexp : nullptr, out, h->stream));
+    JK_CUDA(h, launch_contract(X, H, (int)h->dims[q], L, h->C, U[q], S, out, h->stream));
     *kernels += 1;
     X = out;
     rest.erase(rest.begin() + pos);
@@ -798,7 +764,7 @@ jkcals_status enqueue_sweep(jkcals_ctx* h) {
   TtmState ttm;
   if (h->ttm.use) ttm.counter = h->d_sweep_idx;
   for (int n = 0; n < h->N; ++n) {
-    const bool tts = h->tc && h->tcplan[n].tts && !(h->ttm.use && ttm_choose(h, n, h->ttm.modes, ttm.y) >= 0);
+    const bool tts = h->tc && h->tcplan[n].tts;
     const bool reuse = tts && sliced == h->tcplan[n].a_mode;
     if (h->opt.kernel_timing) JK_CUDA(h, cudaEventRecordWithFlags(h->ev_start[n], h->stream, cudaEventRecordExternal));
     JK_TRY(enqueue_mttkrp(h, n, h->U, h->UT, h->UTlo, h->cmax, reuse, &ttm, &kernels));
@@ -1056,13 +1022,13 @@ namespace {
 size_t ttm_part_elems(const jkcals_ctx* h, int n) {
   size_t most = 0;
   for (int q = 0; q < h->N; ++q)
-    if (q != n) most = std::max(most, (size_t)contract_splits(h->ttm.digits, h->dims[n], (int)h->dims[q], h->C));
+    if (q != n) most = std::max(most, (size_t)contract_splits(h->dims[n], (int)h->dims[q], h->C));
   return most * h->dims[n] * h->C;
 }
 
-// The products' buffers are an addition to what the modes' own kernels need: if the
+// The products' buffers are an addition to what the CUDA-core kernel needs: if the
 // device has no room for them, or T holds a non-finite entry, the handle drops
-// them and runs on those kernels.
+// them and runs on that kernel.
 void ttm_drop(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   void* all[] = {t.At, t.Y, t.Z, t.W[0], t.W[1]};
@@ -1089,12 +1055,13 @@ jkcals_status create_ttm_images(jkcals_ctx* h) {
     for (int a : t.modes) {
       if (a < 0) continue;
       void* img = nullptr;
-      JK_TRY(dalloc(h, &img, ttm_image_bytes(t.digits, (int)h->dims[a], h->J[a], ttm_tile_r(t.digits))));
+      const int rows = ttm_tile_r((int)h->dims[a]);
+      JK_TRY(dalloc(h, &img, ttm_image_bytes((int)h->dims[a], h->J[a], rows)));
       t.Bt[a] = static_cast<unsigned char*>(img);
       JK_TRY(dalloc_t(h, &t.kexp[a], (size_t)h->dims[a]));
-      JK_TRY(dalloc_t(h, &t.rexp[a], (size_t)round_up(h->J[a], ttm_tile_r(t.digits))));
+      JK_TRY(dalloc_t(h, &t.rexp[a], (size_t)round_up(h->J[a], rows)));
       JK_CUDA(h, launch_slice_exponents(h->Tn64[a], h->dims[a], h->J[a], t.kexp[a], d_bad, st));
-      JK_CUDA(h, launch_slice_tensor(t.digits, h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], st));
+      JK_CUDA(h, launch_slice_tensor(h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], st));
     }
     return JKCALS_OK;
   };
@@ -1119,7 +1086,7 @@ jkcals_status create_ttm_workspace(jkcals_ctx* h) {
     for (int a : t.modes) {
       if (a < 0) continue;
       JK_TRY(dalloc_t(h, &t.cexp[a], (size_t)round_up(h->C, kTtmTileC)));
-      at = std::max(at, ttm_image_bytes(t.digits, (int)h->dims[a], h->C, kTtmTileC));
+      at = std::max(at, ttm_image_bytes((int)h->dims[a], h->C, kTtmTileC));
       if (h->N > 2) y = std::max(y, (size_t)h->J[a] * h->C);
       for (int q = 0; q < h->N && h->N >= 4; ++q) {
         if (q == a) continue;
@@ -1131,11 +1098,12 @@ jkcals_status create_ttm_workspace(jkcals_ctx* h) {
     void* img = nullptr;
     JK_TRY(dalloc(h, &img, at));
     t.At = static_cast<unsigned char*>(img);
-    if (y > 0) JK_TRY(dalloc(h, &t.Y, 8 * y));
-    if (z > 0) JK_TRY(dalloc(h, &t.Z, 8 * z));
-    for (int k = 0; k < 2 && w > 0; ++k) JK_TRY(dalloc(h, &t.W[k], 8 * w));
+    if (y > 0) JK_TRY(dalloc_t(h, &t.Y, y));
+    if (z > 0) JK_TRY(dalloc_t(h, &t.Z, z));
+    for (int k = 0; k < 2 && w > 0; ++k) JK_TRY(dalloc_t(h, &t.W[k], w));
     JK_TRY(create_error_word(h));
-    JK_CUDA(h, prepare_ttm(t.digits));
+    for (int a : t.modes)
+      if (a >= 0) JK_CUDA(h, prepare_ttm((int)h->dims[a]));
     return JKCALS_OK;
   };
   const jkcals_status s = build();
@@ -1253,8 +1221,6 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
                                         p.Ia_pad, p.Jp, mp, h->rowexp[n], p.BN, p.tiles_n, p.nkt, h->Tt[n], st));
       h->Ipad[n] = round_up(h->dims[n], chunk);
     }
-    choose_ttm_modes(h);
-    JK_TRY(create_ttm_images(h));
     JK_CUDA(h, cudaStreamSynchronize(st));
     for (int n = 0; n < N; ++n) {
       dfree(h, h->Tn64[n], true);
@@ -2070,14 +2036,12 @@ struct jkcals_batch_ctx {
 namespace {
 
 // A batch sweep runs as grouped launches when every problem uses the same
-// tensor-core form and order, no mode takes the two-step form or a
-// tensor-times-matrix product and no handle
+// tensor-core form and order, no mode takes the two-step form and no handle
 // asked for per-problem branches.
 bool batch_groupable(const std::vector<jkcals_ctx*>& hs) {
   for (jkcals_ctx* h : hs) {
     if (h->opt.batch_branches || !h->tc || h->opt.precision != hs[0]->opt.precision || h->N != hs[0]->N)
       return false;
-    if (h->ttm.use) return false;   // grouped launches run the modes' own kernels
     for (int n = 0; n < h->N; ++n)
       if (h->tcplan[n].tts) return false;
   }

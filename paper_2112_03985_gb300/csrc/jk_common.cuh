@@ -163,7 +163,7 @@ struct jkcals_ctx {
   double* gG[jk::kMaxModes] = {nullptr};
   double* geg = nullptr;  // K per-block losses + their sum
 
-  // tensor-times-matrix products (jk_ttm.cu)
+  // FP64 form: tensor-times-matrix products on the tensor cores (jk_ttm.cu)
   struct Ttm {
     int modes[2] = {-1, -1};                       // contracted modes with images of T (-1: none)
     bool use = false;                              // the current plan's MTTKRPs go through them
@@ -173,11 +173,9 @@ struct jkcals_ctx {
     int* rexp[jk::kMaxModes] = {nullptr};          // exponents of T_(a)'s scaled columns (padded to tiles)
     unsigned char* At = nullptr;                   // digit images of Ubar^(a), rewritten per product
     int* cexp[jk::kMaxModes] = {nullptr};          // exponents of its scaled columns (padded to tiles)
-    // FP64 values, FP32 pairs (exact-chain form) or FP32 values:
-    void* Y = nullptr;                             // the product, J_a x C
-    void* Z = nullptr;                             // N >= 4: Y contracted with one more mode
-    void* W[2] = {nullptr, nullptr};               // N >= 5: the further contractions
-    int digits = 8;                                // of 7 bits per operand, by form
+    double* Y = nullptr;                           // the product, J_a x C
+    double* Z = nullptr;                           // N >= 4: Y contracted with one more mode
+    double* W[2] = {nullptr, nullptr};             // N >= 5: the further contractions
   } ttm;
   int part_S = 1;  // splits of the partial sums in `part` (set by each MTTKRP)
 
@@ -357,8 +355,10 @@ cudaError_t launch_reduce_partials_f32(const float* part, int S, int64_t count, 
 
 // ---- tensor-times-matrix products on the tensor cores (jk_ttm.cu) -------------
 constexpr int kTtmTileC = 128;                   // tile of Y: columns c
-// its rows r: what the levels' accumulators leave of TMEM (see jk_ttm.cu)
-constexpr int ttm_tile_r(int digits) { return digits == 2 ? 128 : (digits == 3 ? 80 : 64); }
+// Its rows r, by the contraction's length K: 64 with an exposed drain, or for short
+// contractions, where that drain would take more than the MMAs, 32 with a hidden one
+// (jk_ttm.cu has both sides' figures).
+constexpr int ttm_tile_r(int K) { return K > 64 ? 64 : 32; }
 // longest contraction whose level sums are exact: (l + 3) 2^12 K <= 2^24 for l <= 6
 constexpr int kTtmChainMax = 448;
 constexpr int kTtmBadExp = 2147483647;           // exponent of a column with a non-finite entry
@@ -370,27 +370,25 @@ struct TtmArgs {
   const int* rexp;           // per row r of Y (padded to tiles)
   int nk, K, C, tiles_c;
   int64_t J, tiles_r;
-  void* Y;                   // J x C: FP64 (eight digits), FP32 pairs (four) or FP32, the latter without 2^cexp
-  const double* Tn;          // T_(a), K x J (eight digits: columns with non-finite entries)
+  double* Y;                 // J x C
+  const double* Tn;          // T_(a), K x J (columns of Ubar^(a) with non-finite entries)
   const double* U;           // Ubar^(a), K x C
   int* err;
 };
-inline size_t ttm_image_bytes(int digits, int K, int64_t M, int tile) {
-  return (size_t)((M + tile - 1) / tile) * ttm_ksteps(K) * digits * tile * 32;
+inline size_t ttm_image_bytes(int K, int64_t M, int tile) {   // eight digits of 32 bytes per 16 rows
+  return (size_t)((M + tile - 1) / tile) * ttm_ksteps(K) * 8 * tile * 32;
 }
 cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* kexp, int* bad, cudaStream_t s);
-cudaError_t launch_slice_tensor(int digits, const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt,
+cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt,
                                 int* rexp, cudaStream_t s);
-cudaError_t launch_slice_factor(int digits, const double* U, int I, int C, const int* kexp, unsigned char* At,
+cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At,
                                 int* cexp, int* counter, cudaStream_t s);
-cudaError_t prepare_ttm(int digits);
-cudaError_t launch_ttm(int digits, const TtmArgs& a, int num_sms, cudaStream_t s);
+cudaError_t prepare_ttm(int K);
+cudaError_t launch_ttm(const TtmArgs& a, int num_sms, cudaStream_t s);
 // out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c]
-int contract_splits(int digits, int64_t HL, int Mm, int C);
-// X, out: FP64 (eight digits), FP32 pairs (four) or FP32; cexp: the columns' exponents,
-// for the last contraction of an MTTKRP of fewer than eight digits (else null)
-cudaError_t launch_contract(int digits, const void* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
-                            const int* cexp, void* out, cudaStream_t s);
+int contract_splits(int64_t HL, int Mm, int C);
+cudaError_t launch_contract(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S, double* out,
+                            cudaStream_t s);
 
 // Storage of split-K partials: FP64, FP32, or an unevaluated FP32 pair (hi, lo).
 constexpr int kPartF64 = 0, kPartF32 = 1, kPartF32x2 = 2;

