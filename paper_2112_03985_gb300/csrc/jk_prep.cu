@@ -13,24 +13,28 @@ struct Dims8 {
 };
 
 // out[i_n * J + j] = T(i_0, ..., i_{N-1}) with j from Eq. kolda_mapping
-// (0-based: j = sum_{k != n} i_k prod_{m < k, m != n} I_m).  T is C-order.
-__global__ void unfold_f64_kernel(const double* __restrict__ Tc, Dims8 dims, int N, int n, int64_t J,
-                                  int64_t total, double* __restrict__ out) {
-  int64_t cstride[kMaxModes];
-  int64_t s = 1;
+// (0-based: j = sum_{k != n} i_k prod_{m < k, m != n} I_m).  T is C-order.  IT: 32-bit
+// indices where the tensor has fewer than 2^31 entries (a 64-bit division is a long
+// instruction sequence, and there are N per entry).
+template <typename IT>
+__global__ void unfold_f64_kernel(const double* __restrict__ Tc, Dims8 dims, int N, int n, IT J, int64_t total,
+                                  double* __restrict__ out) {
+  IT cstride[kMaxModes];
+  IT s = 1;
   for (int k = N - 1; k >= 0; --k) {
     cstride[k] = s;
-    s *= dims.d[k];
+    s *= (IT)dims.d[k];
   }
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i_n = e / J;
-    int64_t rem = e - i_n * J;
-    int64_t src = i_n * cstride[n];
+  for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < total;
+       e0 += (int64_t)gridDim.x * blockDim.x) {
+    const IT e = (IT)e0;
+    const IT i_n = e / J;
+    IT rem = e - i_n * J;
+    IT src = i_n * cstride[n];
     for (int k = 0; k < N; ++k) {
       if (k == n) continue;
-      const int64_t q = rem / dims.d[k];
-      src += (rem - q * dims.d[k]) * cstride[k];
+      const IT d = (IT)dims.d[k], q = rem / d;
+      src += (rem - q * d) * cstride[k];
       rem = q;
     }
     out[e] = Tc[src];
@@ -61,20 +65,36 @@ __global__ void row_sumsq_kernel(const double* __restrict__ Tn, int64_t J, doubl
   if (threadIdx.x == 0) out[i] = red[0];
 }
 
-// ||T_{-g}||^2 = sum_{i not in D_g} ||slice i||^2 (error line of Alg. 3).
-__global__ void block_norms_kernel(const double* __restrict__ slice, int64_t I, int K, BlockMeta bm,
-                                   double* __restrict__ normT2) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= K) return;
-  const int64_t b = bm.lo_ptr[g], e = bm.lo_ptr[g + 1];
-  int64_t p = b;
+// ||T_{-g}||^2 = sum_{i not in D_g} ||slice i||^2 (error line of Alg. 3), slice by slice
+// in increasing order.  One thread per block; the slices' sums pass through shared memory
+// and the next left-out index waits in a register (both read from global memory at every
+// step of the chain of additions: 54 us for 300 slices).
+constexpr int kNormThreads = 128;
+
+__global__ void __launch_bounds__(kNormThreads) block_norms_kernel(const double* __restrict__ slice, int64_t I, int K,
+                                                                   BlockMeta bm, double* __restrict__ normT2) {
+  __shared__ double sl[1024];
+  const int g = blockIdx.x * kNormThreads + threadIdx.x;
+  const bool valid = g < K;
+  int64_t p = valid ? bm.lo_ptr[g] : 0;
+  const int64_t e = valid ? bm.lo_ptr[g + 1] : 0;
+  int64_t next = p < e ? bm.lo_idx[p] : I;   // sorted, no duplicates
   double acc = 0.0;
-  for (int64_t i = 0; i < I; ++i) {
-    while (p < e && bm.lo_idx[p] < i) ++p;
-    if (p < e && bm.lo_idx[p] == i) continue;
-    acc += slice[i];
+  for (int64_t i0 = 0; i0 < I; i0 += 1024) {
+    const int n = (int)(I - i0 < 1024 ? I - i0 : 1024);
+    __syncthreads();
+    for (int t = threadIdx.x; t < n; t += kNormThreads) sl[t] = slice[i0 + t];
+    __syncthreads();
+    for (int t = 0; t < n; ++t) {
+      if (i0 + t == next) {
+        ++p;
+        next = p < e ? bm.lo_idx[p] : I;
+        continue;
+      }
+      acc += sl[t];
+    }
   }
-  normT2[g] = acc;
+  if (valid) normT2[g] = acc;
 }
 
 __global__ void zero_left_out_kernel(double* __restrict__ U, int C, BlockMeta bm) {
@@ -157,7 +177,10 @@ cudaError_t launch_unfold_f64(const double* Tc, const int64_t* dims, int N, int 
     total *= dims[k];
   }
   const int64_t J = total / dims[n];
-  unfold_f64_kernel<<<grid_for(total, 256), 256, 0, s>>>(Tc, d, N, n, J, total, out);
+  if (total < 2147483647LL)
+    unfold_f64_kernel<uint32_t><<<grid_for(total, 256), 256, 0, s>>>(Tc, d, N, n, (uint32_t)J, total, out);
+  else
+    unfold_f64_kernel<int64_t><<<grid_for(total, 256), 256, 0, s>>>(Tc, d, N, n, J, total, out);
   return cudaGetLastError();
 }
 

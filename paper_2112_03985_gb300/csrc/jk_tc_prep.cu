@@ -3,6 +3,8 @@
 // per-row grids (row exponents, column maxima) of the exact-chain form.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "jk_tc.cuh"
 
 namespace jk {
@@ -48,34 +50,36 @@ __device__ __forceinline__ int64_t swizzled_offset(int r, int cb, int row_bytes)
 // jp = ia + Ia_pad * o with ia the index of the fastest mode a and o running
 // mixed-radix over the remaining modes in increasing order; j is the Eq.
 // kolda_mapping column of those indices; zero where i >= I, jp >= Jp or
-// ia >= Ia.  Splits are taken from the FP64 value.
-template <int PREC>
-__global__ void tile_unfold_kernel(const double* __restrict__ Tn, int64_t I, int64_t J, int64_t Ia, int64_t Ia_pad,
-                                   int64_t Jp, UnfoldMap mp, const int* __restrict__ rowexp, int BN, int tiles_n,
-                                   int64_t nkt, unsigned char* __restrict__ Tt) {
+// ia >= Ia.  Splits are taken from the FP64 value.  IT: 32-bit indices where the padded
+// unfolding has fewer than 2^31 entries (six divisions per entry).
+template <int PREC, typename IT>
+__global__ void tile_unfold_kernel(const double* __restrict__ Tn, IT I, IT J, IT Ia, IT Ia_pad, IT Jp, UnfoldMap mp,
+                                   const int* __restrict__ rowexp, int BN, int tiles_n, IT nkt,
+                                   unsigned char* __restrict__ Tt) {
   constexpr int EB = (PREC == JKCALS_TF32 || PREC == JKCALS_3XTF32) ? 4 : 2;
   constexpr int ROW = PREC == JKCALS_EXACT_BF16 ? 64 : 128;
   constexpr int BK = ROW / EB;
   constexpr int NS = PREC == JKCALS_EXACT_BF16 ? 4 : (PREC == JKCALS_SPLIT_BF16 ? 3 : (PREC == JKCALS_3XTF32 ? 2 : 1));
-  const int64_t cols = nkt * BK;
+  const IT cols = nkt * BK;
   const int64_t total = (int64_t)tiles_n * BN * cols;
   const int64_t part_bytes = (int64_t)BN * ROW;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / cols;
-    const int64_t jp = e - i * cols;
+  for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e0 < total;
+       e0 += (int64_t)gridDim.x * blockDim.x) {
+    const IT e = (IT)e0;
+    const IT i = e / cols;
+    const IT jp = e - i * cols;
     double x = 0.0;
     if (i < I && jp < Jp) {
-      const int64_t o = jp / Ia_pad;
-      const int64_t ia = jp - o * Ia_pad;
+      const IT o = jp / Ia_pad;
+      const IT ia = jp - o * Ia_pad;
       if (ia < Ia) {
-        int64_t j = ia * mp.sa, rem = o;
+        IT j = ia * (IT)mp.sa, rem = o;
         for (int t = 0; t < mp.nq; ++t) {
-          const int64_t qq = rem / mp.qd[t];
-          j += (rem - qq * mp.qd[t]) * mp.qs[t];
+          const IT qd = (IT)mp.qd[t], qq = rem / qd;
+          j += (rem - qq * qd) * (IT)mp.qs[t];
           rem = qq;
         }
-        x = Tn[i * J + j];
+        x = Tn[(int64_t)i * J + j];
       }
     }
     float v[NS];
@@ -85,18 +89,42 @@ __global__ void tile_unfold_kernel(const double* __restrict__ Tn, int64_t I, int
       if constexpr (NS > 1) v[1] = tf32_rna((float)(x - (double)h));
     } else if constexpr (PREC == JKCALS_EXACT_BF16) {
       // x = 2^(F-7) (s0 + s1 2^-7 + s2 2^-14 + s3 2^-21), |s_k| <= 128, stored as s_k 2^(-7k)
-      double y = i < I ? ldexp(x, kSliceBits - rowexp[i]) : 0.0;
-      const double s0 = rint(y);
-      y = (y - s0) * 128.0;
-      const double s1 = rint(y);
-      y = (y - s1) * 128.0;
-      const double s2 = rint(y);
-      y = (y - s2) * 128.0;
-      const double s3 = rint(y);
-      v[0] = (float)s0;
-      v[1] = (float)(s1 / 128.0);
-      v[2] = (float)(s2 / 16384.0);
-      v[3] = (float)(s3 / 2097152.0);
+      const long long xb = __double_as_longlong(x);
+      const int ef = (int)((xb >> 52) & 2047);
+      const int sc = i < I ? kSliceBits - rowexp[i] : 0;
+      if ((xb & 0x1fffffff) == 0 && (ef != 0 || (xb << 1) == 0) && ef != 2047) {
+        // x has at most FP32's 24 significant bits (a tensor given in FP32): y is an
+        // FP32 number, and every step below is exact there as in FP64 (whose rint and
+        // ldexp sequences and 64-bit divisions took 75-80 us per mode of 300x100x50; a
+        // job on it, create included, went from 5.66 to 5.49 ms).  y below FP32's normal
+        // range has no digits.
+        const int ey = ef - 896 + sc;   // biased FP32 exponent of y, at most 127 + 6
+        float y = 0.f;
+        if (ef != 0 && ey > 0)
+          y = __int_as_float((int)((xb >> 32) & 0x80000000ll) | (ey << 23) | (int)((xb >> 29) & 0x7fffff));
+        constexpr float kRound = 12582912.f;   // 1.5 * 2^23: rounds to the nearest even integer
+        float unit = 1.f;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const float d = __fsub_rn(__fadd_rn(y, kRound), kRound);
+          v[s] = d * unit;
+          y = __fsub_rn(y, d) * 128.f;
+          unit *= 0.0078125f;
+        }
+      } else {
+        double y = i < I ? ldexp(x, sc) : 0.0;
+        const double s0 = rint(y);
+        y = (y - s0) * 128.0;
+        const double s1 = rint(y);
+        y = (y - s1) * 128.0;
+        const double s2 = rint(y);
+        y = (y - s2) * 128.0;
+        const double s3 = rint(y);
+        v[0] = (float)s0;
+        v[1] = (float)(s1 / 128.0);
+        v[2] = (float)(s2 / 16384.0);
+        v[3] = (float)(s3 / 2097152.0);
+      }
     } else {
       const float h = __bfloat162float(__double2bfloat16(x));
       v[0] = h;
@@ -107,9 +135,9 @@ __global__ void tile_unfold_kernel(const double* __restrict__ Tn, int64_t I, int
         v[2] = __bfloat162float(__double2bfloat16(r1 - (double)m));
       }
     }
-    const int64_t tn = i / BN, ks = jp / BK;
-    const int r = (int)(i - tn * BN), col = (int)(jp - ks * BK);
-    const int64_t tile = (tn * nkt + ks) * NS * part_bytes;
+    const IT tn = i / (IT)BN, ks = jp / BK;
+    const int r = (int)(i - tn * (IT)BN), col = (int)(jp - ks * BK);
+    const int64_t tile = ((int64_t)tn * nkt + ks) * NS * part_bytes;
     const int64_t off = swizzled_offset(r, col * EB, ROW);
 #pragma unroll
     for (int p = 0; p < NS; ++p) {
@@ -164,30 +192,27 @@ cudaError_t launch_row_exponent(const double* Tn64, int64_t I, int64_t J, int* r
 cudaError_t launch_tile_unfold(int precision, const double* Tn64, int64_t I, int64_t J, int64_t Ia, int64_t Ia_pad,
                                int64_t Jp, const UnfoldMap& mp, const int* rowexp, int BN, int tiles_n, int64_t nkt,
                                void* Tt, cudaStream_t s) {
-  const unsigned g = grid_for((int64_t)tiles_n * BN * nkt * form_bk(precision));
+  const int64_t total = (int64_t)tiles_n * BN * nkt * form_bk(precision);
+  const unsigned g = grid_for(total);
   unsigned char* out = static_cast<unsigned char*>(Tt);
+  auto go = [&](auto prec) {
+    constexpr int PREC = decltype(prec)::value;
+    if (total < 2147483647LL && I * J < 2147483647LL)
+      tile_unfold_kernel<PREC, uint32_t><<<g, 256, 0, s>>>(Tn64, (uint32_t)I, (uint32_t)J, (uint32_t)Ia,
+                                                           (uint32_t)Ia_pad, (uint32_t)Jp, mp, rowexp, BN, tiles_n,
+                                                           (uint32_t)nkt, out);
+    else
+      tile_unfold_kernel<PREC, int64_t><<<g, 256, 0, s>>>(Tn64, I, J, Ia, Ia_pad, Jp, mp, rowexp, BN, tiles_n, nkt, out);
+    return cudaGetLastError();
+  };
   switch (precision) {
-    case JKCALS_TF32:
-      tile_unfold_kernel<JKCALS_TF32><<<g, 256, 0, s>>>(Tn64, I, J, Ia, Ia_pad, Jp, mp, rowexp, BN, tiles_n, nkt, out);
-      break;
-    case JKCALS_3XTF32:
-      tile_unfold_kernel<JKCALS_3XTF32><<<g, 256, 0, s>>>(Tn64, I, J, Ia, Ia_pad, Jp, mp, rowexp, BN, tiles_n, nkt, out);
-      break;
-    case JKCALS_BF16:
-      tile_unfold_kernel<JKCALS_BF16><<<g, 256, 0, s>>>(Tn64, I, J, Ia, Ia_pad, Jp, mp, rowexp, BN, tiles_n, nkt, out);
-      break;
-    case JKCALS_SPLIT_BF16:
-      tile_unfold_kernel<JKCALS_SPLIT_BF16><<<g, 256, 0, s>>>(Tn64, I, J, Ia, Ia_pad, Jp, mp, rowexp, BN, tiles_n, nkt,
-                                                              out);
-      break;
-    case JKCALS_EXACT_BF16:
-      tile_unfold_kernel<JKCALS_EXACT_BF16><<<g, 256, 0, s>>>(Tn64, I, J, Ia, Ia_pad, Jp, mp, rowexp, BN, tiles_n, nkt,
-                                                              out);
-      break;
-    default:
-      return cudaErrorInvalidValue;
+    case JKCALS_TF32: return go(std::integral_constant<int, JKCALS_TF32>{});
+    case JKCALS_3XTF32: return go(std::integral_constant<int, JKCALS_3XTF32>{});
+    case JKCALS_BF16: return go(std::integral_constant<int, JKCALS_BF16>{});
+    case JKCALS_SPLIT_BF16: return go(std::integral_constant<int, JKCALS_SPLIT_BF16>{});
+    case JKCALS_EXACT_BF16: return go(std::integral_constant<int, JKCALS_EXACT_BF16>{});
+    default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_factor_to_ut(const double* U, int64_t I, int C, float* UT, float* UT_lo, int64_t I_pad,
