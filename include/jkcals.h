@@ -61,7 +61,10 @@ typedef enum {
   JKCALS_FP64 = 0,        /* FP64 accuracy: products and sums on the CUDA cores, or, where
                              cheaper, tensor-times-matrix products shared by several modes
                              whose operands are cut into eight 7-bit BF16 digits and summed
-                             exactly on the tensor cores, rounded to FP64 once           */
+                             exactly on the tensor cores, rounded to FP64 once; entries of a
+                             product whose terms lie far below their vectors' maxima (an
+                             outlying sample left out, tails of separated peaks) are summed
+                             in FP64, so that each is accurate relative to its own terms */
   JKCALS_TF32 = 1,        /* tcgen05 kind::tf32, FP32 accumulation in TMEM             */
   JKCALS_3XTF32 = 2,      /* hi*hi + hi*lo + lo*hi TF32 products, FP32 accumulation    */
   JKCALS_BF16 = 3,        /* tcgen05 kind::f16 with BF16 operands, FP32 accumulation   */

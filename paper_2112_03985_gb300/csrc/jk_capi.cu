@@ -563,6 +563,8 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
     g.Bt = t.Bt[a];
     g.cexp = t.cexp[a];
     g.rexp = t.rexp[a];
+    g.cmag = t.cmag[a];
+    g.rmag = t.rmag[a];
     g.K = (int)h->dims[a];
     g.nk = ttm_ksteps(g.K);
     g.C = h->C;
@@ -574,7 +576,8 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
     g.Tn = h->Tn64[a];
     g.U = U[a];
     g.err = h->d_err;
-    JK_CUDA(h, launch_slice_factor(U[a], g.K, h->C, t.kexp[a], t.At, t.cexp[a], st.counter, h->stream));
+    JK_CUDA(h, launch_slice_factor(U[a], g.K, h->C, t.kexp[a], t.At, t.cexp[a], t.cmag[a], st.counter,
+                                   h->stream));
     st.counter = nullptr;
     JK_CUDA(h, launch_ttm(g, h->num_sms, h->stream));
     t.ran = true;
@@ -1038,6 +1041,8 @@ void ttm_drop(jkcals_ctx* h) {
     dfree(h, t.kexp[n], true);
     dfree(h, t.rexp[n], true);
     dfree(h, t.cexp[n], true);
+    dfree(h, t.rmag[n], true);
+    dfree(h, t.cmag[n], true);
   }
   t = jkcals_ctx::Ttm{};
   set_error("");
@@ -1061,7 +1066,8 @@ jkcals_status create_ttm_images(jkcals_ctx* h) {
       JK_TRY(dalloc_t(h, &t.kexp[a], (size_t)h->dims[a]));
       JK_TRY(dalloc_t(h, &t.rexp[a], (size_t)round_up(h->J[a], rows)));
       JK_CUDA(h, launch_slice_exponents(h->Tn64[a], h->dims[a], h->J[a], t.kexp[a], d_bad, st));
-      JK_CUDA(h, launch_slice_tensor(h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], st));
+      JK_TRY(dalloc_t(h, &t.rmag[a], (size_t)round_up(h->J[a], rows) * ttm_ksteps((int)h->dims[a]) * 16));
+      JK_CUDA(h, launch_slice_tensor(h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], t.rmag[a], st));
     }
     return JKCALS_OK;
   };
@@ -1086,6 +1092,7 @@ jkcals_status create_ttm_workspace(jkcals_ctx* h) {
     for (int a : t.modes) {
       if (a < 0) continue;
       JK_TRY(dalloc_t(h, &t.cexp[a], (size_t)round_up(h->C, kTtmTileC)));
+      JK_TRY(dalloc_t(h, &t.cmag[a], (size_t)round_up(h->C, kTtmTileC) * ttm_ksteps((int)h->dims[a]) * 16));
       at = std::max(at, ttm_image_bytes((int)h->dims[a], h->C, kTtmTileC));
       if (h->N > 2) y = std::max(y, (size_t)h->J[a] * h->C);
       for (int q = 0; q < h->N && h->N >= 4; ++q) {

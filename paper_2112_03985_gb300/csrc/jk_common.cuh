@@ -170,9 +170,11 @@ struct jkcals_ctx {
     bool ran = false;                              // one was enqueued since the last error check
     unsigned char* Bt[jk::kMaxModes] = {nullptr};  // digit images of T_(a)
     int* kexp[jk::kMaxModes] = {nullptr};          // I_a slice exponents
-    int* rexp[jk::kMaxModes] = {nullptr};          // exponents of T_(a)'s scaled columns (padded to tiles)
+    int2* rexp[jk::kMaxModes] = {nullptr};         // exponents of T_(a)'s scaled columns (padded to tiles)
+    unsigned char* rmag[jk::kMaxModes] = {nullptr};   // their magnitudes' leading bits
     unsigned char* At = nullptr;                   // digit images of Ubar^(a), rewritten per product
-    int* cexp[jk::kMaxModes] = {nullptr};          // exponents of its scaled columns (padded to tiles)
+    int2* cexp[jk::kMaxModes] = {nullptr};         // exponents of its scaled columns (padded to tiles)
+    unsigned char* cmag[jk::kMaxModes] = {nullptr};   // their magnitudes' leading bits
     double* Y = nullptr;                           // the product, J_a x C
     double* Z = nullptr;                           // N >= 4: Y contracted with one more mode
     double* W[2] = {nullptr, nullptr};             // N >= 5: the further contractions
@@ -362,16 +364,19 @@ constexpr int ttm_tile_r(int K) { return K > 64 ? 64 : 32; }
 // longest contraction whose level sums are exact: (l + 3) 2^12 K <= 2^24 for l <= 6
 constexpr int kTtmChainMax = 448;
 constexpr int kTtmBadExp = 2147483647;           // exponent of a column with a non-finite entry
+constexpr int kTtmZeroExp = -(1 << 28);          // exponent of a zero column
 inline int ttm_ksteps(int K) { return (K + 15) / 16; }
 struct TtmArgs {
   const unsigned char* At;   // digit images of Ubar^(a): tiles_c x nk steps of 16 rows
   const unsigned char* Bt;   // digit images of T_(a): tiles_r x nk steps
-  const int* cexp;           // per column c (padded to tiles)
-  const int* rexp;           // per row r of Y (padded to tiles)
+  const int2* cexp;          // per column c (padded to tiles): exponent, entries near the largest
+  const int2* rexp;          // per row r of Y (padded to tiles)
+  const unsigned char* cmag; // magnitudes of the scaled column, 16 nk bytes per column c
+  const unsigned char* rmag; // the same per row r
   int nk, K, C, tiles_c;
   int64_t J, tiles_r;
   double* Y;                 // J x C
-  const double* Tn;          // T_(a), K x J (columns of Ubar^(a) with non-finite entries)
+  const double* Tn;          // T_(a), K x J (entries that the digits do not carry)
   const double* U;           // Ubar^(a), K x C
   int* err;
 };
@@ -380,9 +385,9 @@ inline size_t ttm_image_bytes(int K, int64_t M, int tile) {   // eight digits of
 }
 cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* kexp, int* bad, cudaStream_t s);
 cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt,
-                                int* rexp, cudaStream_t s);
+                                int2* rexp, unsigned char* rmag, cudaStream_t s);
 cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At,
-                                int* cexp, int* counter, cudaStream_t s);
+                                int2* cexp, unsigned char* cmag, int* counter, cudaStream_t s);
 cudaError_t prepare_ttm(int K);
 cudaError_t launch_ttm(const TtmArgs& a, int num_sms, cudaStream_t s);
 // out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c]

@@ -20,15 +20,29 @@
 // accumulator in TMEM.  A level's terms are integers and its sum stays below
 // (l + 3) 2^12 K <= 2^24 for chains of K <= kTtmChainMax, so levels 0 to 6 are
 // exact whatever the order of the additions; level 7 may truncate in its own
-// last bits (2^-63 of the product of the vectors' maxima).  What is dropped is
-// the operands' rounding (2^-59) and the products beyond level 7 (seven terms
-// of about 2^-60 each): below the rounding of a single FP64 multiply-add per
-// term.  The drain adds the levels as 64-bit integers and rounds once to FP64.
+// last bits (2^-63 of the product of the vectors' maxima).  The drain adds the levels as
+// 64-bit integers and rounds once to FP64.
+//
+// Bound.  Let 2^E and 2^F bound the two vectors' magnitudes and S be the sum of the
+// magnitudes of an entry's K terms.  Dropped are the operands' rounding (at most 2^-58 per
+// term) and the products beyond level 7 (seven of at most 2^-58 per term): at most
+// K 2^-55 2^(E+F), typically sqrt(7 K) 2^-60 2^(E+F).  That is measured by the vectors'
+// maxima, not by the entry's own terms, so it is accepted only where S >= 2^-5 2^(E+F):
+// the error is then at most 8 K 2^-53 S and typically 0.7 sqrt(K) 2^-53 S or less, that of
+// an FP64 chain of about 10 K terms (K <= 448; the CUDA-core kernel's chains are 800 to
+// 1200 terms at 300x100x50, K 100 and 300, and 12000 at 400x400x400).  The
+// drain finds S from below by the entry's own value, or else by the products of the
+// magnitudes' leading eight bits (stored with the digits); an entry that neither certifies
+// is computed as a plain FP64 dot product (plain_entries).  Of random data none is, of noisy
+// fluorescence-like data 0 to 1 entry in 100; data whose vectors do not overlap (sparse
+// tensors, separated bumps without noise) take more of them and more time.
 //
 // Along the contraction the two operands are equilibrated by powers of two
-// (exact): T_(a)(i, :) 2^(-F_i) against Ubar^(a)(i, :) 2^(F_i), F_i the exponent
-// of the largest entry of slice i.  A slice much larger than the others (an
-// outlying sample) then costs no digits in submodels that leave it out.
+// (exact): T_(a)(i, :) 2^(-F_i) against Ubar^(a)(i, :) 2^(F_i), F_i the mean exponent of
+// slice i's non-zero entries: slices of different scale (an outlying sample) then cost no
+// digits, and a single large entry sets no slice's scale: it is the maximum of its own
+// column of T_(a) alone, and only that column's entries need the dot products where a
+// submodel leaves it out.
 //
 // Measured (GB300), against the CUDA-core MTTKRP of every mode: an FP64 sweep of
 // 300x100x50 with 1500 columns 16.0 -> 0.46 ms, of 400x400x400 with 400 columns
@@ -67,7 +81,8 @@ constexpr int kEpiWarps = 16;
 constexpr int kTmaWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
 constexpr int kThreads = 32 * (kEpiWarps + 2);
 constexpr uint32_t kTmemCols = 512;           // all of TMEM
-constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + (2 * kStages + 5) * 8 + 16;
+constexpr uint32_t kListBytes = kEpiWarps * 32 * 16 * 2;   // the draining warps' lists (plain_entries)
+constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + kListBytes + (2 * kStages + 5) * 8 + 16;
 
 // ---- digits ---------------------------------------------------------------------
 // One operand matrix X (K x M, row stride ld; K the contraction) into stage images:
@@ -75,12 +90,15 @@ constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + (2 * kStages + 5) * 8
 // the 32-byte swizzle (16-byte chunk XOR bit 2 of the row): one bulk copy per
 // operand and stage.  A block takes 8 columns, thread (m, g) the 8-row chunks g
 // and g + 32, loaded once into registers (K <= kTtmChainMax: at most 56 chunks):
-// first each column's exponent (expo[m]: scaled magnitudes < 2^expo), then the
+// first each column's exponent (expo[m].x: scaled magnitudes < 2^expo), then the
 // digits.  sgn = +1 / -1 scales row k by 2^(+-kexp[k]).  Integer arithmetic
 // throughout: an FP64 rint per digit would take 18 us of the FP64 pipe for
 // 300 x 1500 entries.  counter: a sweep's first slicing also advances the sweep
-// counter (null otherwise).
+// counter (null otherwise).  mag: every scaled
+// magnitude in units of 2^(expo - 8), rounded down (16 nk bytes per column); expo[m].y: how
+// many are at least kFlat of them.
 constexpr int kSliceCols = 8;   // columns per block
+constexpr uint32_t kFlat = 16;  // 2^-4 of a column's power of two, in units of 2^-8
 
 // Half of every digit's field below d_0: 256 of the last one's nine bits, 64 of the
 // others' seven.
@@ -93,13 +111,15 @@ constexpr long long half_fields() {
 template <int TILE>
 __global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict__ X, int K, int64_t M, int64_t ld,
                                                         const int* __restrict__ kexp, int sgn, int nk, int64_t Mpad,
-                                                        unsigned char* __restrict__ img, int* __restrict__ expo,
+                                                        unsigned char* __restrict__ img, int2* __restrict__ expo,
+                                                        unsigned char* __restrict__ mag,
                                                         int* __restrict__ counter) {
   if (counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *counter += 1;
   constexpr int kCols = kSliceCols, kGroups = 256 / kCols;
   constexpr int kTop = 9 + 7 * (P - 2);   // position of d_0; the last digit's field has two bits more
   static_assert(2 * kGroups * 8 >= kTtmChainMax, "two chunks per thread hold a column");
   __shared__ int red[kGroups][kCols + 1];
+  __shared__ int flat[kCols];
   const int ml = threadIdx.x % kCols, g = threadIdx.x / kCols;
   for (int64_t m0 = (int64_t)blockIdx.x * kCols; m0 < Mpad; m0 += (int64_t)gridDim.x * kCols) {
     const int64_t m = m0 + ml;
@@ -127,17 +147,31 @@ __global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict
       }
     __syncthreads();   // red of the previous columns is consumed
     red[g][ml] = top;
+    if (g == 0) flat[ml] = 0;
     __syncthreads();
     for (int i = 0; i < kGroups; ++i) top = max(top, red[i][ml]);
     const bool col_bad = top == INT_MAX;
     const int E = (col_bad || top == INT_MIN) ? 0 : top - 1022;
-    if (g == 0) expo[m] = col_bad ? kTtmBadExp : E;
+    int nflat = 0;
     const int64_t tile = m / TILE;
     const int row = (int)(m - tile * TILE);
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int ch = g + j * kGroups;
       if (ch >= 2 * nk) break;
+      unsigned long long mags = 0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(x[j][e]);
+        const int ef = (int)((b >> 52) & 2047);
+        if (ef > 0 && !col_bad) {   // a normal entry: 1.m 2^(ef - 1023), scaled below 2^E
+          const int sh = E - 1 - (ef + sgn * __ldg(kexp + 8 * ch + e) - 1023);
+          const uint32_t q = sh < 8 ? (0x80u | (uint32_t)((b >> 45) & 0x7f)) >> sh : 0u;
+          mags |= (unsigned long long)q << (8 * e);
+          nflat += q >= kFlat ? 1 : 0;
+        }
+      }
+      *reinterpret_cast<unsigned long long*>(mag + (m * nk * 16 + ch * 8)) = mags;
       uint32_t w[P][4];
 #pragma unroll
       for (int pr = 0; pr < 4; ++pr) {
@@ -180,29 +214,46 @@ __global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict
       for (int s = 0; s < P; ++s)
         *reinterpret_cast<uint4*>(dst + s * (TILE * kRow)) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
     }
+    if (nflat > 0) atomicAdd(&flat[ml], nflat);
+    __syncthreads();
+    if (g == 0) expo[m] = make_int2(col_bad ? kTtmBadExp : (top == INT_MIN ? kTtmZeroExp : E), flat[ml]);
   }
 }
 
-// kexp[i] = exponent F_i with max_j |T_(a)(i, j)| < 2^F_i (0 for a zero slice);
-// *bad = 1 if an entry is Inf or NaN.
+// kexp[i] = F_i, the mean exponent of slice i's non-zero entries (0 for a zero slice): no
+// single entry, and no slice of another mode, sets it.  *bad = 1 if an entry is Inf or NaN.
 __global__ void slice_exponent_kernel(const double* __restrict__ Tn, int64_t J, int* __restrict__ kexp,
                                       int* __restrict__ bad) {
-  __shared__ int red[8];
+  __shared__ long long sums[8], counts[8];
   const int64_t i = blockIdx.x;
-  int top = 0;
+  long long sum = 0, count = 0;
+  bool finite = true;
   for (int64_t j = threadIdx.x; j < J; j += blockDim.x) {
     const unsigned long long u =
         (unsigned long long)__double_as_longlong(__ldg(Tn + i * J + j)) & 0x7fffffffffffffffull;
     const int ef = (int)(u >> 52);
-    if (u != 0) top = max(top, ef > 1 ? ef : 1);
+    finite = finite && ef != 2047;
+    if (u != 0) {
+      sum += (ef > 1 ? ef : 1) - 1022;
+      ++count;
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+  if (!finite) *bad = 1;
+  for (int o = 16; o > 0; o >>= 1) {
+    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    count += __shfl_xor_sync(0xffffffffu, count, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sums[threadIdx.x >> 5] = sum;
+    counts[threadIdx.x >> 5] = count;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)blockDim.x / 32; ++w) top = max(top, red[w]);
-    if (top == 2047) *bad = 1;
-    kexp[i] = top == 0 ? 0 : top - 1022;
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) {
+      sum += sums[w];
+      count += counts[w];
+    }
+    kexp[i] = count == 0 ? 0 : (int)(sum / count);
   }
 }
 
@@ -289,6 +340,72 @@ __device__ __forceinline__ double round_levels(long long hi, uint32_t lo, int ex
   return __longlong_as_double((long long)(q | ((unsigned long long)(s & 0x80000000u) << 32)));
 }
 
+// What certifies an entry of the product (the bound is derived at the top of this file): the
+// sum of its terms' magnitudes is at least 2^-5 of the product of the vectors' maxima,
+//  - because so many of both vectors' entries are at least 2^-4 of their maxima that at
+//    least kFlatTerms rows hold two of them (8 x 2^-8; decided for a warp's 32 columns and
+//    rows at once: dense data of one scale, at no cost per entry),
+//  - by the entry's own value, or
+//  - by the magnitudes in units of 2^-8.
+constexpr int kFlatTerms = 8;
+constexpr long long kCertain = 1ll << 30;      // 2^-5 in units of level 3 (2^-35)
+constexpr uint32_t kCertainMags = 1u << 11;    // 2^-5 in units of 2^-16
+
+// The entries of this warp's tile rows that their own value does not certify (bits of
+// pending: rows r0 .. r0 + NC - 1 of column c0 + lane).  Those that the magnitudes do not
+// certify either, and every entry of a column with a non-finite one (forced), become plain
+// FP64 dot products.  They are gathered in list and taken 32 at a time, a lane each, or fewer
+// by several lanes each: bound by the FP64 pipe (K / 2 clocks of an SM per entry), as
+// submodels that share a factor fail together, rows of whole tiles at a time.
+template <int NC>
+__device__ __noinline__ void plain_entries(const TtmArgs& a, int64_t r0, int c0, uint32_t pending, bool forced,
+                                           unsigned short* list, int lane) {
+  // the magnitudes of sixteen rows k of the contraction at a time, against all pending rows
+  // together: their loads are in flight together, and sixteen are mostly enough
+  uint32_t open = forced ? 0u : pending;
+  const uint4* mr = reinterpret_cast<const uint4*>(a.rmag) + r0 * a.nk;
+  const uint4* mc = reinterpret_cast<const uint4*>(a.cmag) + (int64_t)(c0 + lane) * a.nk;   // padded, as the rows
+  uint32_t sum[NC] = {};
+  for (int w = 0; w < a.nk && __any_sync(0xffffffffu, open != 0); ++w) {
+    const uint4 y = __ldg(mc + w);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+      const uint4 x = __ldg(mr + (int64_t)k * a.nk + w);
+      sum[k] = __dp4a(x.x, y.x, __dp4a(x.y, y.y, __dp4a(x.z, y.z, __dp4a(x.w, y.w, sum[k]))));
+      if (sum[k] >= kCertainMags) open &= ~(1u << k);
+    }
+  }
+  if (!forced) pending = open;
+  if (!__any_sync(0xffffffffu, pending != 0)) return;
+  int at = __popc(pending);
+  for (int o = 1; o < 32; o <<= 1) {
+    const int below = __shfl_up_sync(0xffffffffu, at, o);
+    if (lane >= o) at += below;
+  }
+  const int total = __shfl_sync(0xffffffffu, at, 31);
+  at -= __popc(pending);
+  for (; pending != 0; pending &= pending - 1)
+    list[at++] = (unsigned short)(((__ffs((int)pending) - 1) << 5) | lane);
+  __syncwarp();   // the list, and the digits' sums before the stores below
+  for (int base = 0; base < total; base += 32) {
+    const int cnt = total - base < 32 ? total - base : 32;
+    const int lg = cnt > 16 ? 0 : __clz(cnt > 1 ? cnt - 1 : 0) - 27;   // 32 >> lg entries at a time
+    const int e = lane >> lg, part = lane & ((1 << lg) - 1);
+    const int code = list[base + (e < cnt ? e : 0)];
+    const int64_t r = r0 + (code >> 5);
+    const int c = c0 + (code & 31);
+    const double *t = a.Tn + r, *u = a.U + c;
+    double acc = 0.0;
+#pragma unroll 8
+    for (int i = part; i < a.K; i += 1 << lg)
+      acc = fma(__ldg(t + (int64_t)i * a.J), __ldg(u + (int64_t)i * a.C), acc);
+    __syncwarp();
+    for (int o = 1; o < (1 << lg); o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (e < cnt && part == 0) a.Y[r * a.C + c] = acc;
+  }
+  __syncwarp();   // the list is free again
+}
+
 // Persistent: one CTA per SM (all of TMEM, 4 x 48 KB stages) walks the 128 x
 // BN tiles of Y, C tiles fastest so that the CTAs in flight share T's images in L2.
 //   warp 16  TMA: one lane refills the ring in order, across tile boundaries
@@ -309,7 +426,7 @@ __device__ __forceinline__ double round_levels(long long hi, uint32_t lo, int ex
 // against 147 with BN = 64, 100x60x60x40 over 100 rows 828 against 767; over up to 64
 // rows the halves are even, and fill the SMs more evenly.
 template <int BN>
-__global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const __grid_constant__ TtmArgs a) {
   constexpr int NB = ttm_sets(BN);          // accumulator sets
   constexpr int NC = BN / 4;                // rows r of a draining warp
   constexpr int G = 256 / BN;               // digits of T stacked per MMA
@@ -319,7 +436,8 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* ring =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)kStages * kStage);
+  unsigned short* lists = reinterpret_cast<unsigned short*>(ring + (size_t)kStages * kStage);
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)kStages * kStage + kListBytes);
   uint64_t* empty = full + kStages;
   uint64_t* accum = empty + kStages;      // [2] a tile's MMAs into set b are complete
   uint64_t* tmem_empty = accum + 2;       // [2] the drain has read set b
@@ -431,9 +549,10 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
       const int64_t tr = t / a.tiles_c;
       const int c = (int)(t - tr * a.tiles_c) * kTileM + quarter * 32 + lane;
       const int64_t r0 = tr * BN + NC * grp;
-      const int ec = __ldg(a.cexp + c);   // padded to whole tiles, as rexp
+      const int2 ce = __ldg(a.cexp + c);   // padded to whole tiles, as rexp
+      const int ec = ce.x;
       // this warp's row exponents, in flight while the tile's MMAs run
-      const int re = __ldg(a.rexp + r0 + (lane < NC ? lane : 0));
+      const int2 re = __ldg(a.rexp + r0 + (lane < NC ? lane : 0));
       const uint32_t b = use % NB;
       const uint32_t base = tmem + ((uint32_t)(quarter * 32) << 16) + b * kSetCols + (uint32_t)(NC * grp);
       bool have = wait_sleepy(&accum[b], (use / NB) & 1u, abort_flag, a.err, 5);
@@ -448,21 +567,20 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const TtmArgs a) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&tmem_empty[b]);
       // ... and round and store them meanwhile
-      double* y = static_cast<double*>(a.Y) + r0 * a.C + c;
+      const bool forced = ec == kTtmBadExp;
+      double* y = a.Y + r0 * a.C + c;
+      uint32_t pending = 0;   // rows whose sum is below kCertain of the vectors' maxima
 #pragma unroll
       for (int k = 0; k < NC; ++k, y += a.C) {
-        const int64_t r = r0 + k;
-        const int er = __shfl_sync(0xffffffffu, re, k);
-        if (r >= a.J || c >= a.C) continue;
-        if (ec == kTtmBadExp) {
-          double acc = 0.0;
-          for (int i = 0; i < a.K; ++i)
-            acc = fma(__ldg(a.Tn + (int64_t)i * a.J + r), __ldg(a.U + (int64_t)i * a.C + c), acc);
-          *y = acc;
-        } else {
-          *y = round_levels(hi[k], lo[k], ec + er);
-        }
+        const int er = __shfl_sync(0xffffffffu, re.x, k);
+        if (r0 + k >= a.J || c >= a.C) continue;
+        const bool sure = (unsigned long long)(hi[k] + kCertain) >= 2ull * kCertain;
+        if (forced || (!sure && er != kTtmZeroExp && ec != kTtmZeroExp)) pending |= 1u << k;
+        if (!forced) *y = round_levels(hi[k], lo[k], ec + er);
       }
+      const int rflat = __reduce_min_sync(0xffffffffu, re.y);
+      if (ce.y + rflat >= a.K + kFlatTerms) pending = 0;
+      if (__any_sync(0xffffffffu, pending != 0)) plain_entries<NC>(a, r0, c - lane, pending, forced, lists + warp * (32 * NC), lane);
     }
   }
 
@@ -545,11 +663,11 @@ __global__ void __launch_bounds__(256) contract_kernel(const double* __restrict_
 
 template <int TILE>
 cudaError_t launch_slice(const double* X, int K, int64_t M, int64_t ld, const int* kexp, int sgn, unsigned char* img,
-                         int* expo, int* counter, cudaStream_t s) {
+                         int2* expo, unsigned char* mag, int* counter, cudaStream_t s) {
   const int64_t Mpad = (M + TILE - 1) / TILE * TILE;
   const int64_t blocks = Mpad / kSliceCols;
   slice_f64_kernel<TILE><<<(unsigned)(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
-      X, K, M, ld, kexp, sgn, ttm_ksteps(K), Mpad, img, expo, counter);
+      X, K, M, ld, kexp, sgn, ttm_ksteps(K), Mpad, img, expo, mag, counter);
   return cudaGetLastError();
 }
 
@@ -560,15 +678,15 @@ cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt, int* rexp,
-                                cudaStream_t s) {
-  return ttm_tile_r(I) == 32 ? launch_slice<32>(Tn, I, J, J, kexp, -1, Bt, rexp, nullptr, s)
-                             : launch_slice<64>(Tn, I, J, J, kexp, -1, Bt, rexp, nullptr, s);
+cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt, int2* rexp,
+                                unsigned char* rmag, cudaStream_t s) {
+  return ttm_tile_r(I) == 32 ? launch_slice<32>(Tn, I, J, J, kexp, -1, Bt, rexp, rmag, nullptr, s)
+                             : launch_slice<64>(Tn, I, J, J, kexp, -1, Bt, rexp, rmag, nullptr, s);
 }
 
-cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At, int* cexp,
-                                int* counter, cudaStream_t s) {
-  return launch_slice<kTileM>(U, I, C, C, kexp, +1, At, cexp, counter, s);
+cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At, int2* cexp,
+                                unsigned char* cmag, int* counter, cudaStream_t s) {
+  return launch_slice<kTileM>(U, I, C, C, kexp, +1, At, cexp, cmag, counter, s);
 }
 
 cudaError_t prepare_ttm(int K) {
