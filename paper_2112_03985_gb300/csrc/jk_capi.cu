@@ -563,6 +563,8 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
     g.Bt = t.Bt[a];
     g.cexp = t.cexp[a];
     g.rexp = t.rexp[a];
+    g.kexp = t.kexp[a];
+    g.power = t.ypower[a];
     g.cmag = t.cmag[a];
     g.rmag = t.rmag[a];
     g.K = (int)h->dims[a];
@@ -576,8 +578,8 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
     g.Tn = h->Tn64[a];
     g.U = U[a];
     g.err = h->d_err;
-    JK_CUDA(h, launch_slice_factor(U[a], g.K, h->C, t.kexp[a], t.At, t.cexp[a], t.cmag[a], st.counter,
-                                   h->stream));
+    JK_CUDA(h, launch_slice_factor(U[a], g.K, h->C, t.kexp[a], t.At, t.cexp[a], t.cmag[a],
+                                   N == 2 ? nullptr : t.range[a], t.ypower[a], st.counter, h->stream));
     st.counter = nullptr;
     JK_CUDA(h, launch_ttm(g, h->num_sms, h->stream));
     t.ran = true;
@@ -591,6 +593,7 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
   for (int k = 0; k < N; ++k)
     if (have_z ? (k != st.z_a && k != st.z_q) : k != a) rest.push_back(k);
   if (have_z) X = t.Z;
+  const int* power = have_z ? t.zpower : t.ypower[a];
   int w = 0;
   while (rest.size() > 1) {
     size_t pos = rest.size() - 1;
@@ -614,7 +617,9 @@ jkcals_status enqueue_ttm(jkcals_ctx* h, int n, int a, double* const* U, TtmStat
       out = t.W[w];
       w ^= 1;
     }
-    JK_CUDA(h, launch_contract(X, H, (int)h->dims[q], L, h->C, U[q], S, out, h->stream));
+    int* out_power = out == part ? nullptr : out == t.Z ? t.zpower : t.wpower[out == t.W[1]];
+    JK_CUDA(h, launch_contract(X, H, (int)h->dims[q], L, h->C, U[q], S, power, out_power, out, h->stream));
+    power = out_power;
     *kernels += 1;
     X = out;
     rest.erase(rest.begin() + pos);
@@ -1034,13 +1039,15 @@ size_t ttm_part_elems(const jkcals_ctx* h, int n) {
 // them and runs on that kernel.
 void ttm_drop(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
-  void* all[] = {t.At, t.Y, t.Z, t.W[0], t.W[1]};
+  void* all[] = {t.At, t.Y, t.Z, t.W[0], t.W[1], t.zpower, t.wpower[0], t.wpower[1]};
   for (void* p : all) dfree(h, p, true);
   for (int n = 0; n < kMaxModes; ++n) {
     dfree(h, t.Bt[n], true);
     dfree(h, t.kexp[n], true);
     dfree(h, t.rexp[n], true);
     dfree(h, t.cexp[n], true);
+    dfree(h, t.range[n], true);
+    dfree(h, t.ypower[n], true);
     dfree(h, t.rmag[n], true);
     dfree(h, t.cmag[n], true);
   }
@@ -1068,6 +1075,8 @@ jkcals_status create_ttm_images(jkcals_ctx* h) {
       JK_CUDA(h, launch_slice_exponents(h->Tn64[a], h->dims[a], h->J[a], t.kexp[a], d_bad, st));
       JK_TRY(dalloc_t(h, &t.rmag[a], (size_t)round_up(h->J[a], rows) * ttm_ksteps((int)h->dims[a]) * 16));
       JK_CUDA(h, launch_slice_tensor(h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], t.rmag[a], st));
+      JK_TRY(dalloc_t(h, &t.range[a], 1));
+      JK_CUDA(h, launch_range(t.kexp[a], (int)h->dims[a], t.rexp[a], h->J[a], t.range[a], st));
     }
     return JKCALS_OK;
   };
@@ -1092,6 +1101,7 @@ jkcals_status create_ttm_workspace(jkcals_ctx* h) {
     for (int a : t.modes) {
       if (a < 0) continue;
       JK_TRY(dalloc_t(h, &t.cexp[a], (size_t)round_up(h->C, kTtmTileC)));
+      JK_TRY(dalloc_t(h, &t.ypower[a], (size_t)round_up(h->C, kTtmTileC)));
       JK_TRY(dalloc_t(h, &t.cmag[a], (size_t)round_up(h->C, kTtmTileC) * ttm_ksteps((int)h->dims[a]) * 16));
       at = std::max(at, ttm_image_bytes((int)h->dims[a], h->C, kTtmTileC));
       if (h->N > 2) y = std::max(y, (size_t)h->J[a] * h->C);
@@ -1106,8 +1116,14 @@ jkcals_status create_ttm_workspace(jkcals_ctx* h) {
     JK_TRY(dalloc(h, &img, at));
     t.At = static_cast<unsigned char*>(img);
     if (y > 0) JK_TRY(dalloc_t(h, &t.Y, y));
-    if (z > 0) JK_TRY(dalloc_t(h, &t.Z, z));
-    for (int k = 0; k < 2 && w > 0; ++k) JK_TRY(dalloc_t(h, &t.W[k], w));
+    if (z > 0) {
+      JK_TRY(dalloc_t(h, &t.Z, z));
+      JK_TRY(dalloc_t(h, &t.zpower, (size_t)h->C));
+    }
+    for (int k = 0; k < 2 && w > 0; ++k) {
+      JK_TRY(dalloc_t(h, &t.W[k], w));
+      JK_TRY(dalloc_t(h, &t.wpower[k], (size_t)h->C));
+    }
     JK_TRY(create_error_word(h));
     for (int a : t.modes)
       if (a >= 0) JK_CUDA(h, prepare_ttm((int)h->dims[a]));

@@ -172,6 +172,10 @@ struct jkcals_ctx {
     int* kexp[jk::kMaxModes] = {nullptr};          // I_a slice exponents
     int2* rexp[jk::kMaxModes] = {nullptr};         // exponents of T_(a)'s scaled columns (padded to tiles)
     unsigned char* rmag[jk::kMaxModes] = {nullptr};   // their magnitudes' leading bits
+    int2* range[jk::kMaxModes] = {nullptr};        // exponents of T_(a) (jk_ttm.cu)
+    int* ypower[jk::kMaxModes] = {nullptr};        // powers of two that the columns of mode a's product,
+    int* zpower = nullptr;                         // of Z
+    int* wpower[2] = {nullptr, nullptr};           // and of W are held without
     unsigned char* At = nullptr;                   // digit images of Ubar^(a), rewritten per product
     int2* cexp[jk::kMaxModes] = {nullptr};         // exponents of its scaled columns (padded to tiles)
     unsigned char* cmag[jk::kMaxModes] = {nullptr};   // their magnitudes' leading bits
@@ -376,6 +380,8 @@ struct TtmArgs {
   int nk, K, C, tiles_c;
   int64_t J, tiles_r;
   double* Y;                 // J x C
+  const int* kexp;           // per row of the contraction: its slice's exponent
+  const int* power;          // per column c: Y holds it times 2^-power
   const double* Tn;          // T_(a), K x J (entries that the digits do not carry)
   const double* U;           // Ubar^(a), K x C
   int* err;
@@ -384,16 +390,19 @@ inline size_t ttm_image_bytes(int K, int64_t M, int tile) {   // eight digits of
   return (size_t)((M + tile - 1) / tile) * ttm_ksteps(K) * 8 * tile * 32;
 }
 cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* kexp, int* bad, cudaStream_t s);
+cudaError_t launch_range(const int* kexp, int K, const int2* rexp, int64_t J, int2* range, cudaStream_t s);
 cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt,
                                 int2* rexp, unsigned char* rmag, cudaStream_t s);
 cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At,
-                                int2* cexp, unsigned char* cmag, int* counter, cudaStream_t s);
+                                int2* cexp, unsigned char* cmag, const int2* range, int* power, int* counter,
+                                cudaStream_t s);
 cudaError_t prepare_ttm(int K);
 cudaError_t launch_ttm(const TtmArgs& a, int num_sms, cudaStream_t s);
-// out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c]
+// out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c], column c of X times
+// 2^power[c]; out_power: the powers that out's columns are left without (null: none)
 int contract_splits(int64_t HL, int Mm, int C);
-cudaError_t launch_contract(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S, double* out,
-                            cudaStream_t s);
+cudaError_t launch_contract(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
+                            const int* power, int* out_power, double* out, cudaStream_t s);
 
 // Storage of split-K partials: FP64, FP32, or an unevaluated FP32 pair (hi, lo).
 constexpr int kPartF64 = 0, kPartF32 = 1, kPartF32x2 = 2;

@@ -108,11 +108,21 @@ constexpr long long half_fields() {
   return h;
 }
 
+// Columns whose products T Ubar^(a) (or those times another factor) may leave FP64's range
+// where the Khatri-Rao product does not: a tensor or a factor of extreme scale (beyond about
+// 1e60, 1e120).  Y holds such a column times 2^-column_power, so that it has T's own scale,
+// and the contractions carry the power to the end.  ec: the column's exponent.
+__device__ __forceinline__ int column_power(int ec, int2 range) {
+  const bool ordinary = abs(range.x) <= 200 && abs(ec) <= 400 && ec + range.y <= 1014;
+  return ordinary ? 0 : ec - range.x;
+}
+
 template <int TILE>
 __global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict__ X, int K, int64_t M, int64_t ld,
                                                         const int* __restrict__ kexp, int sgn, int nk, int64_t Mpad,
                                                         unsigned char* __restrict__ img, int2* __restrict__ expo,
                                                         unsigned char* __restrict__ mag,
+                                                        const int2* __restrict__ range, int* __restrict__ power,
                                                         int* __restrict__ counter) {
   if (counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *counter += 1;
   constexpr int kCols = kSliceCols, kGroups = 256 / kCols;
@@ -216,7 +226,10 @@ __global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict
     }
     if (nflat > 0) atomicAdd(&flat[ml], nflat);
     __syncthreads();
-    if (g == 0) expo[m] = make_int2(col_bad ? kTtmBadExp : (top == INT_MIN ? kTtmZeroExp : E), flat[ml]);
+    if (g == 0) {
+      expo[m] = make_int2(col_bad ? kTtmBadExp : (top == INT_MIN ? kTtmZeroExp : E), flat[ml]);
+      if (power != nullptr) power[m] = range == nullptr || col_bad || top == INT_MIN ? 0 : column_power(E, *range);
+    }
   }
 }
 
@@ -254,6 +267,25 @@ __global__ void slice_exponent_kernel(const double* __restrict__ Tn, int64_t J, 
       count += counts[w];
     }
     kexp[i] = count == 0 ? 0 : (int)(sum / count);
+  }
+}
+
+// range: g, about T's own exponent, at most what keeps every sum of T(., r) and a column of
+// size 1 finite, and the largest exponent of rexp.
+__global__ void range_kernel(const int* __restrict__ kexp, int K, const int2* __restrict__ rexp, int64_t J,
+                             int2* __restrict__ range) {
+  __shared__ int red[32];
+  int top = kTtmZeroExp;
+#pragma unroll 8
+  for (int64_t r = threadIdx.x; r < J; r += blockDim.x) top = max(top, __ldg(rexp + r).x);
+  top = __reduce_max_sync(0xffffffffu, top);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = top;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int sum = 0;
+    for (int i = 0; i < K; ++i) sum += __ldg(kexp + i);
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) top = max(top, red[w]);
+    *range = make_int2(min(sum / K, 1014 - top), top);   // K < 2^9 terms below 2^1014
   }
 }
 
@@ -395,10 +427,19 @@ __device__ __noinline__ void plain_entries(const TtmArgs& a, int64_t r0, int c0,
     const int64_t r = r0 + (code >> 5);
     const int c = c0 + (code & 31);
     const double *t = a.Tn + r, *u = a.U + c;
+    const int ec = __ldg(a.cexp + c).x;
+    const int power = __ldg(a.power + c);
     double acc = 0.0;
+    if (power != 0) {
+      for (int i = part; i < a.K; i += 1 << lg) {
+        const int f = __ldg(a.kexp + i);
+        acc = fma(scalbn(__ldg(t + (int64_t)i * a.J), ec - power - f), scalbn(__ldg(u + (int64_t)i * a.C), f - ec), acc);
+      }
+    } else {
 #pragma unroll 8
-    for (int i = part; i < a.K; i += 1 << lg)
-      acc = fma(__ldg(t + (int64_t)i * a.J), __ldg(u + (int64_t)i * a.C), acc);
+      for (int i = part; i < a.K; i += 1 << lg)
+        acc = fma(__ldg(t + (int64_t)i * a.J), __ldg(u + (int64_t)i * a.C), acc);
+    }
     __syncwarp();
     for (int o = 1; o < (1 << lg); o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (e < cnt && part == 0) a.Y[r * a.C + c] = acc;
@@ -551,6 +592,7 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const __grid_constant_
       const int64_t r0 = tr * BN + NC * grp;
       const int2 ce = __ldg(a.cexp + c);   // padded to whole tiles, as rexp
       const int ec = ce.x;
+      const int power = __ldg(a.power + c);
       // this warp's row exponents, in flight while the tile's MMAs run
       const int2 re = __ldg(a.rexp + r0 + (lane < NC ? lane : 0));
       const uint32_t b = use % NB;
@@ -568,6 +610,7 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const __grid_constant_
       if (lane == 0) mbar_arrive(&tmem_empty[b]);
       // ... and round and store them meanwhile
       const bool forced = ec == kTtmBadExp;
+      const int ex = ec - power;
       double* y = a.Y + r0 * a.C + c;
       uint32_t pending = 0;   // rows whose sum is below kCertain of the vectors' maxima
 #pragma unroll
@@ -576,7 +619,7 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const __grid_constant_
         if (r0 + k >= a.J || c >= a.C) continue;
         const bool sure = (unsigned long long)(hi[k] + kCertain) >= 2ull * kCertain;
         if (forced || (!sure && er != kTtmZeroExp && ec != kTtmZeroExp)) pending |= 1u << k;
-        if (!forced) *y = round_levels(hi[k], lo[k], ec + er);
+        if (!forced) *y = round_levels(hi[k], lo[k], ex + er);
       }
       const int rflat = __reduce_min_sync(0xffffffffu, re.y);
       if (ce.y + rflat >= a.K + kFlatTerms) pending = 0;
@@ -593,13 +636,28 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const __grid_constant_
 }
 
 // ---- contraction with one more factor ------------------------------------------------
+// v 2^e in exact factors (but for an underflow), without scalbn's registers.
+__device__ __forceinline__ double times_power(double v, int e) {
+#pragma unroll 1
+  while (e != 0) {
+    const int k = e > 1000 ? 1000 : (e < -1000 ? -1000 : e);
+    v *= __hiloint2double((k + 1023) << 20, 0);
+    e -= k;
+  }
+  return v;
+}
+
 // out[s][h][l][c] = sum over split s of m of X[h][m][l][c] U[m][c].  A thread takes RB
 // outputs (h, l) of V adjacent columns: one load of U serves RB of X, and a load of two
-// columns is 16 bytes.  Bound: X read once, or the FP64 pipe's two multiply-adds per clock
+// columns is 16 bytes.  A column that X holds times a power of two (see column_power) is
+// contracted with its factor's column scaled to at most 1; the powers go into the result, or,
+// if that is contracted again, to out_power.  Bound: X read once, or the FP64 pipe's
+// two multiply-adds per clock
 // and SM (400x400x400, 400 columns: 130 us, 512 MB at 3.9 TB/s and 490 G multiply-adds/s).
 template <int RB, int V>
 __global__ void __launch_bounds__(256) contract_kernel(const double* __restrict__ X, int64_t H, int Mm, int64_t L,
                                                        int C, const double* __restrict__ U, int mchunk,
+                                                       const int* __restrict__ power, int* __restrict__ out_power,
                                                        double* __restrict__ out) {
   constexpr int UN = RB * V >= 8 ? 2 : (RB * V >= 4 ? 4 : 8);   // terms loaded together
   const int64_t HL = H * L, groups = (HL + RB - 1) / RB;
@@ -630,6 +688,9 @@ __global__ void __launch_bounds__(256) contract_kernel(const double* __restrict_
       v[0] = __ldg(p);
     }
   };
+  bool shifted = false;
+#pragma unroll
+  for (int w = 0; w < V; ++w) shifted = shifted || __ldg(power + c + w) != 0;
   auto terms = [&](auto nt) {   // N <= UN terms, all loaded first
     constexpr int N = decltype(nt)::value;
     double uv[N][V], xv[N][RB][V];
@@ -649,9 +710,35 @@ __global__ void __launch_bounds__(256) contract_kernel(const double* __restrict_
 #pragma unroll
     for (int q = 0; q < RB; ++q) x[q] += N * step;
   };
-  int m = mb;
-  for (; m + UN <= me; m += UN) terms(std::integral_constant<int, UN>{});
-  for (; m < me; ++m) terms(std::integral_constant<int, 1>{});
+  if (shifted) {
+#pragma unroll
+    for (int w = 0; w < V; ++w) {
+      int pw = __ldg(power + c + w);
+      double most = 0.0;
+#pragma unroll 1
+      for (int k = 0; k < Mm; ++k) most = fmax(most, fabs(__ldg(U + (int64_t)k * C + c + w)));
+      const int ue = pw != 0 && most > 0.0 && isfinite(most) ? (__double2hiint(most) >> 20) - 1022 : 0;
+#pragma unroll 1
+      for (int k = mb; k < me; ++k) {
+        const double uv = times_power(__ldg(U + (int64_t)k * C + c + w), -ue);
+#pragma unroll
+        for (int q = 0; q < RB; ++q) acc[q][w] = fma(__ldg(x[q] + (k - mb) * step + w), uv, acc[q][w]);
+      }
+      pw += ue;   // true: acc 2^pw
+      if (out_power != nullptr)
+        out_power[c + w] = pw;   // the same from every thread of the column
+      else
+#pragma unroll
+        for (int q = 0; q < RB; ++q) acc[q][w] = times_power(acc[q][w], pw);
+    }
+  } else {
+    int m = mb;
+    for (; m + UN <= me; m += UN) terms(std::integral_constant<int, UN>{});
+    for (; m < me; ++m) terms(std::integral_constant<int, 1>{});
+    if (out_power != nullptr)
+#pragma unroll
+      for (int w = 0; w < V; ++w) out_power[c + w] = 0;
+  }
 #pragma unroll
   for (int q = 0; q < RB; ++q)
     if (g * RB + q < HL) {
@@ -663,11 +750,11 @@ __global__ void __launch_bounds__(256) contract_kernel(const double* __restrict_
 
 template <int TILE>
 cudaError_t launch_slice(const double* X, int K, int64_t M, int64_t ld, const int* kexp, int sgn, unsigned char* img,
-                         int2* expo, unsigned char* mag, int* counter, cudaStream_t s) {
+                         int2* expo, unsigned char* mag, const int2* range, int* power, int* counter, cudaStream_t s) {
   const int64_t Mpad = (M + TILE - 1) / TILE * TILE;
   const int64_t blocks = Mpad / kSliceCols;
   slice_f64_kernel<TILE><<<(unsigned)(blocks < 65535 ? blocks : 65535), 256, 0, s>>>(
-      X, K, M, ld, kexp, sgn, ttm_ksteps(K), Mpad, img, expo, mag, counter);
+      X, K, M, ld, kexp, sgn, ttm_ksteps(K), Mpad, img, expo, mag, range, power, counter);
   return cudaGetLastError();
 }
 
@@ -678,15 +765,20 @@ cudaError_t launch_slice_exponents(const double* Tn, int64_t I, int64_t J, int* 
   return cudaGetLastError();
 }
 
+cudaError_t launch_range(const int* kexp, int K, const int2* rexp, int64_t J, int2* range, cudaStream_t s) {
+  range_kernel<<<1, 1024, 0, s>>>(kexp, K, rexp, J, range);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_slice_tensor(const double* Tn, int I, int64_t J, const int* kexp, unsigned char* Bt, int2* rexp,
                                 unsigned char* rmag, cudaStream_t s) {
-  return ttm_tile_r(I) == 32 ? launch_slice<32>(Tn, I, J, J, kexp, -1, Bt, rexp, rmag, nullptr, s)
-                             : launch_slice<64>(Tn, I, J, J, kexp, -1, Bt, rexp, rmag, nullptr, s);
+  return ttm_tile_r(I) == 32 ? launch_slice<32>(Tn, I, J, J, kexp, -1, Bt, rexp, rmag, nullptr, nullptr, nullptr, s)
+                             : launch_slice<64>(Tn, I, J, J, kexp, -1, Bt, rexp, rmag, nullptr, nullptr, nullptr, s);
 }
 
 cudaError_t launch_slice_factor(const double* U, int I, int C, const int* kexp, unsigned char* At, int2* cexp,
-                                unsigned char* cmag, int* counter, cudaStream_t s) {
-  return launch_slice<kTileM>(U, I, C, C, kexp, +1, At, cexp, cmag, counter, s);
+                                unsigned char* cmag, const int2* range, int* power, int* counter, cudaStream_t s) {
+  return launch_slice<kTileM>(U, I, C, C, kexp, +1, At, cexp, cmag, range, power, counter, s);
 }
 
 cudaError_t prepare_ttm(int K) {
@@ -730,20 +822,20 @@ int contract_splits(int64_t HL, int Mm, int C) {
   return (Mm + chunk - 1) / chunk;
 }
 
-cudaError_t launch_contract(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S, double* out,
-                            cudaStream_t s) {
+cudaError_t launch_contract(const double* X, int64_t H, int Mm, int64_t L, int C, const double* U, int S,
+                            const int* power, int* out_power, double* out, cudaStream_t s) {
   const int64_t HL = H * L;
   const int chunk = (Mm + S - 1) / S;
   const int V = contract_vec(C), RB = contract_rb(HL, Mm, C, V);
   const dim3 grid((unsigned)(((HL + RB - 1) / RB * (C / V) + 255) / 256), (unsigned)S);
   if (RB == 4 && V == 2)
-    contract_kernel<4, 2><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+    contract_kernel<4, 2><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, power, out_power, out);
   else if (RB == 4)
-    contract_kernel<4, 1><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+    contract_kernel<4, 1><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, power, out_power, out);
   else if (V == 2)
-    contract_kernel<1, 2><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+    contract_kernel<1, 2><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, power, out_power, out);
   else
-    contract_kernel<1, 1><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, out);
+    contract_kernel<1, 1><<<grid, 256, 0, s>>>(X, H, Mm, L, C, U, chunk, power, out_power, out);
   return cudaGetLastError();
 }
 

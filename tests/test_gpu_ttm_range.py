@@ -135,3 +135,34 @@ def test_sparse_tensor(density):
     U = [rng.standard_normal((I, sum(ranks))) for I in dims]
     U[1][:, 3] = 0.0
     _check(T, left, ranks, U)
+
+
+@pytest.mark.parametrize("dims", [(40, 33, 61), (30, 17, 25, 31)], ids=lambda d: "x".join(map(str, d)))
+@pytest.mark.parametrize("power", [1, -1])
+def test_products_beyond_the_range_that_another_factor_brings_back(dims, power):
+    """T times one factor leaves FP64's range, the Khatri-Rao product of the factors does not."""
+    rng = np.random.default_rng(17)
+    ranks = [5] * 41
+    left = [[] for _ in ranks]
+    T = rng.standard_normal(dims)
+    U = [rng.standard_normal((I, sum(ranks))) for I in dims]
+    T[3, 4, 5] = 1e9
+    U[1][4, ::7] = 0.0   # entries of every kind: by digits and as plain sums
+    refs = [_mttkrp(T, U, n) for n in range(len(dims))]
+    bars = [BAR * _mttkrp(np.abs(T), [np.abs(u) for u in U], n) for n in range(len(dims))]
+    for big in range(len(dims)):
+        for small in range(len(dims)):
+            if big == small:
+                continue
+            V = [u.copy() for u in U]
+            V[big] = np.ldexp(U[big], 560 * power)
+            V[small] = np.ldexp(U[small], -700 * power)
+            S = np.ldexp(T, 480 * power)
+            h, native = _handles(S, left, ranks, V)
+            with h, native:
+                for n in range(len(dims)):
+                    if n in (big, small):
+                        continue
+                    for x in (native, h):
+                        got = np.ldexp(np.asarray(x.mttkrp(n)), -340 * power)
+                        assert (np.abs(got - refs[n]) <= bars[n]).all(), (big, small, n)
