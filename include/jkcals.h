@@ -25,7 +25,9 @@
  *    Factor multi-matrices are row-major I_n x C, FP64.
  *  - Streams.  Work is enqueued on the stream given at create (NULL = the
  *    legacy default stream).  Calls that return values in host memory
- *    synchronise that stream before returning.
+ *    synchronise that stream before returning.  Calls that wait for the stream
+ *    also report a bounded wait of a kernel that expired since the last such
+ *    call (JKCALS_ERR_TIMEOUT).
  *  - Errors.  Every call returns a jkcals_status and never throws across the
  *    ABI.  jkcals_last_error() gives a thread-local message for the last
  *    failing call of the calling thread.  A sticky CUDA error maps to
@@ -375,6 +377,15 @@ jkcals_status jkcals_loss_history(jkcals_t h, int nsweeps, double* losses);
  * or JKCALS_ERR_CUDA otherwise.  Synchronises the device.
  */
 jkcals_status jkcals_selftest_bounded_wait(double limit_ms, int* code, double* left_after_ms);
+
+/*
+ * The same for the report of an expired wait: stores code (> 0) in the handle's
+ * error word, in the order of its stream, as a kernel does whose wait expires.
+ * The next call on the handle that waits for its stream returns
+ * JKCALS_ERR_TIMEOUT, once.  JKCALS_ERR_STATE for a handle without bounded waits
+ * (FP64 on the CUDA cores).
+ */
+jkcals_status jkcals_selftest_expired_wait(jkcals_t h, int code);
 
 /* Block until the handle's stream is idle. */
 jkcals_status jkcals_sync(jkcals_t h);

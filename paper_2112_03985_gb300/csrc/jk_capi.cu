@@ -899,8 +899,15 @@ jkcals_status check_device_error(jkcals_ctx* h, bool synced = false) {
   }
   if (err != 0)
     return fail(JKCALS_ERR_TIMEOUT, "a bounded wait in the tensor-core MTTKRP expired (code " +
-                                        std::to_string(err) + "); results of that call are invalid");
+                                        std::to_string(err) + "); results since the last call that waited for the handle are invalid");
   return JKCALS_OK;
+}
+
+// Every call that waits for the handle's stream reports a wait that expired before it: calls
+// that only enqueue work leave theirs to the next of these.
+jkcals_status sync_stream(jkcals_ctx* h) {
+  JK_CUDA(h, cudaStreamSynchronize(h->stream));
+  return check_device_error(h, true);
 }
 
 // Set the split-K factor of mode n's MTTKRP to about S (clamped to the
@@ -1544,7 +1551,7 @@ jkcals_status jkcals_kernel_times(jkcals_t h, double* ms) {
   JK_TRY(check_handle(h));
   if (ms == nullptr) return fail(JKCALS_ERR_ARG, "ms is NULL");
   if (!h->opt.kernel_timing) return fail(JKCALS_ERR_STATE, "kernel_timing was not enabled at create");
-  JK_CUDA(h, cudaStreamSynchronize(h->stream));
+  JK_TRY(sync_stream(h));
   for (int n = 0; n < h->N; ++n) {
     float t = 0.f;
     cudaError_t e = cudaEventElapsedTime(&t, h->ev_start[n], h->ev_stop[n]);
@@ -1714,7 +1721,7 @@ jkcals_status jkcals_jackknife_se(jkcals_t h, int ref_block, const double* const
   }
   if (perm != nullptr)
     JK_CUDA(h, cudaMemcpyAsync(perm, a.perm, sizeof(int32_t) * G * R, cudaMemcpyDefault, h->stream));
-  JK_CUDA(h, cudaStreamSynchronize(h->stream));
+  JK_TRY(sync_stream(h));
   if (n_submodels != nullptr) *n_submodels = G;
   return JKCALS_OK;
 }
@@ -1995,8 +2002,7 @@ jkcals_status jkcals_get_factors(jkcals_t h, double* const* U) {
     if (U[n] == nullptr) return fail(JKCALS_ERR_ARG, "U[n] is NULL");
   for (int n = 0; n < h->N; ++n)
     JK_CUDA(h, cudaMemcpyAsync(U[n], h->U[n], sizeof(double) * h->dims[n] * h->C, cudaMemcpyDefault, h->stream));
-  JK_CUDA(h, cudaStreamSynchronize(h->stream));
-  return JKCALS_OK;
+  return sync_stream(h);
 }
 
 jkcals_status jkcals_set_factors(jkcals_t h, const double* const* U) {
@@ -2007,16 +2013,14 @@ jkcals_status jkcals_set_factors(jkcals_t h, const double* const* U) {
   for (int n = 0; n < h->N; ++n)
     JK_CUDA(h, cudaMemcpyAsync(h->U[n], U[n], sizeof(double) * h->dims[n] * h->C, cudaMemcpyDefault, h->stream));
   JK_TRY(refresh_factor_state(h));
-  JK_CUDA(h, cudaStreamSynchronize(h->stream));
-  return JKCALS_OK;
+  return sync_stream(h);
 }
 
 jkcals_status jkcals_get_block_status(jkcals_t h, int32_t* status) {
   JK_TRY(check_handle(h));
   if (status == nullptr) return fail(JKCALS_ERR_ARG, "status is NULL");
   JK_CUDA(h, cudaMemcpyAsync(status, h->d_status, sizeof(int32_t) * h->K, cudaMemcpyDefault, h->stream));
-  JK_CUDA(h, cudaStreamSynchronize(h->stream));
-  return JKCALS_OK;
+  return sync_stream(h);
 }
 
 jkcals_status jkcals_grad(jkcals_t h, const double* const* U, double* const* G, double* loss) {
@@ -2031,12 +2035,21 @@ jkcals_status jkcals_loss_history(jkcals_t h, int nsweeps, double* losses) {
   JK_TRY(check_handle(h));
   if (nsweeps < 0 || nsweeps > h->loss_cap || losses == nullptr)
     return fail(JKCALS_ERR_ARG, "nsweeps outside the loss history, or losses is NULL");
-  return copy_out(h, losses, h->loss_hist, sizeof(double) * nsweeps * h->K);
+  JK_TRY(copy_out(h, losses, h->loss_hist, sizeof(double) * nsweeps * h->K));
+  return is_host_pointer(losses) ? check_device_error(h, true) : JKCALS_OK;
 }
 
 jkcals_status jkcals_sync(jkcals_t h) {
   JK_TRY(check_handle(h));
-  JK_CUDA(h, cudaStreamSynchronize(h->stream));
+  return sync_stream(h);
+}
+
+jkcals_status jkcals_selftest_expired_wait(jkcals_t h, int code) {
+  JK_TRY(check_handle(h));
+  if (code <= 0) return fail(JKCALS_ERR_ARG, "code must be positive");
+  if (h->d_err == nullptr) return fail(JKCALS_ERR_STATE, "no kernel of this handle has a bounded wait");
+  h->ttm.ran = h->ttm.ran || h->ttm.use;
+  JK_CUDA(h, launch_store_error(h->d_err, code, h->stream));
   return JKCALS_OK;
 }
 

@@ -359,6 +359,9 @@ cudaError_t launch_reduce_partials_f64(const double* part, int S, int64_t count,
 cudaError_t launch_reduce_partials_f32(const float* part, int S, int64_t count, double* out,
                                        cudaStream_t s);
 
+// ---- self-test (jk_selftest.cu) ---------------------------------------------
+cudaError_t launch_store_error(int* err, int code, cudaStream_t s);
+
 // ---- tensor-times-matrix products on the tensor cores (jk_ttm.cu) -------------
 constexpr int kTtmTileC = 128;                   // tile of Y: columns c
 // Its rows r, by the contraction's length K: 64 with an exposed drain, or for short

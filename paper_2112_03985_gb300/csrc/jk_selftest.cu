@@ -41,12 +41,21 @@ __global__ void bounded_wait_selftest_kernel(int* err, int* out, uint64_t limit_
   __syncthreads();
 }
 
+// What a kernel does to its handle's error word when a wait expires.
+__global__ void store_error_kernel(int* err, int code) { atomicExch(err, code); }
+
 jkcals_status fail(jkcals_status s, const std::string& msg) {
   set_error(msg);
   return s;
 }
 
 }  // namespace
+
+cudaError_t launch_store_error(int* err, int code, cudaStream_t s) {
+  store_error_kernel<<<1, 1, 0, s>>>(err, code);
+  return cudaGetLastError();
+}
+
 }  // namespace jk
 
 extern "C" jkcals_status jkcals_selftest_bounded_wait(double limit_ms, int* code, double* left_after_ms) {
