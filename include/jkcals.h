@@ -174,7 +174,9 @@ void jkcals_destroy(jkcals_t h);
  * g's columns equal submodel g's own MTTKRP on its sliced tensor (Sec. 4.1);
  * for mode == sampled_mode rows D_g of block g are the full-tensor values that
  * Case I discards.
- *  M_out   I_mode x C row-major FP64, host or device.
+ *  M_out   I_mode x C row-major FP64, host or device.  The FP64 form into device
+ *          memory is only enqueued on the handle's stream; every other case
+ *          waits for it.
  * Errors: ARG (mode out of range, NULL), CUDA, STATE.
  */
 jkcals_status jkcals_mttkrp(jkcals_t h, int mode, double* M_out);

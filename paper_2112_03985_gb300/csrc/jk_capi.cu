@@ -1499,11 +1499,18 @@ jkcals_status jkcals_mttkrp(jkcals_t h, int mode, double* M_out) {
   if (M_out == nullptr) return fail(JKCALS_ERR_ARG, "M_out is NULL");
   JK_TRY(enqueue_mttkrp(h, mode, h->U, h->UT, h->UTlo, h->cmax));
   // memory of the handle's own device takes the sums directly, anything else a copy
-  if (writable_by_kernels(h, M_out)) {
+  const bool direct = writable_by_kernels(h, M_out);
+  if (direct) {
     JK_TRY(reduce_into(h, mode, M_out));
   } else {
     JK_TRY(reduce_into(h, mode, h->mbuf));
     JK_TRY(copy_out(h, M_out, h->mbuf, sizeof(double) * h->dims[mode] * (int64_t)h->C));
+  }
+  // FP64 into device memory is only enqueued (and can be captured); the next call that waits
+  // for the stream reads the error word
+  if (!h->tc && (direct || !is_host_pointer(M_out))) {
+    h->ttm.ran = h->ttm.ran || h->ttm.use;
+    return JKCALS_OK;
   }
   return check_device_error(h);
 }
