@@ -817,6 +817,7 @@ int contract_splits(int64_t HL, int Mm, int C) {
   const int64_t want = kContractSms * (HL * Mm * C * 8 > kLargeX ? 1280 : 512);
   int64_t S = (want + threads - 1) / threads;
   if (S > (Mm + 7) / 8) S = (Mm + 7) / 8;
+  if (S > 65535) S = 65535;   // grid.y
   if (S < 1) S = 1;
   const int chunk = (int)((Mm + S - 1) / S);
   return (Mm + chunk - 1) / chunk;
