@@ -152,6 +152,9 @@ void jkcals_default_options(jkcals_options* opt);
  * the stream is idle).  Memory freed by destroyed handles stays in that pool,
  * up to 2 GiB per device, for the next handle; more is returned to the device
  * at synchronisation points.  Without pool support the handle uses cudaMalloc.
+ * FP64 handles may take 16 bytes per tensor entry for each of up to two modes and
+ * up to 16 GiB for the shared products on top of what the CUDA-core kernel needs,
+ * but only where at least as much stays free (see JKCALS_FP64).
  *
  * Limits: N <= 8, R_g <= 32, prod(dims) < 2^40.
  * Errors: ARG on any invalid value, OOM, CUDA, UNSUPPORTED (limits).

@@ -1041,9 +1041,53 @@ size_t ttm_part_elems(const jkcals_ctx* h, int n) {
   return most * h->dims[n] * h->C;
 }
 
-// The products' buffers are an addition to what the CUDA-core kernel needs: if the
-// device has no room for them, or T holds a non-finite entry, the handle drops
-// them and runs on that kernel.
+// Elements of the products' workspace.
+struct TtmSizes {
+  size_t images = 0, at = 0, y = 0, z = 0, w = 0;   // bytes of T's images; At; doubles of Y, Z, each W
+};
+
+TtmSizes ttm_sizes(const jkcals_ctx* h) {
+  TtmSizes s;
+  for (int a : h->ttm.modes) {
+    if (a < 0) continue;
+    const int K = (int)h->dims[a], rows = ttm_tile_r(K);
+    s.images += ttm_image_bytes(K, h->J[a], rows) + (size_t)round_up(h->J[a], rows) * (ttm_ksteps(K) * 16 + 8);
+    s.at = std::max(s.at, ttm_image_bytes(K, h->C, kTtmTileC));
+    if (h->N > 2) s.y = std::max(s.y, (size_t)h->J[a] * h->C);
+    for (int q = 0; q < h->N && h->N >= 4; ++q) {
+      if (q == a) continue;
+      s.z = std::max(s.z, (size_t)(h->J[a] / h->dims[q]) * h->C);
+      for (int p = 0; p < h->N && h->N >= 5; ++p)
+        if (p != a && p != q) s.w = std::max(s.w, (size_t)(h->J[a] / h->dims[q] / h->dims[p]) * h->C);
+    }
+  }
+  return s;
+}
+
+// The products' buffers are an addition to what the CUDA-core kernel needs.  They come after
+// every buffer that a handle cannot do without, and are taken only where they leave at least
+// as much memory free as they take and what the handle's later calls allocate (gradients,
+// compaction, standard errors, longer loss histories): a device that is nearly full keeps
+// its room for those and for others.
+bool ttm_has_room(const jkcals_ctx* h) {
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  uint64_t reserved = 0, used = 0;   // the library's pool keeps freed memory for its handles
+  if (h->pool && cudaMemPoolGetAttribute(h->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+      cudaMemPoolGetAttribute(h->pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
+    free_bytes += (size_t)(reserved - used);
+  const TtmSizes s = ttm_sizes(h);
+  const size_t extra = s.images + s.at + sizeof(double) * (s.y + s.z + 2 * s.w);
+  size_t later = 64u << 20;
+  for (int n = 0; n < h->N; ++n) later += sizeof(double) * (5 * (size_t)h->dims[n] * h->C + 2 * (size_t)h->gram_total);
+  return free_bytes >= extra + std::max(extra, later);
+}
+
+// If they do not fit after all, or T holds a non-finite entry, the handle drops them and runs
+// on the CUDA-core kernel.
 void ttm_drop(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   void* all[] = {t.At, t.Y, t.Z, t.W[0], t.W[1], t.zpower, t.wpower[0], t.wpower[1]};
@@ -1062,10 +1106,14 @@ void ttm_drop(jkcals_ctx* h) {
   set_error("");
 }
 
-// The digit images of T (while the FP64 unfoldings exist).
+// The digit images of T.
 jkcals_status create_ttm_images(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   if (t.modes[0] < 0) return JKCALS_OK;
+  if (!ttm_has_room(h)) {
+    ttm_drop(h);
+    return JKCALS_OK;
+  }
   cudaStream_t st = h->stream;
   int* d_bad = nullptr;
   auto build = [&]() -> jkcals_status {
@@ -1104,36 +1152,39 @@ jkcals_status create_ttm_workspace(jkcals_ctx* h) {
   jkcals_ctx::Ttm& t = h->ttm;
   if (t.modes[0] < 0) return JKCALS_OK;
   auto build = [&]() -> jkcals_status {
-    size_t at = 0, y = 0, z = 0, w = 0;
+    const TtmSizes n = ttm_sizes(h);
     for (int a : t.modes) {
       if (a < 0) continue;
-      JK_TRY(dalloc_t(h, &t.cexp[a], (size_t)round_up(h->C, kTtmTileC)));
-      JK_TRY(dalloc_t(h, &t.ypower[a], (size_t)round_up(h->C, kTtmTileC)));
-      JK_TRY(dalloc_t(h, &t.cmag[a], (size_t)round_up(h->C, kTtmTileC) * ttm_ksteps((int)h->dims[a]) * 16));
-      at = std::max(at, ttm_image_bytes((int)h->dims[a], h->C, kTtmTileC));
-      if (h->N > 2) y = std::max(y, (size_t)h->J[a] * h->C);
-      for (int q = 0; q < h->N && h->N >= 4; ++q) {
-        if (q == a) continue;
-        z = std::max(z, (size_t)(h->J[a] / h->dims[q]) * h->C);
-        for (int p = 0; p < h->N && h->N >= 5; ++p)
-          if (p != a && p != q) w = std::max(w, (size_t)(h->J[a] / h->dims[q] / h->dims[p]) * h->C);
-      }
+      const size_t cols = (size_t)round_up(h->C, kTtmTileC);
+      JK_TRY(dalloc_t(h, &t.cexp[a], cols));
+      JK_TRY(dalloc_t(h, &t.ypower[a], cols));
+      JK_TRY(dalloc_t(h, &t.cmag[a], cols * ttm_ksteps((int)h->dims[a]) * 16));
     }
     void* img = nullptr;
-    JK_TRY(dalloc(h, &img, at));
+    JK_TRY(dalloc(h, &img, n.at));
     t.At = static_cast<unsigned char*>(img);
-    if (y > 0) JK_TRY(dalloc_t(h, &t.Y, y));
-    if (z > 0) {
-      JK_TRY(dalloc_t(h, &t.Z, z));
+    if (n.y > 0) JK_TRY(dalloc_t(h, &t.Y, n.y));
+    if (n.z > 0) {
+      JK_TRY(dalloc_t(h, &t.Z, n.z));
       JK_TRY(dalloc_t(h, &t.zpower, (size_t)h->C));
     }
-    for (int k = 0; k < 2 && w > 0; ++k) {
-      JK_TRY(dalloc_t(h, &t.W[k], w));
+    for (int k = 0; k < 2 && n.w > 0; ++k) {
+      JK_TRY(dalloc_t(h, &t.W[k], n.w));
       JK_TRY(dalloc_t(h, &t.wpower[k], (size_t)h->C));
     }
     JK_TRY(create_error_word(h));
     for (int a : t.modes)
       if (a >= 0) JK_CUDA(h, prepare_ttm((int)h->dims[a]));
+    // partial sums of the last contraction: about what fills the SMs
+    size_t part_bytes = 0;
+    for (int k = 0; k < h->N; ++k) part_bytes = std::max(part_bytes, sizeof(double) * ttm_part_elems(h, k));
+    if (part_bytes > h->part_bytes) {
+      void* part = nullptr;
+      JK_TRY(dalloc(h, &part, part_bytes));
+      dfree(h, h->part, true);
+      h->part = part;
+      h->part_bytes = part_bytes;
+    }
     return JKCALS_OK;
   };
   const jkcals_status s = build();
@@ -1280,17 +1331,11 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
 
   // plan + workspace
   make_plan(h);
-  if (!h->tc) {
-    choose_ttm_modes(h);
-    JK_TRY(create_ttm_images(h));
-  }
   size_t part_bytes = 0, chunks = 0;
   for (int n = 0; n < N; ++n) {
     const size_t eb = part_kind(h) == kPartF32 ? sizeof(float) : sizeof(double);
     const size_t pb = (size_t)mode_splits(h, n) * h->dims[n] * h->C * eb;
     part_bytes = std::max(part_bytes, pb);
-    if (h->ttm.use)   // partial sums of the last contraction: about what fills the SMs
-      part_bytes = std::max(part_bytes, 8 * ttm_part_elems(h, n));
     chunks = std::max(chunks, (size_t)h->plan[n].upd.RC * K);
   }
   // room for the two-phase update of any subset of the blocks (compaction):
@@ -1314,6 +1359,8 @@ jkcals_status create_impl(jkcals_ctx* h, const void* T, int T_dtype, const int32
   for (int n = 0; n < N; ++n)
     if (h->plan[n].upd.fused) fsmem = std::max(fsmem, h->plan[n].upd.fused_smem);
   if (fsmem > 0) JK_CUDA(h, prepare_update_fused(fsmem, h->Rmax, h->uniform_rank));
+  choose_ttm_modes(h);
+  JK_TRY(create_ttm_images(h));
   JK_TRY(create_ttm_workspace(h));
   h->kernels_per_sweep = count_sweep_kernels(h);
   JK_TRY(refresh_factor_state(h));
