@@ -218,6 +218,8 @@ jkcals_status jkcals_kernel_times(jkcals_t h, double* ms);
  * jkcals_sweep_info -- how one sweep is executed on the device.
  *  kernels_per_sweep  receives the number of kernel launches of one sweep
  *  splits             NULL or N ints (host): the split-K factor of each mode's MTTKRP
+ *                     (FP64: of the CUDA-core kernel, also where sweeps go through
+ *                     shared products)
  */
 jkcals_status jkcals_sweep_info(jkcals_t h, int* kernels_per_sweep, int* splits);
 

@@ -945,7 +945,10 @@ int64_t mode_kchunk(const jkcals_ctx* h, int n) { return h->tc ? h->tcplan[n].kc
 // (three timed runs after one warm-up each, CUDA events on the handle's
 // stream) and keep the fastest.  The partial-sum workspace grows as needed.
 jkcals_status autotune_splits(jkcals_ctx* h) {
-  if (h->ttm.use) return JKCALS_OK;   // the products have no split-K factor to tune
+  // on the products' route: for the calls that still run the CUDA-core kernel (single MTTKRPs,
+  // compacted runs, modes without images)
+  const bool products = h->ttm.use;
+  h->ttm.use = false;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   JK_CUDA(h, cudaEventCreate(&e0));
   JK_CUDA(h, cudaEventCreate(&e1));
@@ -991,6 +994,7 @@ jkcals_status autotune_splits(jkcals_ctx* h) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  h->ttm.use = products;
   if (st != JKCALS_OK) return st;
   return check_device_error(h);
 }
