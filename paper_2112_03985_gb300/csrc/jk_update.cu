@@ -29,6 +29,7 @@ namespace {
 constexpr int NTA = 128;  // threads of phase A = max rows per chunk
 constexpr int NTB = 512;  // the normalisation's divisions spread over them (40 blocks of
                           // 400 rows of rank 10: 32 us with 128 threads, 15 us with 512)
+constexpr int kLossThreads = 128;   // of the loss's H * G term: the grouping of its sum
 constexpr int GP = kMaxRank * kMaxRank;  // stride of one partial Gram
 
 __device__ __forceinline__ bool is_left_out(const BlockMeta& bm, int g, int64_t i) {
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(NTB) update_phase_b(UpdateArgs a) {
   const int go = a.bm.gram_off[g];
   __shared__ double G[kMaxRank][kMaxRank + 1];
   __shared__ double nrm[kMaxRank];
-  __shared__ double red[NTB];
+  __shared__ double red[kLossThreads];
 
   for (int p = tid; p < R * R; p += NTB) {
     const int r = p / R, c = p % R;
@@ -246,16 +247,18 @@ __global__ void __launch_bounds__(NTB) update_phase_b(UpdateArgs a) {
   if (!last) return;
 
   // e_g = ||T_{-g}||^2 + sum(H * G) - 2 sum(U * M)
-  double hg = 0.0;
-  for (int p = tid; p < R * R; p += NTB) {
-    double h = 1.0;
-    for (int k = 0; k < a.N; ++k)
-      if (k != a.n) h *= a.gram[k][go + p];
-    hg = fma(h, G[p / R][p % R], hg);
+  if (tid < kLossThreads) {
+    double hg = 0.0;
+    for (int p = tid; p < R * R; p += kLossThreads) {
+      double h = 1.0;
+      for (int k = 0; k < a.N; ++k)
+        if (k != a.n) h *= a.gram[k][go + p];
+      hg = fma(h, G[p / R][p % R], hg);
+    }
+    red[tid] = hg;
   }
-  red[tid] = hg;
   __syncthreads();
-  for (int w = NTB / 2; w > 0; w >>= 1) {
+  for (int w = kLossThreads / 2; w > 0; w >>= 1) {
     if (tid < w) red[tid] += red[tid + w];
     __syncthreads();
   }
