@@ -1055,7 +1055,7 @@ TtmSizes ttm_sizes(const jkcals_ctx* h) {
   for (int a : h->ttm.modes) {
     if (a < 0) continue;
     const int K = (int)h->dims[a], rows = ttm_tile_r(K);
-    s.images += ttm_image_bytes(K, h->J[a], rows) + (size_t)round_up(h->J[a], rows) * (ttm_ksteps(K) * 16 + 8);
+    s.images += ttm_image_bytes(K, h->J[a], rows) + (size_t)round_up(h->J[a], rows) * (ttm_ksteps(K) * 32 + 8);
     s.at = std::max(s.at, ttm_image_bytes(K, h->C, kTtmTileC));
     if (h->N > 2) s.y = std::max(s.y, (size_t)h->J[a] * h->C);
     for (int q = 0; q < h->N && h->N >= 4; ++q) {
@@ -1132,7 +1132,7 @@ jkcals_status create_ttm_images(jkcals_ctx* h) {
       JK_TRY(dalloc_t(h, &t.kexp[a], (size_t)h->dims[a]));
       JK_TRY(dalloc_t(h, &t.rexp[a], (size_t)round_up(h->J[a], rows)));
       JK_CUDA(h, launch_slice_exponents(h->Tn64[a], h->dims[a], h->J[a], t.kexp[a], d_bad, st));
-      JK_TRY(dalloc_t(h, &t.rmag[a], (size_t)round_up(h->J[a], rows) * ttm_ksteps((int)h->dims[a]) * 16));
+      JK_TRY(dalloc_t(h, &t.rmag[a], (size_t)round_up(h->J[a], rows) * ttm_ksteps((int)h->dims[a]) * 32));
       JK_CUDA(h, launch_slice_tensor(h->Tn64[a], (int)h->dims[a], h->J[a], t.kexp[a], t.Bt[a], t.rexp[a], t.rmag[a], st));
       JK_TRY(dalloc_t(h, &t.range[a], 1));
       JK_CUDA(h, launch_range(t.kexp[a], (int)h->dims[a], t.rexp[a], h->J[a], t.range[a], st));
@@ -1162,7 +1162,7 @@ jkcals_status create_ttm_workspace(jkcals_ctx* h) {
       const size_t cols = (size_t)round_up(h->C, kTtmTileC);
       JK_TRY(dalloc_t(h, &t.cexp[a], cols));
       JK_TRY(dalloc_t(h, &t.ypower[a], cols));
-      JK_TRY(dalloc_t(h, &t.cmag[a], cols * ttm_ksteps((int)h->dims[a]) * 16));
+      JK_TRY(dalloc_t(h, &t.cmag[a], cols * ttm_ksteps((int)h->dims[a]) * 32));
     }
     void* img = nullptr;
     JK_TRY(dalloc(h, &img, n.at));

@@ -378,7 +378,7 @@ struct TtmArgs {
   const unsigned char* Bt;   // digit images of T_(a): tiles_r x nk steps
   const int2* cexp;          // per column c (padded to tiles): exponent, entries near the largest
   const int2* rexp;          // per row r of Y (padded to tiles)
-  const unsigned char* cmag; // magnitudes of the scaled column, 16 nk bytes per column c
+  const unsigned char* cmag; // magnitudes of the scaled column, 32 nk bytes per column c
   const unsigned char* rmag; // the same per row r
   int nk, K, C, tiles_c;
   int64_t J, tiles_r;

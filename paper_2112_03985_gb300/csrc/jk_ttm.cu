@@ -27,15 +27,17 @@
 // magnitudes of an entry's K terms.  Dropped are the operands' rounding (at most 2^-58 per
 // term) and the products beyond level 7 (seven of at most 2^-58 per term): at most
 // K 2^-55 2^(E+F), typically sqrt(7 K) 2^-60 2^(E+F).  That is measured by the vectors'
-// maxima, not by the entry's own terms, so it is accepted only where S >= 2^-5 2^(E+F):
-// the error is then at most 8 K 2^-53 S and typically 0.7 sqrt(K) 2^-53 S or less, that of
-// an FP64 chain of about 10 K terms (K <= 448; the CUDA-core kernel's chains are 800 to
-// 1200 terms at 300x100x50, K 100 and 300, and 12000 at 400x400x400).  The
+// maxima, not by the entry's own terms, so it is accepted only where S >= 2^-6 2^(E+F):
+// the error is then at most 16 K 2^-53 S and typically 1.3 sqrt(K) 2^-53 S or less, and an
+// MTTKRP's sum over many entries averages it (measured below).  The
 // drain finds S from below by the entry's own value, or else by the products of the
-// magnitudes' leading eight bits (stored with the digits); an entry that neither certifies
-// is computed as a plain FP64 dot product (plain_entries).  Of random data none is, of noisy
-// fluorescence-like data 0 to 1 entry in 100; data whose vectors do not overlap (sparse
-// tensors, separated bumps without noise) take more of them and more time.
+// magnitudes' leading 16 bits (stored with the digits); an entry that neither certifies is
+// computed as a plain FP64 dot product (plain_entries).  Of dense data of one scale none is,
+// of noisy fluorescence-like data 0 to 3 entries in 100 (300x100x50, 1500 columns: 0.45 ms a
+// sweep from the start, 0.57 ms at convergence; with 8-bit magnitudes and twice the
+// threshold 1.2 ms).  Data whose vectors hardly overlap take more: 1.3 ms with 1% of the
+// tensor non-zero, 7 ms for separated bumps without noise, against 16 ms of the CUDA-core
+// kernel; 40x33x61: 0.2 against 0.35 ms.
 //
 // Along the contraction the two operands are equilibrated by powers of two
 // (exact): T_(a)(i, :) 2^(-F_i) against Ubar^(a)(i, :) 2^(F_i), F_i the mean exponent of
@@ -47,9 +49,10 @@
 // Measured (GB300), against the CUDA-core MTTKRP of every mode: an FP64 sweep of
 // 300x100x50 with 1500 columns 16.0 -> 0.46 ms, of 400x400x400 with 400 columns
 // 192 -> 3.4 ms; loss and gradient of 100x60x60x40 with 800 columns 166 -> 4.3 ms.
-// Largest MTTKRP error against quadruple precision, relative to the largest
-// entry (300x100x50, modes 0-2): 3.2e-16, 4.9e-16, 5.8e-16, against 6.9e-16,
-// 1.8e-15, 1.6e-15 on the CUDA cores, whose chains of additions are longer.
+// Largest error of an MTTKRP entry against quadruple precision, in units of 2^-53 of the sum
+// of its own terms' magnitudes (41x61x35 to 300x100x50 and 4-way, uniform, normal and bumps,
+// 0 to 5 sweeps): 2 to 5 where the CUDA-core kernel, with longer chains, has 4 to 17; of the
+// largest entry 1.3e-16 to 4.1e-16 against 1.5e-16 to 1.3e-15.
 //
 // A column of Ubar^(a) with a non-finite entry is taken out of the digits and
 // computed by plain FP64 dot products in the drain, so Inf and NaN propagate as
@@ -95,10 +98,10 @@ constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + kListBytes + (2 * kSt
 // throughout: an FP64 rint per digit would take 18 us of the FP64 pipe for
 // 300 x 1500 entries.  counter: a sweep's first slicing also advances the sweep
 // counter (null otherwise).  mag: every scaled
-// magnitude in units of 2^(expo - 8), rounded down (16 nk bytes per column); expo[m].y: how
-// many are at least kFlat of them.
+// magnitude in units of 2^(expo - 16), rounded down (32 nk bytes per column: for 16 rows, the
+// high bytes, then the low ones); expo[m].y: how many have a high byte of at least kFlat.
 constexpr int kSliceCols = 8;   // columns per block
-constexpr uint32_t kFlat = 16;  // 2^-4 of a column's power of two, in units of 2^-8
+constexpr uint32_t kFlat = 16;  // 2^-4 of a column's power of two, in a high byte's units of 2^-8
 
 // Half of every digit's field below d_0: 256 of the last one's nine bits, 64 of the
 // others' seven.
@@ -169,19 +172,22 @@ __global__ void __launch_bounds__(256) slice_f64_kernel(const double* __restrict
     for (int j = 0; j < 2; ++j) {
       const int ch = g + j * kGroups;
       if (ch >= 2 * nk) break;
-      unsigned long long mags = 0;
+      unsigned long long high = 0, low = 0;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(x[j][e]);
         const int ef = (int)((b >> 52) & 2047);
         if (ef > 0 && !col_bad) {   // a normal entry: 1.m 2^(ef - 1023), scaled below 2^E
           const int sh = E - 1 - (ef + sgn * __ldg(kexp + 8 * ch + e) - 1023);
-          const uint32_t q = sh < 8 ? (0x80u | (uint32_t)((b >> 45) & 0x7f)) >> sh : 0u;
-          mags |= (unsigned long long)q << (8 * e);
-          nflat += q >= kFlat ? 1 : 0;
+          const uint32_t q = sh < 16 ? (0x8000u | (uint32_t)((b >> 37) & 0x7fff)) >> sh : 0u;
+          high |= (unsigned long long)(q >> 8) << (8 * e);
+          low |= (unsigned long long)(q & 255u) << (8 * e);
+          nflat += (q >> 8) >= kFlat ? 1 : 0;
         }
       }
-      *reinterpret_cast<unsigned long long*>(mag + (m * nk * 16 + ch * 8)) = mags;
+      unsigned long long* mg = reinterpret_cast<unsigned long long*>(mag + (m * nk + (ch >> 1)) * 32 + (ch & 1) * 8);
+      mg[0] = high;
+      mg[2] = low;
       uint32_t w[P][4];
 #pragma unroll
       for (int pr = 0; pr < 4; ++pr) {
@@ -373,42 +379,55 @@ __device__ __forceinline__ double round_levels(long long hi, uint32_t lo, int ex
 }
 
 // What certifies an entry of the product (the bound is derived at the top of this file): the
-// sum of its terms' magnitudes is at least 2^-5 of the product of the vectors' maxima,
+// sum of its terms' magnitudes is at least 2^-6 of the product of the vectors' maxima,
 //  - because so many of both vectors' entries are at least 2^-4 of their maxima that at
-//    least kFlatTerms rows hold two of them (8 x 2^-8; decided for a warp's 32 columns and
+//    least kFlatTerms rows hold two of them (4 x 2^-8; decided for a warp's 32 columns and
 //    rows at once: dense data of one scale, at no cost per entry),
 //  - by the entry's own value, or
-//  - by the magnitudes in units of 2^-8.
-constexpr int kFlatTerms = 8;
-constexpr long long kCertain = 1ll << 30;      // 2^-5 in units of level 3 (2^-35)
-constexpr uint32_t kCertainMags = 1u << 11;    // 2^-5 in units of 2^-16
+//  - by the magnitudes' leading 16 bits.
+constexpr int kFlatTerms = 4;
+constexpr long long kCertain = 1ll << 29;      // 2^-6 in units of level 3 (2^-35)
+constexpr uint32_t kCertainMags = 1u << 18;    // 2^-6 in units of 2^-24
 
-// The entries of this warp's tile rows that their own value does not certify (bits of
-// pending: rows r0 .. r0 + NC - 1 of column c0 + lane).  Those that the magnitudes do not
-// certify either, and every entry of a column with a non-finite one (forced), become plain
-// FP64 dot products.  They are gathered in list and taken 32 at a time, a lane each, or fewer
-// by several lanes each: bound by the FP64 pipe (K / 2 clocks of an SM per entry), as
-// submodels that share a factor fail together, rows of whole tiles at a time.
-template <int NC>
-__device__ __noinline__ void plain_entries(const TtmArgs& a, int64_t r0, int c0, uint32_t pending, bool forced,
-                                           unsigned short* list, int lane) {
+// Of the entries of this warp's tile rows that their own value does not certify (bits of open:
+// rows r0 .. r0 + 7 of column c0 + lane), those that the magnitudes do not certify either.
+__device__ __noinline__ uint32_t uncertified(const TtmArgs& a, int64_t r0, int c0, uint32_t open, int lane) {
   // the magnitudes of sixteen rows k of the contraction at a time, against all pending rows
-  // together: their loads are in flight together, and sixteen are mostly enough
-  uint32_t open = forced ? 0u : pending;
-  const uint4* mr = reinterpret_cast<const uint4*>(a.rmag) + r0 * a.nk;
-  const uint4* mc = reinterpret_cast<const uint4*>(a.cmag) + (int64_t)(c0 + lane) * a.nk;   // padded, as the rows
-  uint32_t sum[NC] = {};
+  // together (their loads are in flight together): the products of the high bytes, which are
+  // mostly enough, then those of high and low ones
+  const uint4* mr = reinterpret_cast<const uint4*>(a.rmag) + r0 * a.nk * 2;
+  const uint4* mc = reinterpret_cast<const uint4*>(a.cmag) + (int64_t)(c0 + lane) * a.nk * 2;   // padded, as the rows
+  uint32_t sum[8] = {};
+  auto dot = [](const uint4& x, const uint4& y, uint32_t s) {
+    return __dp4a(x.x, y.x, __dp4a(x.y, y.y, __dp4a(x.z, y.z, __dp4a(x.w, y.w, s))));
+  };
   for (int w = 0; w < a.nk && __any_sync(0xffffffffu, open != 0); ++w) {
-    const uint4 y = __ldg(mc + w);
+    const uint4 y = __ldg(mc + 2 * w);
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-      const uint4 x = __ldg(mr + (int64_t)k * a.nk + w);
-      sum[k] = __dp4a(x.x, y.x, __dp4a(x.y, y.y, __dp4a(x.z, y.z, __dp4a(x.w, y.w, sum[k]))));
+    for (int k = 0; k < 8; ++k) {
+      sum[k] += dot(__ldg(mr + ((int64_t)k * a.nk + w) * 2), y, 0u) << 8;
       if (sum[k] >= kCertainMags) open &= ~(1u << k);
     }
   }
-  if (!forced) pending = open;
-  if (!__any_sync(0xffffffffu, pending != 0)) return;
+  for (int w = 0; w < a.nk && __any_sync(0xffffffffu, open != 0); ++w) {
+    const uint4 yh = __ldg(mc + 2 * w), yl = __ldg(mc + 2 * w + 1);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const uint4* xp = mr + ((int64_t)k * a.nk + w) * 2;
+      sum[k] = dot(__ldg(xp), yl, dot(__ldg(xp + 1), yh, sum[k]));
+      if (sum[k] >= kCertainMags) open &= ~(1u << k);
+    }
+  }
+  return open;
+}
+
+// Plain FP64 dot products for the entries in pending (bits as above): those that nothing
+// certifies, and every entry of a column with a non-finite one.  They are gathered in list and
+// taken 32 at a time, a lane each, or fewer by several lanes each: bound by the FP64 pipe
+// (K / 2 clocks of an SM per entry), as submodels that share a factor fail together, rows of
+// whole tiles at a time.
+__device__ __noinline__ void plain_entries(const TtmArgs& a, int64_t r0, int c0, uint32_t pending,
+                                           unsigned short* list, int lane) {
   int at = __popc(pending);
   for (int o = 1; o < 32; o <<= 1) {
     const int below = __shfl_up_sync(0xffffffffu, at, o);
@@ -623,7 +642,13 @@ __global__ void __launch_bounds__(kThreads, 1) ttm_kernel(const __grid_constant_
       }
       const int rflat = __reduce_min_sync(0xffffffffu, re.y);
       if (ce.y + rflat >= a.K + kFlatTerms) pending = 0;
-      if (__any_sync(0xffffffffu, pending != 0)) plain_entries<NC>(a, r0, c - lane, pending, forced, lists + warp * (32 * NC), lane);
+      if (__any_sync(0xffffffffu, pending != 0)) {
+        // a column with a non-finite entry (its magnitudes are zero) needs all of its sums
+        uint32_t left = 0;
+#pragma unroll
+        for (int h = 0; h < NC; h += 8) left |= uncertified(a, r0 + h, c - lane, (pending >> h) & 255u, lane) << h;
+        if (__any_sync(0xffffffffu, left != 0)) plain_entries(a, r0, c - lane, left, lists + warp * (32 * 16), lane);
+      }
     }
   }
 
