@@ -268,47 +268,6 @@ __device__ __forceinline__ double df_to_double(float hi, float lo) {
   return f32_to_f64_exact(s) + f32_to_f64_exact(r);
 }
 
-// FP32 pair of a double u: hi = fl32(u), lo = fl32(u - hi), both rounded to
-// nearest even, as the conversions give them, but formed from u's bit pattern
-// with integer operations: the FP64 pipe (which also runs FP64 conversions) is
-// narrow on this part and the update is bound by it.  hi keeps the top 24
-// significant bits of u's 53 (round half to even on the low 29); u - hi is
-// that remainder, at most 29 bits, converted exactly to FP32 and scaled by the
-// power of two of its unit.  Magnitudes outside [2^-70, 2^120) (and 0, Inf,
-// NaN) take the conversions.
-__device__ __forceinline__ void split_f32_pair(double u, float& hi, float& lo) {
-  const long long bits = __double_as_longlong(u);
-  const uint32_t hw = (uint32_t)((unsigned long long)bits >> 32), lw = (uint32_t)bits;
-  const int e = (int)((hw >> 20) & 0x7ffu) - 1023;   // unbiased exponent
-  if (e < -70 || e >= 120) {
-    hi = __double2float_rn(u);
-    lo = __double2float_rn(u - (double)hi);
-    return;
-  }
-  const uint32_t sign = hw & 0x80000000u;
-  uint32_t keep = ((hw & 0xfffffu) << 3) | (lw >> 29);   // the 23 stored bits of hi
-  const uint32_t rem = lw & 0x1fffffffu;                  // the 29 bits below them
-  const bool up = rem > 0x10000000u || (rem == 0x10000000u && (keep & 1u));
-  uint32_t fexp = (uint32_t)(e + 127);
-  uint32_t r;   // |u - hi| in units of 2^(e - 52)
-  if (up) {
-    r = 0x20000000u - rem;
-    if (++keep == 0x800000u) {
-      keep = 0;
-      ++fexp;
-    }
-  } else {
-    r = rem;
-  }
-  hi = __uint_as_float(sign | (fexp << 23) | keep);
-  if (r == 0) {
-    lo = 0.f;
-    return;
-  }
-  const float mag = __uint2float_rn(r) * __uint_as_float((uint32_t)(e - 52 + 127) << 23);   // exact
-  lo = (up != (sign != 0u)) ? -mag : mag;   // u - hi has u's sign when hi was rounded down
-}
-
 // ---- error plumbing (jk_capi.cu) --------------------------------------------
 void set_error(const std::string& msg);
 
