@@ -29,15 +29,14 @@
 // K 2^-55 2^(E+F), typically sqrt(7 K) 2^-60 2^(E+F).  That is measured by the vectors'
 // maxima, not by the entry's own terms, so it is accepted only where S >= 2^-6 2^(E+F):
 // the error is then at most 16 K 2^-53 S and typically 1.3 sqrt(K) 2^-53 S or less, and an
-// MTTKRP's sum over many entries averages it (measured below).  The
-// drain finds S from below by the entry's own value, or else by the products of the
-// magnitudes' leading 16 bits (stored with the digits); an entry that neither certifies is
-// computed as a plain FP64 dot product (plain_entries).  Of dense data of one scale none is,
-// of noisy fluorescence-like data 0 to 3 entries in 100 (300x100x50, 1500 columns: 0.45 ms a
-// sweep from the start, 0.57 ms at convergence; with 8-bit magnitudes and twice the
-// threshold 1.2 ms).  Data whose vectors hardly overlap take more: 1.3 ms with 1% of the
-// tensor non-zero, 7 ms for separated bumps without noise, against 16 ms of the CUDA-core
-// kernel; 40x33x61: 0.2 against 0.35 ms.
+// MTTKRP's sum over many entries averages it (measured below).  The drain finds S from below
+// by the entry's own value, or else by the products of the magnitudes' leading 16 bits
+// (stored with the digits); an entry that neither certifies is computed as a plain FP64 dot
+// product (plain_entries).  Of dense data of one scale none is, of noisy fluorescence-like
+// data 0 to 3 entries in 100 (300x100x50, 1500 columns: 0.45 ms a sweep from the start,
+// 0.57 ms at convergence; with 8-bit magnitudes and twice the threshold 1.2 ms).  Data whose
+// vectors hardly overlap take more: 1.3 ms with 1% of the tensor non-zero, 7 ms for separated
+// bumps without noise, against 16 ms of the CUDA-core kernel; 40x33x61: 0.2 against 0.35 ms.
 //
 // Along the contraction the two operands are equilibrated by powers of two
 // (exact): T_(a)(i, :) 2^(-F_i) against Ubar^(a)(i, :) 2^(F_i), F_i the mean exponent of
@@ -47,7 +46,7 @@
 // submodel leaves it out.
 //
 // Measured (GB300), against the CUDA-core MTTKRP of every mode: an FP64 sweep of
-// 300x100x50 with 1500 columns 16.0 -> 0.46 ms, of 400x400x400 with 400 columns
+// 300x100x50 with 1500 columns 16.0 -> 0.45 ms, of 400x400x400 with 400 columns
 // 192 -> 3.4 ms; loss and gradient of 100x60x60x40 with 800 columns 166 -> 4.3 ms.
 // Largest error of an MTTKRP entry against quadruple precision, in units of 2^-53 of the sum
 // of its own terms' magnitudes (41x61x35 to 300x100x50 and 4-way, uniform, normal and bumps,
@@ -97,9 +96,9 @@ constexpr size_t kSmem = 1024 + (size_t)kStages * kStage + kListBytes + (2 * kSt
 // digits.  sgn = +1 / -1 scales row k by 2^(+-kexp[k]).  Integer arithmetic
 // throughout: an FP64 rint per digit would take 18 us of the FP64 pipe for
 // 300 x 1500 entries.  counter: a sweep's first slicing also advances the sweep
-// counter (null otherwise).  mag: every scaled
-// magnitude in units of 2^(expo - 16), rounded down (32 nk bytes per column: for 16 rows, the
-// high bytes, then the low ones); expo[m].y: how many have a high byte of at least kFlat.
+// counter (null otherwise).  mag: every scaled magnitude in units of 2^(expo - 16),
+// rounded down (32 nk bytes per column: for 16 rows, the high bytes, then the low ones);
+// expo[m].y: how many have a high byte of at least kFlat.
 constexpr int kSliceCols = 8;   // columns per block
 constexpr uint32_t kFlat = 16;  // 2^-4 of a column's power of two, in a high byte's units of 2^-8
 
@@ -476,8 +475,7 @@ __device__ __noinline__ void plain_entries(const TtmArgs& a, int64_t r0, int c0,
 // Bound: shared-memory bandwidth.  Per 16 rows of the contraction and 128 x 64 tile the
 // MMAs take 1152 cycles of the tensor pipe but read 120 KB of operands while TMA writes
 // 48 KB: 168 KB at 128 bytes a clock are 1344 cycles, and about 1380 were measured
-// (400x400x400, 400 columns: 1310 us).  Two CTAs sharing U's stage by TMA multicast
-// changed nothing: the writes to shared memory stay.
+// (400x400x400, 400 columns: 1310 us).
 // BN = 64 leaves room for one accumulator set, so the next tile's first MMA waits until
 // every level is read (about 5000 cycles): the drain takes the levels into 64-bit integers
 // first and rounds and stores them under the next tile's MMAs.  BN = 32 has two sets and
@@ -676,9 +674,9 @@ __device__ __forceinline__ double times_power(double v, int e) {
 // outputs (h, l) of V adjacent columns: one load of U serves RB of X, and a load of two
 // columns is 16 bytes.  A column that X holds times a power of two (see column_power) is
 // contracted with its factor's column scaled to at most 1; the powers go into the result, or,
-// if that is contracted again, to out_power.  Bound: X read once, or the FP64 pipe's
-// two multiply-adds per clock
-// and SM (400x400x400, 400 columns: 130 us, 512 MB at 3.9 TB/s and 490 G multiply-adds/s).
+// if that is contracted again, to out_power.  Bound: X read once, or the FP64 pipe's two
+// multiply-adds per clock and SM (400x400x400, 400 columns: 130 us, 512 MB at 3.9 TB/s and
+// 490 G multiply-adds/s).
 template <int RB, int V>
 __global__ void __launch_bounds__(256) contract_kernel(const double* __restrict__ X, int64_t H, int Mm, int64_t L,
                                                        int C, const double* __restrict__ U, int mchunk,
