@@ -50,8 +50,8 @@
 // 192 -> 3.4 ms; loss and gradient of 100x60x60x40 with 800 columns 166 -> 4.3 ms.
 // Largest error of an MTTKRP entry against quadruple precision, in units of 2^-53 of the sum
 // of its own terms' magnitudes (41x61x35 to 300x100x50 and 4-way, uniform, normal and bumps,
-// 0 to 5 sweeps): 2 to 5 where the CUDA-core kernel, with longer chains, has 4 to 17; of the
-// largest entry 1.3e-16 to 4.1e-16 against 1.5e-16 to 1.3e-15.
+// 0 to 40 sweeps): 0.1 to 5 where the CUDA-core kernel, with longer chains, has 0.2 to 33; of
+// the largest entry 1.3e-16 to 7.1e-16 against 1.5e-16 to 1.9e-15.
 //
 // A column of Ubar^(a) with a non-finite entry is taken out of the digits and
 // computed by plain FP64 dot products in the drain, so Inf and NaN propagate as
